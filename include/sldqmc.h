@@ -59,7 +59,10 @@ extern "C" {
  * stabilisation (QR), the final determinant, the Green's function and every
  * Monte Carlo decision are FP64 in all modes. */
 typedef enum {
-    SLDQMC_FP64 = 0,   /* FP64 FMA products */
+    SLDQMC_FP64 = 0,   /* FP64-accurate products: FP64 FMA below 128 sites; from 128 sites on
+                          error-free digit splitting on the BF16 tensor cores (errors at the
+                          level of FP64 rounding), or FP64 FMA where its workspace would take
+                          more than a third of the free device memory */
     SLDQMC_3XTF32 = 1, /* split-TF32 tensor-core products: the running product in two TF32
                           parts, exp(-dtau K) in three (five MMAs per K-step), FP32
                           accumulation spread over eight tensor-memory accumulators */
@@ -321,10 +324,10 @@ int sldqmc_weight_noalloc(const sldqmc_params *p, void *stream, const int8_t *d_
  * number Cholesky-QR can take: kappa(X)^2 eps_W < 1).  d_X holds B row-major
  * N x N FP64 matrices (item stride N*N), d_W receives B row-major N x N FP64
  * matrices of which every element on or above the diagonal is written (the
- * rest is unspecified).  Computed exactly as the context's stabilisation does:
- * in the mixed-precision modes with N >= 128 on the BF16 tensor cores by
- * error-free digit splitting (FP64 accuracy: error below ~2^-52 of
- * sqrt(W_ii W_jj)), otherwise by the FP64 GEMM.  1 <= B <= max_batch.
+ * rest is unspecified).  In the mixed-precision modes with N >= 128 computed as
+ * the context's stabilisation does, on the BF16 tensor cores by error-free
+ * digit splitting (FP64 accuracy: error below ~2^-52 of sqrt(W_ii W_jj));
+ * otherwise by the FP64 GEMM.  1 <= B <= max_batch.
  * Stream-ordered on the context's stream; caller-owned device buffers. */
 int sldqmc_gram_batch_dev(sldqmc_ctx *ctx, const double *d_X, int B, double *d_W);
 
@@ -336,13 +339,13 @@ int sldqmc_gram_batch_dev(sldqmc_ctx *ctx, const double *d_X, int B, double *d_W
 int sldqmc_wait_selftest(sldqmc_ctx *ctx, int max_polls);
 
 /* Kernel classes for the timing hooks below. */
-#define SLDQMC_KC_GEMM_F64 0   /* FP64 GEMM (slice products in FP64 mode, Gram, trailing updates) */
+#define SLDQMC_KC_GEMM_F64 0   /* FP64 GEMM (products below 128 sites, Gram entry point in FP64 mode) */
 #define SLDQMC_KC_GEMM_TC 1    /* tensor-core slice products (3xTF32 / BF16) */
 #define SLDQMC_KC_PANEL_F64 2  /* FP64 panel kernels (32x32 Cholesky blocks and inverses, LU panels, triangular solves, pivot sort) */
 #define SLDQMC_KC_EFF 3        /* effective-model sweeps */
 #define SLDQMC_KC_LOCAL 4      /* local-update flips */
 #define SLDQMC_KC_OTHER 5      /* everything else */
-#define SLDQMC_KC_GEMM_OZ 6    /* FP64-accurate digit-split products on the BF16 tensor cores (mixed modes): Gram matrices, Cholesky-QR updates and panels, R2 R1, V update, LU updates */
+#define SLDQMC_KC_GEMM_OZ 6    /* FP64-accurate digit-split products on the BF16 tensor cores: Gram matrices, Cholesky-QR updates and panels, R2 R1, V update, LU and back-substitution updates, delayed corrections; FP64-mode slice products, wraps of the Green's functions */
 #define SLDQMC_KC_SEP 7        /* slice products with the separable exp(-dtau K) (sldqmc_set_kinetic_form) */
 #define SLDQMC_KC_COUNT 8
 

@@ -9,7 +9,9 @@
 // (N/64, M/64, batch) with several CTAs resident per SM, and the next K-slab
 // is prefetched into registers while the current one is consumed.
 //
-// The same kernel serves the slice products of the FP64 mode (with the
+// The tensor cores' digit-split products (oz_gram.cu) replace it from 128
+// sites on; below, and where their workspace does not fit, the same kernel
+// serves the slice products of the FP64 mode (with the
 // field scalings of B_tau = exp(-dtau K) diag(exp(eta dtau xi s)) fused in:
 // the first slice of a block scales the K index, later slices scale the
 // output columns), the Gram matrices and trailing updates of the

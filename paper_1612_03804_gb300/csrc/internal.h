@@ -59,14 +59,16 @@ GemmF64 gemm_desc(int M, int N, int K, const double *A, long long lda, long long
                   const double *B, long long ldb, long long sB, double *C, long long ldc,
                   long long sC, int batch);
 
-// Mixed-precision modes, N >= 128: W = X X^T to FP64 accuracy on the
+// N >= 128: W = X X^T to FP64 accuracy on the
 // BF16 tensor cores (Ozaki splitting; X row stride N, batch stride sX; W row
 // stride ldw, batch stride sW; tiles on or above the diagonal written).
-// oz_prepare leaves c->oz_ws null outside that range.  Defined in oz_gram.cu.
+// oz_prepare leaves c->oz_ws null outside that range, and in the FP64 mode
+// when the planes would take more than a third of the free memory (the FP64
+// pipe then does these products).  Defined in oz_gram.cu.
 int oz_prepare(sldqmc_ctx *c);
 void oz_release(sldqmc_ctx *c);
 void oz_gram(sldqmc_ctx *c, const double *X, long long sX, double *W, long long sW, int ldw, int B);
-// Left-looking Cholesky-QR on the tensor cores (mixed modes, same N range):
+// Left-looking Cholesky-QR on the tensor cores (same N range):
 // oz_chol_begin fixes the digit exponents of R's columns from diag(W);
 // oz_chol_update subtracts the contributions of the finished rows
 // kstart..k0-1 from rows k0..k0+kb of W and of Y = Q^T (k0 - kstart a
@@ -77,10 +79,23 @@ void oz_gram(sldqmc_ctx *c, const double *X, long long sX, double *W, long long 
 void oz_chol_begin(sldqmc_ctx *c, const double *W, long long sW, int B);
 void oz_chol_update(sldqmc_ctx *c, int k0, int kb, int kstart, double *W, long long sW, double *Y, int B);
 void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW, double *Y, double *R, int B);
-// Trailing update of the finalisation's blocked LU without a right-hand side
-// (A row stride lda, item stride sA; panel k0..k0+kb with kb = 32), FP64-
-// accurate on the tensor cores.
-void oz_lu_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B);
+// Rank-32 updates (row stride lda, item stride sA; panel k0..k0+kb), FP64-
+// accurate on the tensor cores: the finalisation's LU (rhs: also the
+// right-hand side in columns N..2N-1), its back substitution, and the pending
+// pairs G_f -= U_f V_f of the delayed local update (U: N x 32, V: 32 x N).
+void oz_lu_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B, int rhs);
+void oz_back_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B);
+void oz_delayed_update(sldqmc_ctx *c, double *const *G, const double *const *U, const double *const *V, int B);
+// Products with exp(-+dtau K) on the tensor cores, FP64-accurate.  oz_have_e
+// builds the digit planes of both propagators on first use and says whether
+// they are there; oz_slice_product: Xt = X diag(d) E (d from the field slice
+// sk); oz_similarity: dst_f = P src_f P^-1 of both flavours, P = E or, with
+// inv, E^-1, rows and columns then scaled by d_i / d_j of the field slice s
+// (null: no scaling), T_f an N x N scratch per item.
+bool oz_have_e(sldqmc_ctx *c);
+void oz_slice_product(sldqmc_ctx *c, const double *X, const int8_t *sk, double cu, double cd, double *Xt, int B);
+void oz_similarity(sldqmc_ctx *c, const double *const *src, double *const *T, double *const *dst, int inv,
+                   const int8_t *s, const double (*ex)[2], int B);
 // R = R2 R1 of the two passes on the tensor cores (tiles on or above the
 // diagonal written); oz_keep_bounds saves the first pass's column bounds of R
 // before the second pass replaces them.

@@ -1,23 +1,37 @@
 // oz_gram.cu -- FP64-accurate products on the BF16 tensor cores (Ozaki's
-// error-free splitting) for the stabilisation and the determinant of the
-// mixed-precision modes: Gram matrices, the left-looking Cholesky-QR updates
-// and panel products (with the inverse of each 32 x 32 diagonal factor,
-// formed here in FP64), R = R2 R1, the V update and the trailing updates of
-// the determinant's LU.  The Gram matrix shows the scheme:
+// error-free splitting) for N >= 128: the stabilisation and the determinant in
+// every mode (Gram matrices, the left-looking Cholesky-QR updates and panel
+// products with the inverse of each 32 x 32 diagonal factor, formed here in
+// FP64, R = R2 R1, the V update, the trailing updates of the LU and the back
+// substitution of G), the slice products of the FP64 mode, and the wraps and
+// delayed corrections of the local sweep's Green's functions.
+//
+// Why not the FP64 pipe in the FP64 mode: it runs at 1.05-1.10 TFLOP/s however
+// a product is tiled (64 lanes-clocks per warp instruction), these products
+// at 11-33 TFLOP/s (N = 400, 4 items: 47 us against 560; N = 576, 8 items and
+// two flavours: 185 us against 5600).  The largest error of a product against
+// extended precision is about a tenth of the FP64 GEMM's (Q D E, G E^-1,
+// E G E^-1 at N = 144 .. 576: 0.7e-16 .. 1.2e-16 against 1.0e-15 .. 1.7e-15 of the
+// largest element).  Below N = 128 (one tile row) the FP64 pipe keeps them.
+//
+// The Gram matrix shows the scheme:
 //
 // W = X X^T for the rows x_i of X (N x N per batch item).  Each row is
 // scaled by a power of two, 2^-E_i with |x_ik| < 2^E_i, and written as eight
 // balanced base-2^7 digits,
-//   x_ik 2^-E_i = sum_{p=1..8} a_p,ik 2^-7p   (|a_1| <= 128, |a_p| <= 64, p > 1),
-// exact up to the rounding of x_ik 2^-E_i to a multiple of 2^-56.  Then
-//   W_ij 2^-(E_i+E_j) = sum_{p,q} 2^-7(p+q) sum_k a_p,ik a_q,jk,
+//   x_ik 2^-E_i = sum_{p=1..8} a_p,ik 2^-(7p+1)   (|a_1| <= 256, |a_p| <= 64, p > 1),
+// exact up to the rounding of x_ik 2^-E_i to a multiple of 2^-57.  Then
+//   W_ij 2^-(E_i+E_j) = sum_{p,q} 2^-(7(p+q)+2) sum_k a_p,ik a_q,jk,
 // of which the 36 products with p + q <= 9 are kept: each dropped term is
-// below 2^-56 of the row maxima, the same order as FP64's own rounding of the
-// sum.  The digit planes are BF16 integers; the products of one group
+// below 2^-58 of the row maxima.  (The leading digit may use all of BF16's
+// integers up to 256.  With |a_1| <= 128 the dropped terms are four times as
+// large, 5e-17 rms of the row maxima's product at K = 256, which at the block
+// condition limit, 16 x 16, n_wrap = 16, dtau = 0.1, left G off by 1.5e-13 where
+// the FP64 pipe's is off by 4e-14.)  The digit planes are BF16 integers; the products of one group
 // g = p + q share one FP32 tensor-memory accumulator, and every partial sum
-// of a group is an integer of magnitude < K (2 * 8192 + 6 * 4096) < 2^24 for
-// K <= 384, so the tensor-core accumulation is exact.  Longer contractions
-// run in chunks of at most 384: the epilogue converts each chunk's eight
+// of a group is an integer of magnitude <= K 2^16 (the leading group; K (2^15 +
+// 6 * 4096) the others) <= 2^24 for K <= 256, so the tensor-core accumulation
+// is exact.  Longer contractions run in chunks of at most 256: the epilogue converts each chunk's eight
 // group sums to integers, combines them in two 64-bit integers, forms the
 // chunk's FP64 value with one rounding and adds the chunks in FP64.
 //
@@ -48,7 +62,8 @@ using namespace tcx;
 constexpr int OZ_S = 8;           // digit planes
 constexpr int OZ_BETA = 7;        // bits per digit
 constexpr int OZ_G = 8;           // groups p + q = 2..9
-constexpr int OZ_KCHUNK = 12;     // K-blocks (of 32) per exactly accumulated chunk: K <= 384
+constexpr int OZ_BITS = 57;       // bits of a scaled entry: x 2^-E = v 2^-57, seven digits below the leading one
+constexpr int OZ_KCHUNK = 8;      // K-blocks (of 32) per exactly accumulated chunk: K <= 256
 constexpr int OBM = 128, OBN = 32;
 constexpr int OKE = 32;           // BF16 elements per K-block (64-byte rows)
 constexpr int OSTAGES = 2;
@@ -58,6 +73,14 @@ constexpr int OSTAGE = OZ_S * (OTILE_A + OTILE_B);
 constexpr int OEPI = 8;            // epilogue warps, two per TMEM lane quarter
 constexpr int OTHREADS = 64 + 32 * OEPI;
 constexpr int OTMEM = 2 * OZ_G * OBN;  // two buffers of eight 32-column accumulators
+
+constexpr int OZ_NONFINITE = 1 << 20;  // exponent of a row with an infinity or a NaN
+
+// Exponent of a row whose largest |entry| has the biased exponent ef_max.
+__device__ __forceinline__ int oz_exponent(int ef_max)
+{
+    return ef_max == 0x7FF ? OZ_NONFINITE : (ef_max > 0 ? ef_max - 1022 : 0);
+}
 
 constexpr size_t oz_smem_bytes() { return (size_t)OSTAGES * OSTAGE + 1024 + 256; }
 
@@ -89,10 +112,10 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, 
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
-// Balanced base-2^7 digits of v = round(|x| 2^(56 - E)) < 2^56 for a double x
+// Balanced base-2^7 digits of v = round(|x| 2^(57 - E)) < 2^57 for a double x
 // with |x| < 2^E (E the frexp exponent of its row's maximum, ef_max its
 // biased exponent, 0 for a row of zeros or subnormals): x 2^-E = sum_p
-// dg[p] 2^-7(p+1), p = 0..7.
+// dg[p] 2^-(7p+8), p = 0..7.
 __device__ __forceinline__ void oz_digits(double x, int E, int ef_max, int dg[OZ_S])
 {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
@@ -101,8 +124,8 @@ __device__ __forceinline__ void oz_digits(double x, int E, int ef_max, int dg[OZ
     if (ef > 0 && ef_max > 0) {
         // x = m 2^(ef - 1075)
         const unsigned long long m = (u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-        const int sh = ef - 1075 + 56 - E;
-        if (sh >= 0) v = (long long)(m << sh);  // sh <= 3 since |x| < 2^E
+        const int sh = ef - 1075 + OZ_BITS - E;
+        if (sh >= 0) v = (long long)(m << sh);  // sh <= 4 since |x| < 2^E
         else if (sh > -60) v = (long long)((m + (1ull << (-sh - 1))) >> (-sh));
     }
 #pragma unroll
@@ -115,31 +138,48 @@ __device__ __forceinline__ void oz_digits(double x, int E, int ef_max, int dg[OZ
         }
         dg[p] = d;
     }
-    dg[0] = (int)v;  // 0..128
+    dg[0] = (int)v;  // 0..256
     if (u >> 63)
 #pragma unroll
         for (int p = 0; p < OZ_S; ++p) dg[p] = -dg[p];
 }
 
-// Digits of the rows of X (rows x cols, row stride ld, item stride sX): row i
-// becomes plane row i (prow plane rows per item, leading dimension ldp) with
-// K positions 0..cols-1 and exponent E[b * prow + i]; the planes' columns
-// beyond cols are left as they are (zero pads of the buffer).  One warp per
-// row, eight rows per CTA: the row's maximum by warp shuffles, then each lane
-// converts pairs of adjacent entries and stores each plane's pair as one
-// BF16x2.
-__global__ void __launch_bounds__(256) k_oz_slice(const double *X, long long sX, int rows, int cols, int ld, int prow,
-                                                  int ldp, long long plane_stride, __nv_bfloat16 *planes, int *E)
+// Digits of the rows of one or two matrices (rows x cols, row stride ld, item
+// stride sX; blockIdx.z selects the matrix): row i becomes plane row i (prow
+// plane rows per item, leading dimension ldp) with K positions 0..cols-1 and
+// exponent E[b * prow + i]; the planes' columns beyond cols are left as they
+// are (zero pads of the buffer).  With a field slice sk the entries of column
+// k are first multiplied by cu where sk > 0 and by cd otherwise (the D of a
+// slice product X D E).  One warp per row, eight rows per CTA: the row's
+// maximum by warp shuffles, then each lane converts pairs of adjacent entries
+// and stores each plane's pair as one BF16x2.
+struct OzRows {
+    const double *X[2];
+    __nv_bfloat16 *planes[2];
+    int *E[2];
+    const int8_t *sk;
+    long long sSk;
+    double cu, cd;
+};
+
+template <bool SCALE>
+__global__ void __launch_bounds__(256) k_oz_slice(OzRows a, long long sX, int rows, int cols, int ld, int prow,
+                                                  int ldp, long long plane_stride)
 {
     const int b = blockIdx.y, lane = threadIdx.x & 31;
     const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= rows) return;  // whole warps
     const int N = cols;
-    const double *x = X + (long long)b * sX + (long long)i * ld;
+    const double *x = (blockIdx.z ? a.X[1] : a.X[0]) + (long long)b * sX + (long long)i * ld;
+    const int8_t *sk = SCALE ? a.sk + (long long)b * a.sSk : nullptr;
+    auto at = [&](int k) {
+        const double v = x[k];
+        return SCALE ? v * (sk[k] > 0 ? a.cu : a.cd) : v;
+    };
     // the largest |x_ik| (non-negative doubles order like their bit patterns)
     unsigned long long mx = 0;
     for (int k = lane; k < N; k += 32) {
-        const unsigned long long u = (unsigned long long)__double_as_longlong(x[k]) & 0x7FFFFFFFFFFFFFFFull;
+        const unsigned long long u = (unsigned long long)__double_as_longlong(at(k)) & 0x7FFFFFFFFFFFFFFFull;
         mx = u > mx ? u : mx;
     }
 #pragma unroll
@@ -148,16 +188,16 @@ __global__ void __launch_bounds__(256) k_oz_slice(const double *X, long long sX,
         mx = v > mx ? v : mx;
     }
     const int ef_max = (int)(mx >> 52);
-    const int Ei = ef_max > 0 ? ef_max - 1022 : 0;
-    if (lane == 0) E[(long long)b * prow + i] = Ei;
-    const long long row = ((long long)b * prow + i) * ldp;
+    const int Ei = oz_exponent(ef_max);
+    if (lane == 0) (blockIdx.z ? a.E[1] : a.E[0])[(long long)b * prow + i] = Ei;
+    __nv_bfloat16 *row = (blockIdx.z ? a.planes[1] : a.planes[0]) + ((long long)b * prow + i) * ldp;
     for (int k = 2 * lane; k < N; k += 64) {
         int d0[OZ_S], d1[OZ_S];
-        oz_digits(x[k], Ei, ef_max, d0);
-        oz_digits(k + 1 < N ? x[k + 1] : 0.0, Ei, ef_max, d1);
+        oz_digits(at(k), Ei, ef_max, d0);
+        oz_digits(k + 1 < N ? at(k + 1) : 0.0, Ei, ef_max, d1);
 #pragma unroll
         for (int p = 0; p < OZ_S; ++p)
-            *reinterpret_cast<__nv_bfloat162 *>(planes + (long long)p * plane_stride + row + k) =
+            *reinterpret_cast<__nv_bfloat162 *>(row + (long long)p * plane_stride + k) =
                 __floats2bfloat162_rn((float)d0[p], (float)d1[p]);
     }
 }
@@ -213,7 +253,7 @@ __device__ __forceinline__ void oz_slice_block(int bx, const double *src, long l
         }
         if (j >= Nc) return;
         const int ef_max = (int)(mx >> 52);
-        const int E = ef_max > 0 ? ef_max - 1022 : 0;
+        const int E = oz_exponent(ef_max);
         if (q == 0) Ej[(long long)b * sE + j] = E;
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj) oz_digits(tile[4 * q + jj][r], E, ef_max, dg[jj]);
@@ -310,7 +350,7 @@ __global__ void __launch_bounds__(256) k_oz_col_max_exponents(const double *src,
 #pragma unroll
         for (int q = 1; q < 8; ++q) mx = part[q][lane] > mx ? part[q][lane] : mx;
         const int ef = (int)(mx >> 52);
-        E[(long long)b * cols + j] = ef > 0 ? ef - 1022 : 0;
+        E[(long long)b * cols + j] = oz_exponent(ef);
     }
 }
 
@@ -442,6 +482,8 @@ struct OzPart {
     int M, arow0;
     const int *EA;
     long long sEA;
+    const int *EB;  // row exponents of the part's B
+    long long sEB;
     double *C;
     long long sC;
     int ldc;
@@ -452,23 +494,29 @@ struct OzPart {
 };
 
 // x 2^e, exact: through the exponent field while the result stays normal
-// (integer arithmetic, off the FP64 pipe), otherwise scalbn.
+// (integer arithmetic, off the FP64 pipe), otherwise scalbn; NaN for the
+// exponent of a row that holds an infinity or a NaN (its digits are zero).
 __device__ __forceinline__ double oz_scale2(double x, int e)
 {
     const long long bits = __double_as_longlong(x);
     const int ex = (int)((bits >> 52) & 0x7FF);
     if (ex != 0 && ex + e > 0 && ex + e < 2047) return __longlong_as_double(bits + ((long long)e << 52));
+    if (e > OZ_NONFINITE / 2) return __longlong_as_double(0x7FF8000000000000ll);
     return scalbn(x, e);
 }
 
 struct OzArgs {
-    OzPart pt[2];           // pt[1] only with nparts = 2 (its A rows through the second A map)
+    OzPart pt[2];           // pt[1] only with nparts = 2 (its A rows and B through the second maps)
     int nparts;
     int Nn, brow0;          // rows of B (columns of C), first plane row of B
     int batch, nk;          // items, 32-wide K-blocks
     int kA0, kB0;           // first K positions (elements) of A and B in their planes
-    const int *EB;          // row exponents of B
-    long long sEB;
+    int b_shared;           // one B for every item
+    int stack;              // > 0: the items' rows lie one after another (batch = 1, M = items x stack), and
+                            // row m of the product belongs to row m % stack of item m / stack of C
+    const int8_t *sgn;      // TRANS without SUB, stacked: C[n][i] is scaled by d_n / d_i, d = cu where the item's
+    long long sSgn;         // field slice is > 0 and cd otherwise (r_ud = cu / cd, r_du = cd / cu)
+    double r_ud[2], r_du[2];  // per part
     long long splane_stride;  // SLICE: plane stride, leading dimension, plane rows per item,
     int sldp, srows, skoff;   // and the K position of n = 0
     int a_tri, b_tri;         // A upper triangular (A[m][k] = 0 for k < m) / B^T upper triangular
@@ -579,7 +627,7 @@ __device__ __forceinline__ void oz_locate(const OzArgs &a, int t, int tiles0, in
 template <bool UPPER, bool SUB, bool TRANS = false, bool SLICE = false>
 __global__ void __launch_bounds__(OTHREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap tA0, const __grid_constant__ CUtensorMap tA1,
-              const __grid_constant__ CUtensorMap tB, OzArgs a)
+              const __grid_constant__ CUtensorMap tB0, const __grid_constant__ CUtensorMap tB1, OzArgs a)
 {
     static_assert(!SLICE || (TRANS && !SUB), "SLICE needs TRANS and C = A B^T");
     extern __shared__ uint8_t smem_raw[];
@@ -624,6 +672,8 @@ __global__ void __launch_bounds__(OTHREADS, 1)
                 int part, b, m0, n0;
                 oz_locate<UPPER>(a, t, tiles0, part, b, m0, n0);
                 const CUtensorMap *mA = part ? &tA1 : &tA0;
+                const CUtensorMap *mB = part ? &tB1 : &tB0;
+                const int bB = a.b_shared ? 0 : b;
                 const int arow0 = part ? a.pt[1].arow0 : a.pt[0].arow0;
                 int k_lo, k_hi;
                 oz_krange(a, m0, n0, k_lo, k_hi);
@@ -636,7 +686,7 @@ __global__ void __launch_bounds__(OTHREADS, 1)
 #pragma unroll
                     for (int p = 0; p < OZ_S; ++p) {
                         tma_load_4d(st + p * OTILE_A, mA, a.kA0 + k0, arow0 + m0, b, p, &full[s]);
-                        tma_load_4d(st + OZ_S * OTILE_A + p * OTILE_B, &tB, a.kB0 + k0, a.brow0 + n0, b, p, &full[s]);
+                        tma_load_4d(st + OZ_S * OTILE_A + p * OTILE_B, mB, a.kB0 + k0, a.brow0 + n0, bB, p, &full[s]);
                     }
                 }
             }
@@ -703,10 +753,11 @@ __global__ void __launch_bounds__(OTHREADS, 1)
             const int Ei = mm < M ? EA[(long long)b * sEA + mm] : 0;
             // element (mm, n) at o[n * cs]; for an update, the old values of this
             // thread's row segment, fetched while the MMAs run
-            double *o = C + (long long)b * sC + (TRANS ? (long long)mm : (long long)mm * ldc);
+            const int item = a.stack ? mm / a.stack : b, mi = a.stack ? mm - item * a.stack : mm;
+            double *o = C + (long long)item * sC + (TRANS ? (long long)mi : (long long)mi * ldc);
             const long long cs = TRANS ? ldc : 1;
             const int nb = n0 + hc;
-            const int *eb = a.EB + (long long)b * a.sEB;
+            const int *eb = (part ? a.pt[1].EB : a.pt[0].EB) + (a.b_shared ? 0 : (long long)b * (part ? a.pt[1].sEB : a.pt[0].sEB));
             double cold[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) cold[j] = (SUB && mm < M && nb + j < a.Nn) ? o[(nb + j) * cs] : 0.0;
@@ -730,7 +781,7 @@ __global__ void __launch_bounds__(OTHREADS, 1)
                 for (int half = 0; half < 2; ++half) {
                     // group sums as exact integers, folded as they arrive: groups 0..3
                     // (p + q = 2..5) into h, 4..7 (6..9) into l, so that
-                    // sum_g acc_g 2^-7(g+2) = h 2^-35 + l 2^-63
+                    // sum_g acc_g 2^-(7(g+2)+2) = h 2^-37 + l 2^-65
                     long long h[8], l[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) h[j] = l[j] = 0;
@@ -763,12 +814,18 @@ __global__ void __launch_bounds__(OTHREADS, 1)
             }
             if (!ok) break;
             if (mm >= M) continue;
+            const int8_t *sg = (TRANS && !SUB && !SLICE && a.sgn) ? a.sgn + (long long)item * a.sSgn : nullptr;
+            const bool up = sg && sg[mi] > 0;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const int n = nb + j;
                 double v = 0.0;
                 if (n < a.Nn) {
-                    v = oz_scale2(w[j], Ei + (SUB ? eb[n] : ebv[j]) - 35);
+                    v = oz_scale2(w[j], Ei + (SUB ? eb[n] : ebv[j]) - 37);
+                    if (sg) {
+                        const bool un = sg[n] > 0;
+                        if (un != up) v *= un ? a.r_ud[part] : a.r_du[part];
+                    }
                     o[n * cs] = SUB ? cold[j] - v : v;
                 }
                 if (SLICE) w[j] = v;
@@ -835,6 +892,20 @@ struct OzWs {
     long long tplane_stride;
     int *ET, *EPY, *EPW;
     CUtensorMap mapT;
+    CUtensorMap mapAS, mapRAS;  // planes and rplanes with the items' rows one after another (128-row boxes)
+    // rank-32 updates: digit planes of the N x 32 left factors (two matrices
+    // per item), their row exponents
+    __nv_bfloat16 *lplanes[2];
+    long long lplane_stride;
+    int *EL[2];
+    CUtensorMap mapL[2];
+    // digit planes of exp(-dtau K) and exp(+dtau K) (built on first use)
+    void *emem;
+    long long eplane_stride;
+    __nv_bfloat16 *eplanes[2];
+    int *EE[2];
+    CUtensorMap mapE[2];
+    int e_tried;
     int num_sms;
 };
 
@@ -866,24 +937,44 @@ int oz_prepare(sldqmc_ctx *c)
     w->tplane_stride = (long long)c->cap * 32 * 32;
     const size_t tbytes = (size_t)OZ_S * w->tplane_stride * sizeof(__nv_bfloat16);
     const size_t tebytes = sizeof(int) * (size_t)c->cap * 32;
-    const size_t eoff = 2 * pbytes + tbytes;  // the int arrays follow the planes
+    w->lplane_stride = (long long)c->cap * N * 32;
+    const size_t lbytes = (size_t)OZ_S * w->lplane_stride * sizeof(__nv_bfloat16);
+    const size_t eoff = 2 * pbytes + tbytes + 2 * lbytes;  // the int arrays follow the planes
+    const size_t total = eoff + 7 * ebytes + tebytes + sizeof(int) * N;
+    // The FP64 mode also runs without this workspace (on the FP64 pipe), so
+    // there it is taken only when it leaves most of the free memory.
+    const bool optional = c->p.prec == SLDQMC_FP64;
+    if (optional) {
+        size_t free_b = 0, total_b = 0;
+        if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || 3.0 * (double)total > (double)free_b) {
+            cudaGetLastError();
+            delete w;
+            return SLDQMC_OK;
+        }
+    }
     void *mem = nullptr;
-    if (cudaMalloc(&mem, eoff + 5 * ebytes + tebytes + sizeof(int) * N) != cudaSuccess) {
+    if (cudaMalloc(&mem, total) != cudaSuccess) {
         cudaGetLastError();
         delete w;
-        return SLDQMC_ERR_OOM;
+        return optional ? SLDQMC_OK : SLDQMC_ERR_OOM;
     }
     w->planes = (__nv_bfloat16 *)mem;
     w->rplanes = (__nv_bfloat16 *)((uint8_t *)mem + pbytes);
     w->tplanes = (__nv_bfloat16 *)((uint8_t *)mem + 2 * pbytes);
+    w->lplanes[0] = (__nv_bfloat16 *)((uint8_t *)mem + 2 * pbytes + tbytes);
+    w->lplanes[1] = (__nv_bfloat16 *)((uint8_t *)mem + 2 * pbytes + tbytes + lbytes);
     w->E = (int *)((uint8_t *)mem + eoff);
     w->ER = w->E + (size_t)c->cap * N;
     w->ER1 = w->ER + (size_t)c->cap * N;
     w->EPY = w->ER1 + (size_t)c->cap * N;
     w->EPW = w->EPY + (size_t)c->cap * N;
-    w->ET = w->EPW + (size_t)c->cap * N;
+    w->EL[0] = w->EPW + (size_t)c->cap * N;
+    w->EL[1] = w->EL[0] + (size_t)c->cap * N;
+    w->ET = w->EL[1] + (size_t)c->cap * N;
     w->EQ = w->ET + (size_t)c->cap * 32;
-    cudaMemsetAsync(mem, 0, eoff + 5 * ebytes + tebytes, c->st);  // zero pads: never written
+    w->emem = nullptr;
+    w->e_tried = 0;
+    cudaMemsetAsync(mem, 0, eoff + 7 * ebytes + tebytes, c->st);  // zero pads: never written
     {
         std::vector<int> ones((size_t)N, 1);
         if (cudaMemcpyAsync(w->EQ, ones.data(), sizeof(int) * N, cudaMemcpyHostToDevice, c->st) != cudaSuccess ||
@@ -896,7 +987,11 @@ int oz_prepare(sldqmc_ctx *c)
     if (!encode4(&w->mapA, w->planes, w->ldp, N, c->cap, OBM) || !encode4(&w->mapB, w->planes, w->ldp, N, c->cap, OBN) ||
         !encode4(&w->mapRA, w->rplanes, w->ldp, N, c->cap, OBM) ||
         !encode4(&w->mapRB, w->rplanes, w->ldp, N, c->cap, OBN) ||
-        !encode4(&w->mapT, w->tplanes, 32, 32, c->cap, OBN)) {
+        !encode4(&w->mapT, w->tplanes, 32, 32, c->cap, OBN) ||
+        !encode4(&w->mapAS, w->planes, w->ldp, N * c->cap, 1, OBM) ||
+        !encode4(&w->mapRAS, w->rplanes, w->ldp, N * c->cap, 1, OBM) ||
+        !encode4(&w->mapL[0], w->lplanes[0], 32, N, c->cap, OBN) ||
+        !encode4(&w->mapL[1], w->lplanes[1], 32, N, c->cap, OBN)) {
         cudaFree(mem);
         delete w;
         return SLDQMC_ERR_CUDA;
@@ -905,14 +1000,12 @@ int oz_prepare(sldqmc_ctx *c)
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&w->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || w->num_sms < 1)
         w->num_sms = 148;
-    cudaFuncSetAttribute(k_oz_gemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oz_smem_bytes());
-    cudaFuncSetAttribute(k_oz_gemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oz_smem_bytes());
-    cudaFuncSetAttribute(k_oz_gemm<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)oz_smem_bytes());
-    cudaFuncSetAttribute(k_oz_gemm<false, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)oz_smem_bytes());
-    cudaFuncSetAttribute(k_oz_gemm<false, true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)oz_smem_bytes());
+    const int sh = (int)oz_smem_bytes();
+    cudaFuncSetAttribute(k_oz_gemm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh);
+    cudaFuncSetAttribute(k_oz_gemm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh);
+    cudaFuncSetAttribute(k_oz_gemm<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh);
+    cudaFuncSetAttribute(k_oz_gemm<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh);
+    cudaFuncSetAttribute(k_oz_gemm<false, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh);
     c->oz_ws = w;
     return SLDQMC_OK;
 }
@@ -922,23 +1015,41 @@ void oz_release(sldqmc_ctx *c)
     OzWs *w = (OzWs *)c->oz_ws;
     if (!w) return;
     cudaFree(w->planes);
+    cudaFree(w->emem);
     delete w;
     c->oz_ws = nullptr;
 }
 
 namespace {
 
-OzPart oz_part(int M, int arow0, const int *EA, long long sEA, double *C, long long sC, int ldc)
+OzPart oz_part(int M, int arow0, const int *EA, long long sEA, const int *EB, long long sEB, double *C, long long sC,
+               int ldc)
 {
     OzPart p{};
     p.M = M;
     p.arow0 = arow0;
     p.EA = EA;
     p.sEA = sEA;
+    p.EB = EB;
+    p.sEB = sEB;
     p.C = C;
     p.sC = sC;
     p.ldc = ldc;
     return p;
+}
+
+// Rows of one matrix (or of two, X2 into rplanes and E2) split with their own maxima.
+void oz_slice_rows(sldqmc_ctx *c, const double *X, const double *X2, int *E2, long long sX, int rows, int cols, int ld, int B,
+                   const int8_t *sk = nullptr, double cu = 1.0, double cd = 1.0)
+{
+    OzWs *w = (OzWs *)c->oz_ws;
+    OzRows r{{X, X2}, {w->planes, w->rplanes}, {w->E, E2}, sk, (long long)c->M * c->N, cu, cd};
+    const dim3 grid((rows + 7) / 8, B, X2 ? 2 : 1);
+    prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice");
+    if (sk) k_oz_slice<true><<<grid, 256, 0, c->st>>>(r, sX, rows, cols, ld, c->N, w->ldp, w->plane_stride);
+    else k_oz_slice<false><<<grid, 256, 0, c->st>>>(r, sX, rows, cols, ld, c->N, w->ldp, w->plane_stride);
+    prof_end(c);
+    c->launches++;
 }
 
 template <bool UPPER>
@@ -956,23 +1067,19 @@ void oz_gram(sldqmc_ctx *c, const double *X, long long sX, double *W, long long 
 {
     OzWs *w = (OzWs *)c->oz_ws;
     const int N = c->N;
-    prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice");
-    k_oz_slice<<<dim3((N + 7) / 8, B), 256, 0, c->st>>>(X, sX, N, N, N, N, w->ldp, w->plane_stride, w->planes,
-                                                         w->E);
-    prof_end(c);
+    oz_slice_rows(c, X, nullptr, nullptr, sX, N, N, N, B);
     OzArgs a{};
-    a.pt[0] = oz_part(N, 0, w->E, N, W, sW, ldw);
+    a.pt[0] = oz_part(N, 0, w->E, N, w->E, N, W, sW, ldw);
     a.nparts = 1;
     a.Nn = N;
     a.batch = B;
     a.nk = w->ldp / OKE;
-    a.EB = w->E;
-    a.sEB = N;
     a.flag = c->d_flag;
     prof_begin(c, SLDQMC_KC_GEMM_OZ, (double)N * N * (N + 1) * B, "oz_gram");
-    k_oz_gemm<true, false><<<oz_grid<true>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapA, w->mapB, a);
+    k_oz_gemm<true, false>
+        <<<oz_grid<true>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapA, w->mapB, w->mapB, a);
     prof_end(c);
-    c->launches += 2;
+    c->launches++;
 }
 
 // Left-looking Cholesky-QR of W = X X^T (row stride N, item stride sW) that
@@ -1002,8 +1109,9 @@ void oz_chol_update(sldqmc_ctx *c, int k0, int kb, int kstart, double *W, long l
     OzWs *w = (OzWs *)c->oz_ws;
     const int N = c->N;
     OzArgs a{};
-    a.pt[0] = oz_part(N, 0, w->EQ, 0, Y + (long long)k0 * N, c->nn, N);                    // rows n: columns of Q^T
-    a.pt[1] = oz_part(N - k0, k0, w->ER + k0, N, W + (long long)k0 * N + k0, sW, N);      // rows n: columns k0.. of R
+    // rows n of the parts: columns of Q^T, columns k0.. of R
+    a.pt[0] = oz_part(N, 0, w->EQ, 0, w->ER + k0, N, Y + (long long)k0 * N, c->nn, N);
+    a.pt[1] = oz_part(N - k0, k0, w->ER + k0, N, w->ER + k0, N, W + (long long)k0 * N + k0, sW, N);
     a.nparts = 2;
     a.Nn = kb;
     a.brow0 = k0;
@@ -1011,13 +1119,11 @@ void oz_chol_update(sldqmc_ctx *c, int k0, int kb, int kstart, double *W, long l
     a.kA0 = kstart;
     a.kB0 = kstart;
     a.nk = (k0 - kstart) / OKE;
-    a.EB = w->ER + k0;
-    a.sEB = N;
     a.flag = c->d_flag;
     prof_begin(c, SLDQMC_KC_GEMM_OZ, 2.0 * (2 * N - k0) * kb * (k0 - kstart) * B,
                kstart ? "oz_chol_update_inner" : "oz_chol_update");
     k_oz_gemm<false, true, true>
-        <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapRA, w->mapRB, a);
+        <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapRA, w->mapRB, w->mapRB, a);
     prof_end(c);
     c->launches++;
 }
@@ -1057,12 +1163,12 @@ void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW,
                                            c->d_flag);
     prof_end(c);
     OzArgs a{};
-    a.pt[0] = oz_part(N, 0, w->EPY, N, Y + (long long)k0 * N, c->nn, N);
+    a.pt[0] = oz_part(N, 0, w->EPY, N, w->ET, 32, Y + (long long)k0 * N, c->nn, N);
     a.pt[0].sp = w->planes;
     a.pt[0].SE = w->EQ;
     a.pt[0].sSE = 0;
     a.pt[0].srow0 = 0;
-    a.pt[1] = oz_part(nW, j0, w->EPW + j0, N, R + (long long)k0 * N + j0, c->nn, N);
+    a.pt[1] = oz_part(nW, j0, w->EPW + j0, N, w->ET, 32, R + (long long)k0 * N + j0, c->nn, N);
     a.pt[1].sp = w->rplanes;
     a.pt[1].SE = w->ER;
     a.pt[1].sSE = N;
@@ -1074,8 +1180,6 @@ void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW,
     a.nk = 1;
     a.kA0 = k0;
     a.kB0 = 0;
-    a.EB = w->ET;
-    a.sEB = 32;
     a.splane_stride = w->plane_stride;
     a.sldp = w->ldp;
     a.srows = N;
@@ -1083,50 +1187,200 @@ void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW,
     a.flag = c->d_flag;
     prof_begin(c, SLDQMC_KC_GEMM_OZ, 2.0 * (N + nW) * kb * kb * B, "oz_chol_panel");
     k_oz_gemm<false, false, true, true>
-        <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapRA, w->mapT, a);
+        <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapRA, w->mapT, w->mapT, a);
     prof_end(c);
     c->launches += 3;
 }
 
-// Trailing update of the finalisation's blocked LU without a right-hand
-// side, A[i][j] -= sum_l L[i][k0+l] U[k0+l][j] for i, j >= k0 + kb (A row
-// stride lda, item stride sA), FP64-accurate on the tensor cores: the rows of
-// L21 and the columns of U12 each split with their own maximum (K = kb = 32,
-// one exactly accumulated chunk).
-void oz_lu_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B)
+namespace {
+
+// Rank-32 updates C[i][j] -= sum_l L[i][l] R[l][j] of up to two matrices or
+// column ranges, FP64-accurate on the tensor cores: the rows of L (rows x
+// kb, row stride ldl) and the columns of R each split with their own maximum
+// (K = kb <= 32, one exactly accumulated chunk).  The product is computed
+// with rows j and columns i and stored transposed, so that a warp's 32 reads
+// and writes of C are contiguous.
+struct RankPart {
+    const double *L;  // null: the first part's
+    const double *R;  // kb x cols, columns j0 .. j0 + cols - 1 of a matrix whose row 0 starts at R
+    int j0, cols;
+    double *C;        // element (0, j0)
+};
+
+void oz_rank_update(sldqmc_ctx *c, const RankPart *pt, int nparts, int rows, int kb, long long ldl, long long sL,
+                    long long ldr, long long sR, int ldc, long long sC, int B, const char *site)
 {
     OzWs *w = (OzWs *)c->oz_ws;
     const int N = c->N;
-    const int j0 = k0 + kb, M = N - j0;
-    prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice");
-    k_oz_slice<<<dim3((M + 7) / 8, B), 256, 0, c->st>>>(A + (long long)j0 * lda + k0, sA, M, kb, lda, N, w->ldp,
-                                                         w->plane_stride, w->planes, w->E);
-    prof_end(c);
+    const bool two_l = nparts > 1 && pt[1].L;
+    {
+        OzRows r{{pt[0].L, two_l ? pt[1].L : nullptr}, {w->lplanes[0], w->lplanes[1]}, {w->EL[0], w->EL[1]}, nullptr, 0, 1.0, 1.0};
+        prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice");
+        k_oz_slice<false><<<dim3((rows + 7) / 8, B, two_l ? 2 : 1), 256, 0, c->st>>>(r, sL, rows, kb, (int)ldl, N, 32,
+                                                                                   w->lplane_stride);
+        prof_end(c);
+    }
     OzPanelSlice sl{};
-    sl.src[0] = A + (long long)k0 * lda;
-    sl.sS[0] = sA;
-    sl.j0[0] = j0;
-    sl.planes[0] = w->rplanes;
-    sl.E[0] = w->EPW;
-    sl.nb0 = (M + 31) / 32;
-    prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice_panel");
-    k_oz_slice_panel<<<dim3(sl.nb0, B), 256, 0, c->st>>>(sl, N, lda, kb, 0, w->plane_stride, w->ldp, c->d_flag);
-    prof_end(c);
     OzArgs a{};
-    a.pt[0] = oz_part(M, 0, w->E, N, A + (long long)j0 * lda + j0, sA, lda);
-    a.nparts = 1;
-    a.Nn = M;
-    a.brow0 = j0;
+    double cols = 0.0;
+    __nv_bfloat16 *pl[2] = {w->rplanes, w->planes};
+    int *ep[2] = {w->EPW, w->EPY};
+    for (int p = 0; p < nparts; ++p) {
+        sl.src[p] = pt[p].R;
+        sl.sS[p] = sR;
+        sl.j0[p] = pt[p].j0;
+        sl.planes[p] = pl[p];
+        sl.E[p] = ep[p];
+        a.pt[p] = oz_part(pt[p].cols, pt[p].j0, ep[p] + pt[p].j0, N, w->EL[p && two_l], N, pt[p].C, sC, ldc);
+        cols += pt[p].cols;
+    }
+    const int nb0 = (pt[0].cols + 31) / 32, nb1 = nparts > 1 ? (pt[1].cols + 31) / 32 : 0;
+    sl.nb0 = nb0;
+    prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice_panel");
+    k_oz_slice_panel<<<dim3(nb0 + nb1, B), 256, 0, c->st>>>(sl, N, (int)ldr, kb, 0, w->plane_stride, w->ldp, c->d_flag);
+    prof_end(c);
+    a.nparts = nparts;
+    a.Nn = rows;
     a.batch = B;
     a.nk = 1;
-    a.EB = w->EPW + j0;
-    a.sEB = N;
     a.flag = c->d_flag;
-    prof_begin(c, SLDQMC_KC_GEMM_OZ, 2.0 * M * M * kb * B, "oz_lu_update");
-    k_oz_gemm<false, true, false, false>
-        <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapA, w->mapRB, a);
+    prof_begin(c, SLDQMC_KC_GEMM_OZ, 2.0 * rows * cols * kb * B, site);
+    k_oz_gemm<false, true, true><<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(
+        w->mapRA, w->mapA, w->mapL[0], w->mapL[two_l], a);
     prof_end(c);
     c->launches += 3;
+}
+
+// Digit planes of exp(-dtau K) and exp(+dtau K), on first use; false when
+// there is no room for them (the callers then stay on the FP64 pipe).
+bool oz_e_planes(sldqmc_ctx *c)
+{
+    OzWs *w = (OzWs *)c->oz_ws;
+    if (w->e_tried) return w->emem != nullptr;
+    w->e_tried = 1;
+    const int N = c->N;
+    w->eplane_stride = (long long)N * w->ldp;
+    const size_t pb = (size_t)OZ_S * w->eplane_stride * sizeof(__nv_bfloat16);
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || 6.0 * (double)pb > (double)free_b ||
+        cudaMalloc(&w->emem, 2 * pb + 2 * sizeof(int) * N) != cudaSuccess) {
+        cudaGetLastError();
+        w->emem = nullptr;
+        return false;
+    }
+    cudaMemsetAsync(w->emem, 0, 2 * pb, c->st);
+    for (int e = 0; e < 2; ++e) {
+        w->eplanes[e] = (__nv_bfloat16 *)((uint8_t *)w->emem + e * pb);
+        w->EE[e] = (int *)((uint8_t *)w->emem + 2 * pb) + e * N;
+        if (!encode4(&w->mapE[e], w->eplanes[e], w->ldp, N, 1, OBN)) {
+            cudaFree(w->emem);  // waits for the memset
+            w->emem = nullptr;
+            return false;
+        }
+    }
+    OzRows r{{c->d_E, c->d_Einv}, {w->eplanes[0], w->eplanes[1]}, {w->EE[0], w->EE[1]}, nullptr, 0, 1.0, 1.0};
+    k_oz_slice<false><<<dim3((N + 7) / 8, 1, 2), 256, 0, c->st>>>(r, 0, N, N, N, N, w->ldp, w->eplane_stride);
+    c->launches++;
+    return true;
+}
+
+}  // namespace
+
+// Trailing update of the finalisation's blocked LU, A[i][j] -= sum_l L[i][k0+l]
+// U[k0+l][j] for i, j >= k0 + kb; with rhs also for the right-hand side's
+// columns N..2N-1.
+void oz_lu_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B, int rhs)
+{
+    const int N = c->N, j0 = k0 + kb;
+    double *low = A + (long long)j0 * lda;  // row k0 + kb
+    const RankPart pt[2] = {{low + k0, A + (long long)k0 * lda, j0, N - j0, low + j0},
+                            {nullptr, A + (long long)k0 * lda + N, 0, N, low + N}};
+    oz_rank_update(c, pt, rhs ? 2 : 1, N - j0, kb, lda, sA, lda, sA, lda, sA, B, "oz_lu_update");
+}
+
+// Back substitution: the rows above k0 of the right-hand side lose the share
+// of its solved rows k0..k0+kb, Y[i][j] -= sum_l U[i][k0+l] X[k0+l][j].
+void oz_back_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B)
+{
+    const int N = c->N;
+    const RankPart pt = {A + k0, A + (long long)k0 * lda + N, 0, N, A + N};
+    oz_rank_update(c, &pt, 1, k0, kb, lda, sA, lda, sA, lda, sA, B, "oz_back_update");
+}
+
+// The pending rank-32 corrections of the delayed local update, G_f -= U_f V_f.
+void oz_delayed_update(sldqmc_ctx *c, double *const *G, const double *const *U, const double *const *V, int B)
+{
+    const int N = c->N;
+    const RankPart pt[2] = {{U[0], V[0], 0, N, G[0]}, {U[1], V[1], 0, N, G[1]}};
+    oz_rank_update(c, pt, 2, N, 32, 32, 32LL * N, N, 32LL * N, N, c->nn, B, "oz_delayed_update");
+}
+
+bool oz_have_e(sldqmc_ctx *c) { return c->oz_ws && oz_e_planes(c); }
+
+// FP64-accurate slice product X^T D E for B items into Xt (which may be X
+// itself): the rows of X^T D split with their own maxima against E's planes.
+// The rows of all items lie one after another, so a 128-row tile may span
+// items and only the last tile is ragged.
+void oz_slice_product(sldqmc_ctx *c, const double *X, const int8_t *sk, double cu, double cd, double *Xt, int B)
+{
+    OzWs *w = (OzWs *)c->oz_ws;
+    const int N = c->N;
+    oz_slice_rows(c, X, nullptr, nullptr, c->nn, N, N, N, B, sk, cu, cd);
+    OzArgs a{};
+    a.pt[0] = oz_part(B * N, 0, w->E, 0, w->EE[0], 0, Xt, c->nn, N);
+    a.nparts = 1;
+    a.Nn = N;
+    a.batch = 1;
+    a.b_shared = 1;
+    a.stack = N;
+    a.nk = w->ldp / OKE;
+    a.flag = c->d_flag;
+    prof_begin(c, SLDQMC_KC_GEMM_OZ, 2.0 * N * N * N * B, "oz_slice_product");
+    k_oz_gemm<false, false>
+        <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapAS, w->mapAS, w->mapE[0], w->mapE[0], a);
+    prof_end(c);
+    c->launches++;
+}
+
+// dst_f = P src_f P^-1 for both flavours f (B items each), with P = E (inv =
+// 0) or E^-1 (inv = 1); with a field slice s, row i and column j of dst_f are
+// scaled by d_i / d_j (d_f = cu[f] where s > 0, cd[f] otherwise).  T = src P^-1
+// is stored transposed, so that its columns are the rows of the second
+// product dst^T = T^T P.
+void oz_similarity(sldqmc_ctx *c, const double *const *src, double *const *T, double *const *dst, int inv,
+                   const int8_t *s, const double (*ex)[2], int B)
+{
+    OzWs *w = (OzWs *)c->oz_ws;
+    const int N = c->N;
+    for (int k = 0; k < 2; ++k) {
+        const int e = k == 0 ? !inv : inv;  // E^-1 first in the wrap
+        const double *const *in = k == 0 ? src : T;
+        double *const *out = k == 0 ? T : dst;
+        oz_slice_rows(c, in[0], in[1], w->EPW, c->nn, N, N, N, B);
+        OzArgs a{};
+        a.pt[0] = oz_part(B * N, 0, w->E, 0, w->EE[e], 0, out[0], c->nn, N);
+        a.pt[1] = oz_part(B * N, 0, w->EPW, 0, w->EE[e], 0, out[1], c->nn, N);
+        a.nparts = 2;
+        a.Nn = N;
+        a.batch = 1;
+        a.b_shared = 1;
+        a.stack = N;
+        a.nk = w->ldp / OKE;
+        if (k == 1 && s) {
+            a.sgn = s;
+            a.sSgn = (long long)c->M * N;
+            for (int f = 0; f < 2; ++f) {
+                a.r_ud[f] = ex[f][0] / ex[f][1];
+                a.r_du[f] = ex[f][1] / ex[f][0];
+            }
+        }
+        a.flag = c->d_flag;
+        prof_begin(c, SLDQMC_KC_GEMM_OZ, 4.0 * N * N * N * B, "oz_similarity");
+        k_oz_gemm<false, false, true>
+            <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapAS, w->mapRAS, w->mapE[e], w->mapE[e], a);
+        prof_end(c);
+        c->launches++;
+    }
 }
 
 // V <- T P^T V with T = D^-1 R D_p (upper triangular; R row stride N),
@@ -1140,27 +1394,25 @@ void oz_update_V(sldqmc_ctx *c, const double *R, double *V, double *Ts, int B)
     prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_make_T");
     k_oz_make_T<<<dim3((N + 255) / 256, N, B), 256, 0, c->st>>>(R, c->nn, N, c->d_D, c->d_Dp, Ts);
     prof_end(c);
-    k_oz_slice<<<dim3((N + 7) / 8, B), 256, 0, c->st>>>(Ts, c->nn, N, N, N, N, w->ldp, w->plane_stride, w->planes,
-                                                         w->E);
+    oz_slice_rows(c, Ts, nullptr, nullptr, c->nn, N, N, N, B);
     prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_col_max_exponents");
     k_oz_col_max_exponents<<<dim3((N + 31) / 32, B), 256, 0, c->st>>>(V, c->nn, N, N, w->ER1);
     prof_end(c);
     k_oz_slice_fixed<<<dim3((N + 31) / 32, B, (N + 31) / 32), 256, 0, c->st>>>(
         V, c->nn, N, 0, N, N, 0, w->plane_stride, N, w->ldp, w->rplanes, w->ER1, N, c->d_flag, c->d_perm, N);
     OzArgs a{};
-    a.pt[0] = oz_part(N, 0, w->E, N, V, c->nn, N);
+    a.pt[0] = oz_part(N, 0, w->E, N, w->ER1, N, V, c->nn, N);
     a.nparts = 1;
     a.Nn = N;
     a.batch = B;
     a.nk = w->ldp / OKE;
-    a.EB = w->ER1;
-    a.sEB = N;
     a.a_tri = 1;  // T is upper triangular: tile rows m0.. need K >= m0 only
     a.flag = c->d_flag;
     prof_begin(c, SLDQMC_KC_GEMM_OZ, (double)N * N * (N + 1) * B, "oz_update_V");
-    k_oz_gemm<false, false><<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapA, w->mapRB, a);
+    k_oz_gemm<false, false>
+        <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapA, w->mapRB, w->mapRB, a);
     prof_end(c);
-    c->launches += 5;
+    c->launches += 4;
 }
 
 // Keeps the current column bounds of R (a first Cholesky-QR pass) for the
@@ -1179,27 +1431,23 @@ void oz_r2r1(sldqmc_ctx *c, const double *R2, const double *R1, double *R, int B
 {
     OzWs *w = (OzWs *)c->oz_ws;
     const int N = c->N;
-    prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice");
-    k_oz_slice<<<dim3((N + 7) / 8, B), 256, 0, c->st>>>(R2, c->nn, N, N, N, N, w->ldp, w->plane_stride, w->planes,
-                                                         w->E);
-    prof_end(c);
+    oz_slice_rows(c, R2, nullptr, nullptr, c->nn, N, N, N, B);
     k_oz_slice_fixed<<<dim3((N + 31) / 32, B, (N + 31) / 32), 256, 0, c->st>>>(
         R1, c->nn, N, 0, N, N, 0, w->plane_stride, N, w->ldp, w->rplanes, w->ER1, N, c->d_flag);
     OzArgs a{};
-    a.pt[0] = oz_part(N, 0, w->E, N, R, c->nn, N);
+    a.pt[0] = oz_part(N, 0, w->E, N, w->ER1, N, R, c->nn, N);
     a.nparts = 1;
     a.Nn = N;
     a.batch = B;
     a.nk = w->ldp / OKE;
-    a.EB = w->ER1;
-    a.sEB = N;
     a.a_tri = 1;  // R2[m][l] = 0 for l < m and R1[l][n] = 0 for l > n
     a.b_tri = 1;
     a.flag = c->d_flag;
     prof_begin(c, SLDQMC_KC_GEMM_OZ, (double)N * N * N / 3.0 * B, "oz_r2r1");
-    k_oz_gemm<true, false><<<oz_grid<true>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapA, w->mapRB, a);
+    k_oz_gemm<true, false>
+        <<<oz_grid<true>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapA, w->mapRB, w->mapRB, a);
     prof_end(c);
-    c->launches += 3;
+    c->launches += 2;
 }
 
 }  // namespace sldqmc

@@ -197,11 +197,16 @@ int weight_run(sldqmc_ctx *c, const int8_t *d_s, int B, int eta, int tau0, doubl
     double *Ut = c->buf[0], *Yb = c->buf[5], *X1 = c->buf[2], *X2 = c->buf[3];
     launch_init_udv(c, Ut, c->buf[1], B);
     std::vector<int> slices;
+    const bool oz = c->p.prec == SLDQMC_FP64 && c->kinetic != SLDQMC_KINETIC_SEPARABLE && oz_have_e(c);
     for (int m = 0; m < M; m += c->p.n_wrap) {
         const int nb = std::min(c->p.n_wrap, M - m);
         double *Xt;
         if (c->kinetic == SLDQMC_KINETIC_SEPARABLE) {
             sep_chain_block(c, Ut, d_s, B, cu, cd, (tau0 + m) % M, nb, c->d_Einv + nn, X1);
+            Xt = X1;
+        } else if (oz) {
+            for (int j = 0; j < nb; ++j)
+                oz_slice_product(c, j == 0 ? Ut : X1, d_s + (long long)((tau0 + m + j) % M) * N, cu, cd, X1, B);
             Xt = X1;
         } else if (c->p.prec == SLDQMC_FP64) {
             const double *cur = Ut;
@@ -374,8 +379,14 @@ static void local_flips_slice(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s
     for (int i0 = 0; i0 < N; i0 += c->local_rank) {
         const int ns = std::min(c->local_rank, N - i0);
         launch_local_flips_delayed(c, Gp, Gm, c->d_U, c->d_V, d_s, B, tau, i0, ns, sweep, seed, c->d_stats);
+        const long long so1 = (long long)c->cap * 32 * N;
+        if (c->oz_ws) {
+            const double *U[2] = {c->d_U, c->d_U + so1}, *V[2] = {c->d_V, c->d_V + so1};
+            oz_delayed_update(c, G, U, V, B);
+            continue;
+        }
         for (int f = 0; f < 2; ++f) {
-            const long long so = (long long)f * c->cap * 32 * N;
+            const long long so = f * so1;
             GemmF64 g = gemm_desc(N, N, 32, c->d_U + so, 32, 32LL * N, c->d_V + so, N, 32LL * N, G[f], N, c->nn, B);
             g.alpha = -1.0;
             g.beta = 1.0;
@@ -657,7 +668,7 @@ int sldqmc_create(const sldqmc_params *p, void *stream, sldqmc_ctx **out)
     c->d_ld_tmp2 = c->d_ld_tmp + cap;
     if ((rc = dalloc(&c->d_stats, 4 * cap + 8 * cap))) goto fail;
     if (p->prec != SLDQMC_FP64 && (rc = tc_prepare(c))) goto fail;
-    if (p->prec != SLDQMC_FP64 && (rc = oz_prepare(c))) goto fail;
+    if ((rc = oz_prepare(c))) goto fail;
     {
         // build K, E, E^{-1}
         double *ex_p = c->d_Einv + nn, *ey_p = ex_p + p->Lx, *ex_m = ey_p + p->Ly, *ey_m = ex_m + p->Lx;
@@ -672,6 +683,7 @@ int sldqmc_create(const sldqmc_params *p, void *stream, sldqmc_ctx **out)
         c->launches += 5;
     }
     if (p->prec != SLDQMC_FP64) tc_convert_E(c);
+    else oz_have_e(c);  // not in the first call, which may be under capture
     set_eff_smem_limits();
     sep_set_limits();
     {
@@ -830,13 +842,21 @@ static int fresh_gt(sldqmc_ctx *c, const int8_t *d_s, int B, int tau1, double *d
     double *Gt = c->d_G[0] + 2 * (size_t)c->cap * nn;  // G(tau1) staging
     double *T = Gt + (size_t)c->cap * nn;
     double *dst[2] = {dstp, dstm};
+    const bool oz = oz_have_e(c);
     for (int f = 0; f < 2; ++f) {
-        int rc = weight_run(c, d_s, B, f == 0 ? 1 : -1, tau1 % c->M, c->d_ld_tmp2, nullptr, Gt, 1.0, 0);
+        // the tensor-core form transforms both flavours in one launch from dst itself
+        int rc = weight_run(c, d_s, B, f == 0 ? 1 : -1, tau1 % c->M, c->d_ld_tmp2, nullptr, oz ? dst[f] : Gt, 1.0, 0);
         if (rc) return rc;
+        if (oz) continue;
         GemmF64 g = gemm_desc(N, N, N, c->d_Einv, N, 0, Gt, N, nn, T, N, nn, B);
         gemm_ctx(c, g, false, false);
         GemmF64 h = gemm_desc(N, N, N, T, N, nn, c->d_E, N, 0, dst[f], N, nn, B);
         gemm_ctx(c, h, false, false);
+    }
+    if (oz) {
+        double *Tt[2] = {Gt, T};
+        const double *src[2] = {dstp, dstm};
+        oz_similarity(c, src, Tt, dst, 1, nullptr, nullptr, B);
     }
     return SLDQMC_OK;
 }
@@ -849,6 +869,11 @@ static void wrap_gt(sldqmc_ctx *c, const int8_t *d_s, int B, int tau, double *sr
     const long long nn = c->nn;
     double *T = c->d_G[0] + 3 * (size_t)c->cap * nn;
     double *src[2] = {srcp, srcm}, *dst[2] = {dstp, dstm};
+    if (oz_have_e(c)) {
+        double *Tt[2] = {T - (size_t)c->cap * nn, T};
+        oz_similarity(c, src, Tt, dst, 0, d_s + (long long)tau * N, c->ex_scale, B);
+        return;
+    }
     for (int f = 0; f < 2; ++f) {
         const double cu = c->ex_scale[f][0], cd = c->ex_scale[f][1];
         GemmF64 g = gemm_desc(N, N, N, src[f], N, nn, c->d_Einv, N, 0, T, N, nn, B);
@@ -873,6 +898,7 @@ int sldqmc_local_sweep_batch_dev(sldqmc_ctx *c, int8_t *d_s, int B, uint64_t see
     if (c->N > 5120 && c->local_rank <= 1) return SLDQMC_ERR_UNSUPPORTED;
     int rc = ensure_local_buffers(c);
     if (rc) return rc;
+    oz_have_e(c);  // allocates on first use, as the buffers above
     const long long V = (long long)c->N * c->M;
     launch_check_field(c, d_s, V * B);
     const long long nn = c->nn;
@@ -1317,7 +1343,7 @@ int sldqmc_gram_batch_dev(sldqmc_ctx *c, const double *d_X, int B, double *d_W)
 {
     if (!c || !d_X || !d_W || B < 1 || B > c->cap) return SLDQMC_ERR_ARG;
     const int N = c->N;
-    if (c->oz_ws) {
+    if (c->oz_ws && c->p.prec != SLDQMC_FP64) {
         oz_gram(c, d_X, c->nn, d_W, c->nn, N, B);
     } else {
         GemmF64 g = gemm_desc(N, N, N, d_X, N, c->nn, d_X, N, c->nn, d_W, N, c->nn, B);

@@ -860,7 +860,7 @@ static void chol_pass(sldqmc_ctx *c, double *W, long long sW, double *Y, double 
     const int N = c->N;
     const long long nn = c->nn;
     cudaMemsetAsync(R, 0, sizeof(double) * nn * B, c->st);
-    // Tensor-core path (mixed modes): left-looking, the panel's rows of W and
+    // Tensor-core path (N >= 128): left-looking, the panel's rows of W and
     // Y are brought up to date just before the panel, the panel's rows of R
     // and Q^T are its rows of W and Y multiplied by the inverse of the
     // diagonal block's factor (all FP64-accurate digit splitting), and that
@@ -971,7 +971,7 @@ void stabilize(sldqmc_ctx *c, double *Xt, double *Wc, double *Y, int B, int pass
     prof_end(c);
     c->launches++;
     if (c->oz_ws) {
-        // mixed-precision modes: V = (D^{-1} R D_p) P^T V, FP64-accurate on the tensor cores
+        // V = (D^{-1} R D_p) P^T V, FP64-accurate on the tensor cores
         oz_update_V(c, R, V, Vg, B);
         return;
     }
@@ -1034,8 +1034,8 @@ void finalize(sldqmc_ctx *c, const double *Ut, int B, double *d_ld, int *d_sign,
             prof_end(c);
             c->launches++;
             int m2 = N - (k0 + kb);
-            if (m2 > 0 && c->oz_ws && !rhs) {
-                oz_lu_update(c, A, sItem, lda, k0, kb, B);
+            if (m2 > 0 && c->oz_ws) {
+                oz_lu_update(c, A, sItem, lda, k0, kb, B, rhs);
             } else if (m2 > 0) {
                 GemmF64 g = gemm_desc(m2, rest, kb, A + (long long)(k0 + kb) * lda + k0, lda, sItem,
                                       A + (long long)k0 * lda + k0 + kb, lda, sItem,
@@ -1055,7 +1055,9 @@ void finalize(sldqmc_ctx *c, const double *Ut, int B, double *d_ld, int *d_sign,
             k_trsm_upper_rhs<32><<<gt, 128, 0, c->st>>>(A, sItem, lda, N, k0, kb);
             prof_end(c);
             c->launches++;
-            if (k0 > 0) {
+            if (k0 > 0 && c->oz_ws) {
+                oz_back_update(c, A, sItem, lda, k0, kb, B);
+            } else if (k0 > 0) {
                 GemmF64 g = gemm_desc(k0, N, kb, A + k0, lda, sItem, A + (long long)k0 * lda + N, lda,
                                       sItem, A + N, lda, sItem, B);
                 g.alpha = -1.0; g.beta = 1.0;
