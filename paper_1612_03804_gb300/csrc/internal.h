@@ -12,6 +12,8 @@ struct sldqmc_ctx;
 
 namespace sldqmc {
 
+struct FlipPairs;
+
 // Error bits raised by kernels into the context's device flag word.
 enum : int {
     FLAG_NUMERICAL = 1,  // non-positive Cholesky pivot, zero LU pivot or non-finite value
@@ -85,7 +87,7 @@ void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW,
 // pairs G_f -= U_f V_f of the delayed local update (U: N x 32, V: 32 x N).
 void oz_lu_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B, int rhs);
 void oz_back_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B);
-void oz_delayed_update(sldqmc_ctx *c, double *const *G, const double *const *U, const double *const *V, int B);
+void oz_delayed_update(sldqmc_ctx *c, double *const *G, const FlipPairs *pairs, int B);
 // Products with exp(-+dtau K) on the tensor cores, FP64-accurate.  oz_have_e
 // builds the digit planes of both propagators on first use and says whether
 // they are there; oz_slice_product: Xt = X diag(d) E (d from the field slice
@@ -111,6 +113,15 @@ bool sep_supported(int Lx, int Ly);
 void sep_set_limits();
 void sep_chain_block(sldqmc_ctx *c, const double *Ut, const int8_t *d_s, int B, double cu, double cd, int t0,
                      int nb, const double *ring, double *Xt_out);
+
+// The accepted flips of one block of up to 32 sites of a slice, one record
+// per chain: the sites in order, and per flavour what is needed to form the
+// pairs u_n, v_n (G <- G - sum_n u_n v_n) at every row and column:
+//   L[n][m] = u_m at site n,  X[m][n] = v_m at site n  (m < n),  coef[n] = Delta_n / R_n.
+struct FlipPairs {
+    double L[2][32][32], X[2][32][32], coef[2][32];
+    int site[32], n;
+};
 
 // Event-bracketed timing of launches (sldqmc_profile_*).
 struct ProfRec {

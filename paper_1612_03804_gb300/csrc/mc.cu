@@ -322,6 +322,155 @@ __global__ void __launch_bounds__(512) k_local_flips_delayed(DelayArgs d)
     }
 }
 
+// The decisions of one block on lattices of 128 sites and more.  They depend
+// on the Green's functions only through the 32 x 32 blocks of rows and columns
+// i0..i0+ns-1, so the block's serial chain runs on those alone, in shared
+// memory, and what the accepted flips do to the other rows and columns is
+// formed afterwards on all SMs (k_flip_pairs and a rank-32 product,
+// oz_gram.cu).  One CTA per chain.  Warp 0 walks the sites up to the next
+// accepted one; then all warps subtract its pair from the rows still to
+// come.  The chain is bound by the latency of dependent FP64 operations, of
+// which the two logarithms of a decision were most: the decision is taken in
+// FP32 where it is clear by a thousandth (its rounding is below 1e-5 of the
+// terms), and otherwise, and near the margin, by the FP64 expression.
+// A block of 32 sites of 8 chains at N = 576: 29 us, and 29 us for the pairs;
+// 247 us when every pair was formed for all rows and columns inside the chain,
+// and 651 us per 32 sites of 16 chains at N = 256 with immediate updates on one
+// SM per chain (2 N^2 FMAs of the FP64 pipe per accepted flip and flavour).
+__global__ void __launch_bounds__(256) k_flip_block(LocalArgs a, FlipPairs *out, int i0, int ns)
+{
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int N = a.Lx * a.Ly, tau = a.tau;
+    __shared__ double g[2][32][33], us[2][32][33], vs[2][32][33];
+    __shared__ double coef[2][32], dls[2][2], lus[32];
+    __shared__ int s_q, sites[32];
+    const uint64_t seed = a.seed + ((uint64_t)b << 32);
+    int8_t *s = a.s + (long long)b * a.M * N;
+    FlipPairs &o = out[b];
+    for (int e = tid; e < 2 * 32 * 32; e += 256) {
+        const int f = e >> 10, r = (e >> 5) & 31, c = e & 31;
+        const double *G = (f ? a.Gm : a.Gp) + (long long)b * a.nn;
+        g[f][r][c] = (r < ns && c < ns) ? G[(long long)(i0 + r) * N + i0 + c] : 0.0;
+    }
+    // warp 0, lane j: spin and neighbour sums of site i0 + j
+    int sold = 1, nsp = 0, ntm = 0, x = 0, y = 0;
+    if (wid == 0) {
+        if (lane < ns) {
+            const int i = i0 + lane;
+            x = i % a.Lx;
+            y = i / a.Lx;
+            sold = s[tau * N + i];
+            if (a.Lx > 1) nsp += s[tau * N + wrapi(x + 1, a.Lx) + a.Lx * y] + s[tau * N + wrapi(x - 1, a.Lx) + a.Lx * y];
+            if (a.Ly > 1) nsp += s[tau * N + x + a.Lx * wrapi(y + 1, a.Ly)] + s[tau * N + x + a.Lx * wrapi(y - 1, a.Ly)];
+            ntm = s[wrapi(tau + 1, a.M) * N + i] + s[wrapi(tau - 1, a.M) * N + i];
+            lus[lane] = log(philox_uniform(seed, (uint32_t)i, (uint32_t)tau, a.sweep, PURPOSE_LOCAL));
+        }
+    } else if (wid == 1 && lane < 4) {
+        const int f = lane >> 1, sp = lane & 1;
+        dls[f][sp] = exp(-2.0 * (f == 0 ? 1.0 : -1.0) * a.dtxi * (sp ? 1.0 : -1.0)) - 1.0;
+    }
+    __syncthreads();
+    long long n_mg = 0;
+    int q = 0, n = 0;
+    for (;;) {
+        if (wid == 0) {
+            int hit = ns;
+            for (; q < ns; ++q) {
+                const int f = lane & 1;  // flavour f on the lanes of its parity
+                const int so = __shfl_sync(0xffffffffu, sold, q);
+                const int np = __shfl_sync(0xffffffffu, nsp, q), nt = __shfl_sync(0xffffffffu, ntm, q);
+                const double Dl = dls[f][so > 0];
+                const double R = __dadd_rn(1.0, __dmul_rn(Dl, __dadd_rn(1.0, -g[f][q][q])));
+                const double lu = lus[q];
+                const float Rf = fabsf((float)R), luf = (float)lu;
+                const float lr = 2.0f * logf(Rf);
+                const float st = -2.0f * (float)so * ((float)a.dtauJ * (float)np + (float)a.Kt * (float)nt);
+                const float lro = __shfl_xor_sync(0xffffffffu, lr, 1);
+                const float d = st + lr + lro - luf;
+                bool clear = fabsf(d) > 1e-3f + 1e-5f * (fabsf(st) + fabsf(lr) + fabsf(lro) + fabsf(luf)) &&
+                             Rf > 1e-30f && Rf < 1e30f;
+                clear = __all_sync(0xffffffffu, clear);
+                bool acc = d > 0.0f;
+                if (!clear) {
+                    const double lR = log(fabs(R)), lRo = __shfl_xor_sync(0xffffffffu, lR, 1);
+                    double logr = __dmul_rn(-2.0 * (double)so,
+                                            __dadd_rn(__dmul_rn(a.dtauJ, (double)np), __dmul_rn(a.Kt, (double)nt)));
+                    logr = __dadd_rn(logr, __dmul_rn(2.0, f ? lRo : lR));
+                    logr = __dadd_rn(logr, __dmul_rn(2.0, f ? lR : lRo));
+                    if (fabs(logr - lu) <= MARGIN) n_mg++;
+                    acc = lu < logr;
+                }
+                if (acc) {
+                    if (lane < 2) coef[f][n] = Dl / R;
+                    hit = q;
+                    break;
+                }
+            }
+            if (lane == 0) {
+                s_q = hit;
+                if (hit < ns) sites[n] = hit;
+            }
+            if (hit < ns) {
+                // the flipped spin, and the sums of its neighbours in the block
+                const int so = __shfl_sync(0xffffffffu, sold, hit);
+                const int xq = __shfl_sync(0xffffffffu, x, hit), yq = __shfl_sync(0xffffffffu, y, hit);
+                int mult = 0;
+                if (a.Lx > 1 && y == yq) mult += (wrapi(x + 1, a.Lx) == xq) + (wrapi(x - 1, a.Lx) == xq);
+                if (a.Ly > 1 && x == xq) mult += (wrapi(y + 1, a.Ly) == yq) + (wrapi(y - 1, a.Ly) == yq);
+                nsp -= 2 * so * mult;
+                if (lane == hit) sold = -so;
+                q = hit + 1;
+            }
+        }
+        __syncthreads();
+        const int hit = s_q;
+        if (hit >= ns) break;
+        if (tid < 64) {
+            const int f = wid;
+            us[f][n][lane] = coef[f][n] * g[f][lane][hit];
+            vs[f][n][lane] = (lane == hit ? 1.0 : 0.0) - g[f][hit][lane];
+        }
+        __syncthreads();
+        {
+            const int f = wid >> 2;
+            const double v = vs[f][n][lane];
+            for (int r = hit + 1 + (wid & 3); r < ns; r += 4) g[f][r][lane] -= us[f][n][r] * v;
+        }
+        ++n;
+        __syncthreads();
+    }
+    for (int e = tid; e < 2 * 32 * 32; e += 256) {
+        const int f = e >> 10, r = (e >> 5) & 31, c = e & 31;
+        // L[r][c] = u_c at accepted site r, X[r][c] = v_r at accepted site c
+        o.L[f][r][c] = c < r && r < n ? us[f][c][sites[r]] : 0.0;
+        o.X[f][r][c] = r < c && c < n ? vs[f][r][sites[c]] : 0.0;
+    }
+    if (tid < 64) o.coef[wid][lane] = lane < n ? coef[wid][lane] : 0.0;
+    if (tid < 32) o.site[tid] = tid < n ? i0 + sites[tid] : 0;
+    if (wid == 0) {
+        if (lane < ns) s[tau * N + i0 + lane] = (int8_t)sold;
+        if (lane == 0) {
+            o.n = n;
+            a.stats[b * 4 + 0] += n;
+            a.stats[b * 4 + 1] += ns;
+            a.stats[b * 4 + 2] += n_mg;
+        }
+    }
+}
+
+void launch_flip_block(sldqmc_ctx *c, double *Gp, double *Gm, FlipPairs *out, int8_t *d_s, int B, int tau, int i0, int ns,
+                       uint32_t sweep, uint64_t seed, long long *stats)
+{
+    LocalArgs a;
+    a.Gp = Gp; a.Gm = Gm; a.nn = c->nn; a.s = d_s;
+    a.Lx = c->p.Lx; a.Ly = c->p.Ly; a.M = c->M; a.tau = tau; a.sweep = sweep; a.seed = seed;
+    a.dtxi = c->p.dtau * c->p.xi; a.dtauJ = c->dtauJ; a.Kt = c->Ktau; a.stats = stats;
+    prof_begin(c, SLDQMC_KC_LOCAL, 0.0, "flip_block");
+    k_flip_block<<<B, 256, 0, c->st>>>(a, out, i0, ns);
+    prof_end(c);
+    c->launches++;
+}
+
 void launch_local_flips_delayed(sldqmc_ctx *c, double *Gp, double *Gm, double *U, double *V, int8_t *d_s, int B,
                                 int tau, int i0, int ns, uint32_t sweep, uint64_t seed, long long *stats)
 {

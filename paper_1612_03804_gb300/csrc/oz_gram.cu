@@ -1194,30 +1194,27 @@ void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW,
 
 namespace {
 
-// Rank-32 updates C[i][j] -= sum_l L[i][l] R[l][j] of up to two matrices or
-// column ranges, FP64-accurate on the tensor cores: the rows of L (rows x
+// Rank-32 updates C[i][j] -= sum_l L[i][l] R[l][j] of up to two column ranges
+// (L, R and C in one matrix of row stride lda, item stride sA), FP64-accurate on the tensor cores: the rows of L (rows x
 // kb, row stride ldl) and the columns of R each split with their own maximum
 // (K = kb <= 32, one exactly accumulated chunk).  The product is computed
 // with rows j and columns i and stored transposed, so that a warp's 32 reads
 // and writes of C are contiguous.
 struct RankPart {
-    const double *L;  // null: the first part's
     const double *R;  // kb x cols, columns j0 .. j0 + cols - 1 of a matrix whose row 0 starts at R
     int j0, cols;
     double *C;        // element (0, j0)
 };
 
-void oz_rank_update(sldqmc_ctx *c, const RankPart *pt, int nparts, int rows, int kb, long long ldl, long long sL,
-                    long long ldr, long long sR, int ldc, long long sC, int B, const char *site)
+void oz_rank_update(sldqmc_ctx *c, const double *L, const RankPart *pt, int nparts, int rows, int kb, int lda, long long sA,
+                    int B, const char *site)
 {
     OzWs *w = (OzWs *)c->oz_ws;
     const int N = c->N;
-    const bool two_l = nparts > 1 && pt[1].L;
     {
-        OzRows r{{pt[0].L, two_l ? pt[1].L : nullptr}, {w->lplanes[0], w->lplanes[1]}, {w->EL[0], w->EL[1]}, nullptr, 0, 1.0, 1.0};
+        OzRows r{{L, nullptr}, {w->lplanes[0], nullptr}, {w->EL[0], nullptr}, nullptr, 0, 1.0, 1.0};
         prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice");
-        k_oz_slice<false><<<dim3((rows + 7) / 8, B, two_l ? 2 : 1), 256, 0, c->st>>>(r, sL, rows, kb, (int)ldl, N, 32,
-                                                                                   w->lplane_stride);
+        k_oz_slice<false><<<dim3((rows + 7) / 8, B), 256, 0, c->st>>>(r, sA, rows, kb, lda, N, 32, w->lplane_stride);
         prof_end(c);
     }
     OzPanelSlice sl{};
@@ -1227,17 +1224,17 @@ void oz_rank_update(sldqmc_ctx *c, const RankPart *pt, int nparts, int rows, int
     int *ep[2] = {w->EPW, w->EPY};
     for (int p = 0; p < nparts; ++p) {
         sl.src[p] = pt[p].R;
-        sl.sS[p] = sR;
+        sl.sS[p] = sA;
         sl.j0[p] = pt[p].j0;
         sl.planes[p] = pl[p];
         sl.E[p] = ep[p];
-        a.pt[p] = oz_part(pt[p].cols, pt[p].j0, ep[p] + pt[p].j0, N, w->EL[p && two_l], N, pt[p].C, sC, ldc);
+        a.pt[p] = oz_part(pt[p].cols, pt[p].j0, ep[p] + pt[p].j0, N, w->EL[0], N, pt[p].C, sA, lda);
         cols += pt[p].cols;
     }
     const int nb0 = (pt[0].cols + 31) / 32, nb1 = nparts > 1 ? (pt[1].cols + 31) / 32 : 0;
     sl.nb0 = nb0;
     prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice_panel");
-    k_oz_slice_panel<<<dim3(nb0 + nb1, B), 256, 0, c->st>>>(sl, N, (int)ldr, kb, 0, w->plane_stride, w->ldp, c->d_flag);
+    k_oz_slice_panel<<<dim3(nb0 + nb1, B), 256, 0, c->st>>>(sl, N, lda, kb, 0, w->plane_stride, w->ldp, c->d_flag);
     prof_end(c);
     a.nparts = nparts;
     a.Nn = rows;
@@ -1246,7 +1243,7 @@ void oz_rank_update(sldqmc_ctx *c, const RankPart *pt, int nparts, int rows, int
     a.flag = c->d_flag;
     prof_begin(c, SLDQMC_KC_GEMM_OZ, 2.0 * rows * cols * kb * B, site);
     k_oz_gemm<false, true, true><<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(
-        w->mapRA, w->mapA, w->mapL[0], w->mapL[two_l], a);
+        w->mapRA, w->mapA, w->mapL[0], w->mapL[0], a);
     prof_end(c);
     c->launches += 3;
 }
@@ -1293,9 +1290,9 @@ void oz_lu_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int k
 {
     const int N = c->N, j0 = k0 + kb;
     double *low = A + (long long)j0 * lda;  // row k0 + kb
-    const RankPart pt[2] = {{low + k0, A + (long long)k0 * lda, j0, N - j0, low + j0},
-                            {nullptr, A + (long long)k0 * lda + N, 0, N, low + N}};
-    oz_rank_update(c, pt, rhs ? 2 : 1, N - j0, kb, lda, sA, lda, sA, lda, sA, B, "oz_lu_update");
+    const RankPart pt[2] = {{A + (long long)k0 * lda, j0, N - j0, low + j0},
+                            {A + (long long)k0 * lda + N, 0, N, low + N}};
+    oz_rank_update(c, low + k0, pt, rhs ? 2 : 1, N - j0, kb, lda, sA, B, "oz_lu_update");
 }
 
 // Back substitution: the rows above k0 of the right-hand side lose the share
@@ -1303,16 +1300,108 @@ void oz_lu_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int k
 void oz_back_update(sldqmc_ctx *c, double *A, long long sA, int lda, int k0, int kb, int B)
 {
     const int N = c->N;
-    const RankPart pt = {A + k0, A + (long long)k0 * lda + N, 0, N, A + N};
-    oz_rank_update(c, &pt, 1, k0, kb, lda, sA, lda, sA, lda, sA, B, "oz_back_update");
+    const RankPart pt = {A + (long long)k0 * lda + N, 0, N, A + N};
+    oz_rank_update(c, A + k0, &pt, 1, k0, kb, lda, sA, B, "oz_back_update");
 }
 
-// The pending rank-32 corrections of the delayed local update, G_f -= U_f V_f.
-void oz_delayed_update(sldqmc_ctx *c, double *const *G, const double *const *U, const double *const *V, int B)
+namespace {
+
+// Forms the pairs of a block of flips at every row and column and splits them
+// for the rank-32 product: blocks of even x the left vectors u_n at 128 rows
+// (thread = row, its 32 values one plane row of lplanes), blocks of odd x the
+// right vectors v_n at 128 columns.  u_n = coef_n (G[:, i_n] - sum_m u_m
+// v_m[i_n]), v_n = e - (G[i_n, :] - sum_m u_m[i_n] v_m): 496 dependent-by-row FMAs
+// per thread on the FP64 pipe, which bound it (17 us per wave; one wave up to
+// 76 x 128 rows of both flavours).
+struct PairArgs {
+    const double *G[2];
+    const FlipPairs *pairs;
+    __nv_bfloat16 *lp[2], *rp[2];
+    int *EL[2], *ER[2];
+    long long lps, rps;
+    int N, ldp;
+};
+
+__global__ void __launch_bounds__(128) k_flip_pairs(PairArgs a)
 {
+    __shared__ double T[32][32], cf[32];
+    __shared__ int site[32];
+    const int b = blockIdx.y, f = blockIdx.z, right = blockIdx.x & 1, tid = threadIdx.x;
+    const FlipPairs &p = a.pairs[b];
+    const int n = p.n, N = a.N;
+    for (int e = tid; e < 32 * 32; e += 128) (&T[0][0])[e] = right ? (&p.L[f][0][0])[e] : (&p.X[f][0][0])[e];
+    if (tid < 32) {
+        cf[tid] = p.coef[f][tid];
+        site[tid] = p.site[tid];
+    }
+    __syncthreads();
+    const int r = (blockIdx.x >> 1) * 128 + tid;
+    if (r >= N) return;
+    const double *G = (f ? a.G[1] : a.G[0]) + (long long)b * N * N;
+    double x[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) x[k] = k < n ? (right ? G[(long long)site[k] * N + r] : G[(long long)r * N + site[k]]) : 0.0;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        if (k < n) {
+            double c = x[k];
+#pragma unroll
+            for (int m = 0; m < k; ++m) c -= x[m] * (right ? T[k][m] : T[m][k]);
+            x[k] = right ? (r == site[k] ? 1.0 : 0.0) - c : cf[k] * c;
+        }
+    }
+    unsigned long long mx = 0;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        const unsigned long long u = (unsigned long long)__double_as_longlong(x[k]) & 0x7FFFFFFFFFFFFFFFull;
+        mx = u > mx ? u : mx;
+    }
+    const int ef_max = (int)(mx >> 52);
+    const int E = oz_exponent(ef_max);
+    const long long row = (long long)b * N + r;
+    (right ? a.ER[f] : a.EL[f])[row] = E;
+    __nv_bfloat16 *dst = right ? a.rp[f] + row * a.ldp : a.lp[f] + row * 32;
+    const long long ps = right ? a.rps : a.lps;
+#pragma unroll
+    for (int k8 = 0; k8 < 32; k8 += 8) {
+        int dg[8][OZ_S];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) oz_digits(x[k8 + k], E, ef_max, dg[k]);
+#pragma unroll
+        for (int q = 0; q < OZ_S; ++q) {
+            __nv_bfloat162 h2[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) h2[k] = __floats2bfloat162_rn((float)dg[2 * k][q], (float)dg[2 * k + 1][q]);
+            *reinterpret_cast<uint4 *>(dst + q * ps + k8) = *reinterpret_cast<const uint4 *>(h2);
+        }
+    }
+}
+
+}  // namespace
+
+// G_f -= sum_n u_n v_n of both flavours for one block of flips.
+void oz_delayed_update(sldqmc_ctx *c, double *const *G, const FlipPairs *pairs, int B)
+{
+    OzWs *w = (OzWs *)c->oz_ws;
     const int N = c->N;
-    const RankPart pt[2] = {{U[0], V[0], 0, N, G[0]}, {U[1], V[1], 0, N, G[1]}};
-    oz_rank_update(c, pt, 2, N, 32, 32, 32LL * N, N, 32LL * N, N, c->nn, B, "oz_delayed_update");
+    PairArgs p{{G[0], G[1]}, pairs, {w->lplanes[0], w->lplanes[1]}, {w->rplanes, w->planes}, {w->EL[0], w->EL[1]},
+               {w->EPW, w->EPY}, w->lplane_stride, w->plane_stride, N, w->ldp};
+    prof_begin(c, SLDQMC_KC_LOCAL, 0.0, "flip_pairs");
+    k_flip_pairs<<<dim3(2 * ((N + 127) / 128), B, 2), 128, 0, c->st>>>(p);
+    prof_end(c);
+    OzArgs a{};
+    a.pt[0] = oz_part(N, 0, w->EPW, N, w->EL[0], N, G[0], c->nn, N);
+    a.pt[1] = oz_part(N, 0, w->EPY, N, w->EL[1], N, G[1], c->nn, N);
+    a.nparts = 2;
+    a.Nn = N;
+    a.batch = B;
+    a.nk = 1;
+    a.flag = c->d_flag;
+    prof_begin(c, SLDQMC_KC_GEMM_OZ, 2.0 * 2.0 * N * N * 32 * B, "oz_delayed_update");
+    k_oz_gemm<false, true, true><<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(
+        w->mapRA, w->mapA, w->mapL[0], w->mapL[1], a);
+    prof_end(c);
+    c->launches += 2;
 }
 
 bool oz_have_e(sldqmc_ctx *c) { return c->oz_ws && oz_e_planes(c); }

@@ -28,6 +28,8 @@ void launch_local_flips(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s, int 
 void launch_drift(sldqmc_ctx *c, const double *Gw, const double *Gf, int B2x, int B, long long *stats);
 void launch_local_flips_delayed(sldqmc_ctx *c, double *Gp, double *Gm, double *U, double *V, int8_t *d_s, int B,
                                 int tau, int i0, int ns, uint32_t sweep, uint64_t seed, long long *stats);
+void launch_flip_block(sldqmc_ctx *c, double *Gp, double *Gm, FlipPairs *out, int8_t *d_s, int B, int tau, int i0, int ns,
+                       uint32_t sweep, uint64_t seed, long long *stats);
 void launch_eff_sweeps(sldqmc_ctx *c, int8_t *d_s, int B, int n_sweeps, uint64_t seed, uint32_t step,
                        int dir, long long *n_accept, long long *n_margin);
 void launch_features(sldqmc_ctx *c, const int8_t *d_s, int B, long long *out);
@@ -364,29 +366,35 @@ int ensure_local_buffers(sldqmc_ctx *c)
     return SLDQMC_OK;
 }
 
-// The flips of slice tau: one launch of immediate rank-1 updates, or blocks
-// of local_rank sites whose pending corrections G -= U V are applied by one
-// batched GEMM per flavour after each block.
+// The flips of slice tau.  From 128 sites on, blocks of 32 sites whatever
+// local_rank says: the decisions on the block's own rows and columns, then the
+// rank-32 correction of both flavours on the tensor cores.  Below: one launch
+// of immediate rank-1 updates, or blocks of local_rank sites whose pending
+// corrections G -= U V are applied by one batched GEMM per flavour after each
+// block.
 static void local_flips_slice(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s, int B, int tau, uint32_t sweep,
                               uint64_t seed)
 {
     const int N = c->N;
+    double *G[2] = {Gp, Gm};
+    if (c->oz_ws) {
+        static_assert(sizeof(FlipPairs) <= 2 * 32 * 128 * sizeof(double), "a record fits a chain's share of d_U");
+        FlipPairs *pairs = reinterpret_cast<FlipPairs *>(c->d_U);
+        for (int i0 = 0; i0 < N; i0 += 32) {
+            launch_flip_block(c, Gp, Gm, pairs, d_s, B, tau, i0, std::min(32, N - i0), sweep, seed, c->d_stats);
+            oz_delayed_update(c, G, pairs, B);
+        }
+        return;
+    }
     if (c->local_rank <= 1) {
         launch_local_flips(c, Gp, Gm, d_s, B, tau, sweep, seed, c->d_stats);
         return;
     }
-    double *G[2] = {Gp, Gm};
     for (int i0 = 0; i0 < N; i0 += c->local_rank) {
         const int ns = std::min(c->local_rank, N - i0);
         launch_local_flips_delayed(c, Gp, Gm, c->d_U, c->d_V, d_s, B, tau, i0, ns, sweep, seed, c->d_stats);
-        const long long so1 = (long long)c->cap * 32 * N;
-        if (c->oz_ws) {
-            const double *U[2] = {c->d_U, c->d_U + so1}, *V[2] = {c->d_V, c->d_V + so1};
-            oz_delayed_update(c, G, U, V, B);
-            continue;
-        }
         for (int f = 0; f < 2; ++f) {
-            const long long so = f * so1;
+            const long long so = (long long)f * c->cap * 32 * N;
             GemmF64 g = gemm_desc(N, N, 32, c->d_U + so, 32, 32LL * N, c->d_V + so, N, 32LL * N, G[f], N, c->nn, B);
             g.alpha = -1.0;
             g.beta = 1.0;
