@@ -32,8 +32,8 @@
 // of a group is an integer of magnitude <= K 2^16 (the leading group; K (2^15 +
 // 6 * 4096) the others) <= 2^24 for K <= 256, so the tensor-core accumulation
 // is exact.  Longer contractions run in chunks of at most 256: the epilogue converts each chunk's eight
-// group sums to integers, combines them in two 64-bit integers, forms the
-// chunk's FP64 value with one rounding and adds the chunks in FP64.
+// group sums to integers and adds them, shifted, to two 64-bit integers, which
+// hold the whole sum exactly (|h| <= K 2^37) and are rounded to FP64 once.
 //
 // One persistent CTA per SM walks the 128 x 32 output tiles of every item
 // (for a Gram matrix only those on or above the diagonal; a launch may carry
@@ -493,16 +493,60 @@ struct OzPart {
     int srow0;
 };
 
-// x 2^e, exact: through the exponent field while the result stays normal
-// (integer arithmetic, off the FP64 pipe), otherwise scalbn; NaN for the
-// exponent of a row that holds an infinity or a NaN (its digits are zero).
-__device__ __forceinline__ double oz_scale2(double x, int e)
+// h 2^e + l 2^(e-28), rounded once to nearest even.  FP64: two conversions and
+// an FMA (a warp's FP64 instruction holds its sub-partition's pipe for 64
+// cycles), the scale through the exponent field while the result stays normal.
+// NaN for the exponent of a row that holds an infinity or a NaN (its digits
+// are zero).
+__device__ __forceinline__ double oz_round_fp(long long h, long long l, int e)
 {
+    const double x = fma((double)l, 0x1p-28, (double)h);
     const long long bits = __double_as_longlong(x);
     const int ex = (int)((bits >> 52) & 0x7FF);
     if (ex != 0 && ex + e > 0 && ex + e < 2047) return __longlong_as_double(bits + ((long long)e << 52));
     if (e > OZ_NONFINITE / 2) return __longlong_as_double(0x7FF8000000000000ll);
     return scalbn(x, e);
+}
+
+// The same by integer operations, for the updates: their subtraction takes the
+// FP64 pipe as well, and with K = 32 there are few MMAs to hide either behind
+// (rank-32 update at N = 576, 16 items: 78 -> 73 us; a Gram matrix at N = 256,
+// 128 items, whose epilogue hides behind its MMAs: 125 -> 128 us, so products
+// without a subtraction keep the form above).
+__device__ __forceinline__ double oz_round(long long h, long long l, int e)
+{
+    // T = h 2^28 + l in three words, then |T|
+    unsigned long long lo = ((unsigned long long)h << 28) + (unsigned long long)l;
+    long long hi = (h >> 36) + (l >> 63) + (lo < (unsigned long long)l ? 1 : 0);
+    const unsigned long long sign = (unsigned long long)hi & 0x8000000000000000ull;
+    if (hi < 0) {
+        lo = 0ull - lo;
+        hi = ~hi + (lo == 0ull ? 1 : 0);
+    }
+    uint32_t t2 = (uint32_t)hi, t1 = (uint32_t)(lo >> 32), t0 = (uint32_t)lo;
+    int ex = e + 95 - 28 + 1023;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (t2 == 0u) {
+            t2 = t1;
+            t1 = t0;
+            t0 = 0u;
+            ex -= 32;
+        }
+    const int s = __clz((int)t2);
+    ex -= s;
+    if (t2 == 0u || (unsigned)(ex - 1) >= 2045u) return oz_round_fp(h, l, e);  // zero, subnormal, too large, NaN
+    const uint32_t a = __funnelshift_l(t1, t2, s), b = __funnelshift_l(t0, t1, s);
+    const uint32_t rem = (b << 21) | ((t0 << s) != 0u ? 1u : 0u);  // the bits below the 53rd
+    unsigned long long m = ((unsigned long long)a << 21) | (b >> 11);
+    m += (rem > 0x80000000u || (rem == 0x80000000u && (m & 1ull))) ? 1ull : 0ull;
+    return __longlong_as_double((long long)(sign | (((unsigned long long)(ex - 1) << 52) + m)));
+}
+
+// acc + v 2^s in one multiply-add
+__device__ __forceinline__ void oz_fold(long long &acc, int v, int s)
+{
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(v), "r"(1 << s));
 }
 
 struct OzArgs {
@@ -766,10 +810,12 @@ __global__ void __launch_bounds__(OTHREADS, 1)
             int ebv[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) ebv[j] = (!SUB && nb + j < a.Nn) ? eb[nb + j] : 0;
-            // sum over K-chunks of the exactly accumulated chunk products
-            double w[16];
+            // The group sums as exact integers, folded as they arrive and added
+            // over the K-chunks (|h| <= K 2^37): groups 0..3 (p + q = 2..5) into h,
+            // 4..7 (6..9) into l, so that sum_g acc_g 2^-(7(g+2)+2) = h 2^-37 + l 2^-65
+            long long h[16], l[16];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) w[j] = 0.0;
+            for (int j = 0; j < 16; ++j) h[j] = l[j] = 0;
             int k_lo, k_hi;
             oz_krange(a, m0, n0, k_lo, k_hi);
             for (int kc0 = k_lo; kc0 < k_hi; kc0 += OZ_KCHUNK, ++cc) {
@@ -778,34 +824,18 @@ __global__ void __launch_bounds__(OTHREADS, 1)
                 fence_after();
                 const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(u * OZ_G * OBN + hc);
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    // group sums as exact integers, folded as they arrive: groups 0..3
-                    // (p + q = 2..5) into h, 4..7 (6..9) into l, so that
-                    // sum_g acc_g 2^-(7(g+2)+2) = h 2^-37 + l 2^-65
-                    long long h[8], l[8];
+                for (int c8 = 0; c8 < 16; c8 += 8) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) h[j] = l[j] = 0;
+                    for (int gg = 0; gg < OZ_G; gg += 4) {
+                        uint32_t r[4][8];
 #pragma unroll
-                    for (int gg = 0; gg < OZ_G; gg += 2) {
-                        uint32_t r0[8], r1[8];
-                        tmem_ld8_nowait(lane_base + (uint32_t)(gg * OBN + half * 8), r0);
-                        tmem_ld8_nowait(lane_base + (uint32_t)((gg + 1) * OBN + half * 8), r1);
-                        tmem_wait_ld8x2(r0, r1);
+                        for (int g = 0; g < 4; ++g) tmem_ld8_nowait(lane_base + (uint32_t)((gg + g) * OBN + c8), r[g]);
+                        tmem_wait_ld8x4(r[0], r[1], r[2], r[3]);
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const long long v0 = (long long)__float2int_rn(__uint_as_float(r0[j]));
-                            const long long v1 = (long long)__float2int_rn(__uint_as_float(r1[j]));
-                            if (gg < 4) h[j] += (v0 << (OZ_BETA * (3 - gg))) + (v1 << (OZ_BETA * (2 - gg)));
-                            else l[j] += (v0 << (OZ_BETA * (7 - gg))) + (v1 << (OZ_BETA * (6 - gg)));
-                        }
-                    }
-                    // the chunk's value (one rounding); the first chunk needs no addition
-                    if (kc0 == k_lo) {
+                        for (int j = 0; j < 8; ++j)
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) w[half * 8 + j] = fma((double)l[j], 0x1p-28, (double)h[j]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) w[half * 8 + j] += fma((double)l[j], 0x1p-28, (double)h[j]);
+                            for (int g = 0; g < 4; ++g)
+                                oz_fold(gg ? l[c8 + j] : h[c8 + j], __float2int_rn(__uint_as_float(r[g][j])), OZ_BETA * (3 - g));
                     }
                 }
                 fence_before();
@@ -821,14 +851,14 @@ __global__ void __launch_bounds__(OTHREADS, 1)
                 const int n = nb + j;
                 double v = 0.0;
                 if (n < a.Nn) {
-                    v = oz_scale2(w[j], Ei + (SUB ? eb[n] : ebv[j]) - 37);
+                    v = SUB ? oz_round(h[j], l[j], Ei + eb[n] - 37) : oz_round_fp(h[j], l[j], Ei + ebv[j] - 37);
                     if (sg) {
                         const bool un = sg[n] > 0;
                         if (un != up) v *= un ? a.r_ud[part] : a.r_du[part];
                     }
                     o[n * cs] = SUB ? cold[j] - v : v;
                 }
-                if (SLICE) w[j] = v;
+                if (SLICE) h[j] = __double_as_longlong(v);
             }
             if (SLICE) {
                 const int srow = (part ? a.pt[1].srow0 : a.pt[0].srow0) + mm;
@@ -847,7 +877,7 @@ __global__ void __launch_bounds__(OTHREADS, 1)
                     int dg[8][OZ_S];
 #pragma unroll
                     for (int jj = 0; jj < 8; ++jj) {
-                        const double x = w[8 * g8 + jj];
+                        const double x = __longlong_as_double(h[8 * g8 + jj]);
                         over |= ((unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull) >= bound;
                         oz_digits(x, E, 1, dg[jj]);
                     }

@@ -117,13 +117,15 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t r[8])
                  : "r"(taddr));
 }
 
-// Waits for outstanding tcgen05.ld and makes two 8-register loads outputs of
+// Waits for outstanding tcgen05.ld and makes four 8-register loads outputs of
 // the wait.
-__device__ __forceinline__ void tmem_wait_ld8x2(uint32_t a[8], uint32_t b[8])
+__device__ __forceinline__ void tmem_wait_ld8x4(uint32_t a[8], uint32_t b[8], uint32_t c[8], uint32_t d[8])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
-                   "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7])
+                   "+r"(b[0]), "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7]),
+                   "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3]), "+r"(c[4]), "+r"(c[5]), "+r"(c[6]), "+r"(c[7]),
+                   "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]), "+r"(d[4]), "+r"(d[5]), "+r"(d[6]), "+r"(d[7])
                  :
                  : "memory");
 }
