@@ -50,6 +50,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "chol32.cuh"
 #include "internal.h"
 #include "tc_common.cuh"
 
@@ -216,9 +217,8 @@ template <bool LOCAL>
 __device__ __forceinline__ void oz_slice_block(int bx, const double *src, long long sS, long long ld, int j0, int Nc,
                                                int krows, int koff, long long plane_stride, int rows_cap, int ldk,
                                                __nv_bfloat16 *planes, int *Ej, long long sE, int *flag,
-                                               const int *rowidx, long long sR)
+                                               const int *rowidx, long long sR, double (*tile)[33])
 {
-    __shared__ double tile[32][33];
     const int b = blockIdx.y, c0 = j0 + bx * 32;
     // blockIdx.z: the 32-row block of the krows source rows (K positions koff + 32 z ..);
     // source row l is rowidx[b * sR + l] when a row index is given
@@ -284,8 +284,9 @@ __global__ void __launch_bounds__(256) k_oz_slice_fixed(const double *src, long 
                                                         int ldk, __nv_bfloat16 *planes, int *Ej, long long sE,
                                                         int *flag, const int *rowidx = nullptr, long long sR = 0)
 {
+    __shared__ double tile[32][33];
     oz_slice_block<false>(blockIdx.x, src, sS, ld, j0, Nc, krows, koff, plane_stride, rows_cap, ldk, planes, Ej, sE,
-                          flag, rowidx, sR);
+                          flag, rowidx, sR, tile);
 }
 
 // The unsolved rows k0..k0+kb of a Cholesky-QR panel in one launch, each
@@ -300,14 +301,20 @@ struct OzPanelSlice {
     int *E[2];
 };
 
+__device__ __forceinline__ void oz_slice_panel(const OzPanelSlice &a, int x, int N, int ld, int kb, int koff,
+                                               long long plane_stride, int ldk, int *flag, double (*tile)[33])
+{
+    const int part = x < a.nb0 ? 0 : 1;
+    oz_slice_block<true>(part ? x - a.nb0 : x, part ? a.src[1] : a.src[0], part ? a.sS[1] : a.sS[0], ld,
+                         part ? a.j0[1] : a.j0[0], N, kb, koff, plane_stride, N, ldk, part ? a.planes[1] : a.planes[0],
+                         part ? a.E[1] : a.E[0], N, flag, nullptr, 0, tile);
+}
+
 __global__ void __launch_bounds__(256) k_oz_slice_panel(OzPanelSlice a, int N, int ld, int kb, int koff,
                                                         long long plane_stride, int ldk, int *flag)
 {
-    const int part = blockIdx.x < a.nb0 ? 0 : 1;
-    const int bx = part ? blockIdx.x - a.nb0 : blockIdx.x;
-    oz_slice_block<true>(bx, part ? a.src[1] : a.src[0], part ? a.sS[1] : a.sS[0], ld, part ? a.j0[1] : a.j0[0], N,
-                         kb, koff, plane_stride, N, ldk, part ? a.planes[1] : a.planes[0], part ? a.E[1] : a.E[0], N,
-                         flag, nullptr, 0);
+    __shared__ double tile[32][33];
+    oz_slice_panel(a, blockIdx.x, N, ld, kb, koff, plane_stride, ldk, flag, tile);
 }
 
 // Bounds for the entries of R's columns in a Cholesky factorisation of the
@@ -368,109 +375,75 @@ __global__ void k_oz_make_T(const double *R, long long nn, int N, const double *
             k >= m ? R[(long long)b * nn + (long long)m * N + k] * Dp[(long long)b * N + k] * rd : 0.0;
 }
 
-// Row j of the diagonal block's factor and of its inverse, finalised by one
-// warp: y = 1/sqrt(d) of the updated pivot d, R_jc = W_jc y (c > j), R_jj =
-// d y, and row j of T scaled by y (it has received its terms l < j).
-__device__ __forceinline__ void oz_chol_finalise_row(double (*Rk)[33], double (*Tm)[33], int j, int lane, int kb,
-                                                     int *flag)
+// What a Cholesky-QR panel needs before its product [R_k,k+ | Q_k^T] = T
+// [W_k,k+ | Y_k] on the tensor cores, in one launch.  Block x = 0 of an item: the
+// factor of the diagonal block, W_kk = R_kk^T R_kk (written to R), and the digit
+// planes of T = R_kk^-T (each row with its own maximum as exponent, ET); the
+// other blocks: the digits of the unsolved rows of Y and W.  Both read only
+// what the previous launch wrote, and the splitting hides behind the factor's
+// chain of pivots.  By events around the launches (32 x 32, 4 items): 34 us for
+// a factor with the library's rsqrt and separate arrays for R and T and 8 us
+// for the splitting; 20.5 us together.
+struct OzPanelPrep {
+    const double *W;
+    long long sW;
+    double *R;
+    long long sR;
+    int N, k0, kb;
+    __nv_bfloat16 *tplanes;
+    long long tps;
+    int *ET;
+};
+
+__global__ void __launch_bounds__(256) k_oz_panel_prep(OzPanelPrep f, OzPanelSlice a, long long plane_stride, int ldk,
+                                                       int *flag)
 {
-    double d = Rk[j][j];
-    if (!(d > 0.0) || !isfinite(d)) {
-        if (lane == 0 && j < kb) atomicOr(flag, FLAG_NUMERICAL);
-        d = 1.0;
+    __shared__ double X[32][33];
+    __shared__ double root[32];
+    if (blockIdx.x > 0) {
+        oz_slice_panel(a, blockIdx.x - 1, f.N, f.N, f.kb, f.k0, plane_stride, ldk, flag, X);
+        return;
     }
-    const double y = rsqrt(d);
-    if (lane > j) Rk[j][lane] *= y;
-    if (lane <= j) Tm[j][lane] *= y;
-    __syncwarp();  // every lane has read the pivot
-    if (lane == j) Rk[j][j] = d * y;
-    __syncwarp();
-}
-
-// Rows r > j of R (upper part c >= r) and of T (finished columns c <= j)
-// lose row j's share: one FMA per warp and row.
-__device__ __forceinline__ void oz_chol_update_row(double (*Rk)[33], double (*Tm)[33], int j, int r, int lane)
-{
-    const double rjr = Rk[j][r];
-    if (lane >= r) Rk[r][lane] -= rjr * Rk[j][lane];
-    else if (lane <= j) Tm[r][lane] -= rjr * Tm[j][lane];
-}
-
-// Cholesky factor of a panel's diagonal block, W_kk = R_kk^T R_kk (R_kk
-// upper triangular, written to R), and the digit planes of T = R_kk^-T
-// (lower triangular; each row with its own maximum as exponent, ET) for the
-// panel's product [R_k,k+ | Q_k^T] = T [W_k,k+ | Y_k] on the tensor cores.
-// One CTA of 128 threads per item; rows and columns kb..31 of R_kk are the
-// identity.  Right-looking: once row j of R and of T is final (T by forward
-// substitution of R_kk^T T = I), every later row loses row j's share.  Warp 0
-// updates row j + 1 first and finalises it (the chain of pivots: update,
-// rsqrt, scale) while warps 1..3 update the rows below, so each step costs one
-// barrier and the pivot chain overlaps the other rows' updates.  Every FP64
-// instruction occupies the pipe for a whole warp, so the work is grouped by
-// rows.
-__global__ void __launch_bounds__(128) k_oz_chol_factor(const double *W, long long sW, int ldw, double *R, long long sR,
-                                                        int N, int k0, int kb, __nv_bfloat16 *tplanes, long long tps,
-                                                        int *ET, int *flag)
-{
-    __shared__ double Rk[32][33];
-    __shared__ double Tm[32][33];
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const double *Wb = W + (long long)b * sW;
-    for (int e = tid; e < 32 * 32; e += blockDim.x) {
+    const int b = blockIdx.y, tid = threadIdx.x, kb = f.kb;
+    const double *Wb = f.W + (long long)b * f.sW + (long long)f.k0 * f.N + f.k0;
+    for (int e = tid; e < 32 * 32; e += 256) {
         const int r = e >> 5, c = e & 31;
-        double v = 0.0;
-        if (r < kb && c < kb) {
-            if (c >= r) v = Wb[(long long)(k0 + r) * ldw + k0 + c];
-        } else if (r == c) {
-            v = 1.0;
-        }
-        Rk[r][c] = v;
-        Tm[r][c] = r == c ? 1.0 : 0.0;
+        X[r][c] = r < kb && c < kb ? (c >= r ? Wb[(long long)r * f.N + c] : 0.0) : (r == c ? 1.0 : 0.0);
     }
     __syncthreads();
-    if (wid == 0) oz_chol_finalise_row(Rk, Tm, 0, lane, kb, flag);
-    __syncthreads();
-    for (int j = 0; j < 31; ++j) {
-        if (wid == 0) {
-            oz_chol_update_row(Rk, Tm, j, j + 1, lane);
-            __syncwarp();
-            oz_chol_finalise_row(Rk, Tm, j + 1, lane, kb, flag);
-        } else {
-            for (int r = j + 1 + wid; r < 32; r += 3) oz_chol_update_row(Rk, Tm, j, r, lane);
-        }
-        __syncthreads();
+    chol32(X, root, kb, flag);
+    double *Rb = f.R + (long long)b * f.sR + (long long)f.k0 * f.N + f.k0;
+    for (int e = tid; e < 32 * 32; e += 256) {
+        const int r = e >> 5, c = e & 31;
+        if (r < kb && c < kb) Rb[(long long)r * f.N + c] = c > r ? X[r][c] : (c == r ? root[r] : 0.0);
     }
-    double *Rb = R + (long long)b * sR;
-    for (int e = tid; e < kb * kb; e += blockDim.x) {
-        const int r = e / kb, c = e % kb;
-        Rb[(long long)(k0 + r) * N + k0 + c] = c >= r ? Rk[r][c] : 0.0;
-    }
-    // digits of T's rows: four threads per row, eight K positions each
-    const int r = tid >> 2, q = tid & 3;
+    // digits of T's rows: eight threads per row, four K positions each
+    const int r = tid >> 3, q = tid & 7;
+    double tv[4];
     unsigned long long mx = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const unsigned long long u = (unsigned long long)__double_as_longlong(Tm[r][8 * q + i]) & 0x7FFFFFFFFFFFFFFFull;
+    for (int i = 0; i < 4; ++i) {
+        tv[i] = 4 * q + i <= r ? X[r][4 * q + i] : 0.0;
+        const unsigned long long u = (unsigned long long)__double_as_longlong(tv[i]) & 0x7FFFFFFFFFFFFFFFull;
         mx = u > mx ? u : mx;
     }
 #pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
+    for (int o = 1; o < 8; o <<= 1) {
         const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
         mx = v > mx ? v : mx;
     }
     const int ef_max = (int)(mx >> 52);
-    const int E = ef_max > 0 ? ef_max - 1022 : 0;
-    if (q == 0) ET[b * 32 + r] = E;
-    int dg[8][OZ_S];
+    const int E = oz_exponent(ef_max);
+    if (q == 0) f.ET[b * 32 + r] = E;
+    int dg[4][OZ_S];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) oz_digits(Tm[r][8 * q + i], E, ef_max, dg[i]);
-    const long long row = ((long long)b * 32 + r) * 32 + 8 * q;
+    for (int i = 0; i < 4; ++i) oz_digits(tv[i], E, ef_max, dg[i]);
+    const long long row = ((long long)b * 32 + r) * 32 + 4 * q;
 #pragma unroll
     for (int p = 0; p < OZ_S; ++p) {
-        __nv_bfloat162 h2[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) h2[i] = __floats2bfloat162_rn((float)dg[2 * i][p], (float)dg[2 * i + 1][p]);
-        *reinterpret_cast<uint4 *>(tplanes + (long long)p * tps + row) = *reinterpret_cast<const uint4 *>(h2);
+        __nv_bfloat162 h2[2] = {__floats2bfloat162_rn((float)dg[0][p], (float)dg[1][p]),
+                                __floats2bfloat162_rn((float)dg[2][p], (float)dg[3][p])};
+        *reinterpret_cast<uint2 *>(f.tplanes + (long long)p * f.tps + row) = *reinterpret_cast<const uint2 *>(h2);
     }
 }
 
@@ -1184,13 +1157,9 @@ void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW,
     sl.j0[1] = j0;
     sl.planes[1] = w->rplanes;
     sl.E[1] = w->EPW;
-    prof_begin(c, SLDQMC_KC_OTHER, 0.0, "k_oz_slice_panel");
-    k_oz_slice_panel<<<dim3(sl.nb0 + (nW + 31) / 32, B), 256, 0, c->st>>>(sl, N, N, kb, k0, w->plane_stride,
-                                                                           w->ldp, c->d_flag);
-    prof_end(c);
-    prof_begin(c, SLDQMC_KC_PANEL_F64, (double)B * 2.0 * kb * kb * kb / 3.0, "oz_chol_factor");
-    k_oz_chol_factor<<<B, 128, 0, c->st>>>(W, sW, N, R, c->nn, N, k0, kb, w->tplanes, w->tplane_stride, w->ET,
-                                           c->d_flag);
+    const OzPanelPrep f{W, sW, R, c->nn, N, k0, kb, w->tplanes, w->tplane_stride, w->ET};
+    prof_begin(c, SLDQMC_KC_PANEL_F64, (double)B * 2.0 * kb * kb * kb / 3.0, "oz_panel_prep");
+    k_oz_panel_prep<<<dim3(1 + sl.nb0 + (nW + 31) / 32, B), 256, 0, c->st>>>(f, sl, w->plane_stride, w->ldp, c->d_flag);
     prof_end(c);
     OzArgs a{};
     a.pt[0] = oz_part(N, 0, w->EPY, N, w->ET, 32, Y + (long long)k0 * N, c->nn, N);
@@ -1219,7 +1188,7 @@ void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW,
     k_oz_gemm<false, false, true, true>
         <<<oz_grid<false>(w, a), OTHREADS, oz_smem_bytes(), c->st>>>(w->mapA, w->mapRA, w->mapT, w->mapT, a);
     prof_end(c);
-    c->launches += 3;
+    c->launches += 2;
 }
 
 namespace {

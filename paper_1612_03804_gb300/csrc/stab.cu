@@ -23,6 +23,7 @@
 
 #include <mutex>
 
+#include "chol32.cuh"
 #include "internal.h"
 
 namespace sldqmc {
@@ -115,112 +116,56 @@ __global__ void k_gather_pivot(const double *W, long long sW, const double *Xt, 
     }
 }
 
-// One block row of the stacked Cholesky-QR: factor the kb x kb diagonal
-// block W_kk = R_kk^T R_kk (in shared memory, every CTA redundantly), then
-// solve R_kk^T y = w for each column: W-columns right of the block give
-// R's block row, Y-columns give Q^T's block row (in place).
-template <int KB, int CPT>
-__global__ void __launch_bounds__(128) k_chol_panel(const double *W, long long sW, int ldw, double *Y,
-                                                    long long sY, double *R, long long sR, int N,
-                                                    int k0, int kb, int *flag)
+// One block row of the stacked Cholesky-QR on the FP64 pipe: factor the kb x
+// kb diagonal block W_kk = R_kk^T R_kk and T = R_kk^-T (in shared memory, every
+// CTA redundantly), then T times the panel's columns: W-columns right of the
+// block give R's block row, Y-columns give Q^T's block row (in place).  A CTA
+// has 32 columns (lanes), its four warps every fourth row each: a warp's FMA
+// holds its sub-partition's FP64 pipe for 64 cycles, so a column's 528 FMAs
+// are spread over all four (4.4 us); one thread per column took 17 us of the
+// same pipe and two columns per thread 35 us, beside a factor of 45 us.
+__global__ void __launch_bounds__(128) k_chol_panel(const double *W, long long sW, int ldw, double *Y, long long sY,
+                                                    double *R, long long sR, int N, int k0, int kb, int *flag)
 {
-    __shared__ double Rk[KB][KB + 1];
-    const int b = blockIdx.y;
+    __shared__ double X[32][33], V[32][33];
+    __shared__ double root[32];
+    const int b = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double *Wb = W + (long long)b * sW;
-    for (int e = threadIdx.x; e < KB * KB; e += blockDim.x) {
-        int r = e / KB, c = e % KB;
-        double v = 0.0;
-        if (r < kb && c < kb) {
-            if (c >= r) v = Wb[(long long)(k0 + r) * ldw + k0 + c];
-        } else if (r == c) {
-            v = 1.0;
-        }
-        Rk[r][c] = v;
+    for (int e = threadIdx.x; e < 32 * 32; e += 128) {
+        const int r = e >> 5, c = e & 31;
+        X[r][c] = r < kb && c < kb ? (c >= r ? Wb[(long long)(k0 + r) * ldw + k0 + c] : 0.0) : (r == c ? 1.0 : 0.0);
     }
-    __syncthreads();
-    // Factor the KB x KB block (right-looking, all threads of the CTA); the
-    // reciprocals of the pivots are kept so that every later division is a
-    // multiplication (FP64 division is many times slower than an FMA here).
-    __shared__ double rinv[KB];
-    for (int j = 0; j < KB; ++j) {
-        if (threadIdx.x == 0) {
-            double d = Rk[j][j];
-            if (!(d > 0.0) || !isfinite(d)) {
-                if (j < kb) atomicOr(flag, FLAG_NUMERICAL);
-                d = 1.0;
-            }
-            d = sqrt(d);
-            Rk[j][j] = d;
-            rinv[j] = 1.0 / d;
-        }
-        __syncthreads();
-        const double ri = rinv[j];
-        for (int c = j + 1 + threadIdx.x; c < KB; c += blockDim.x) Rk[j][c] *= ri;
-        __syncthreads();
-        for (int e = threadIdx.x; e < KB * KB; e += blockDim.x) {
-            int r = e / KB, c = e % KB;
-            if (r > j && c >= r) Rk[r][c] -= Rk[j][r] * Rk[j][c];
-        }
-        __syncthreads();
-    }
-    if (blockIdx.x == 0) {
-        double *Rb = R + (long long)b * sR;
-        for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-            int r = e / kb, c = e % kb;
-            Rb[(long long)(k0 + r) * N + k0 + c] = (c >= r) ? Rk[r][c] : 0.0;
-        }
-    }
+    // this CTA's columns: those of W right of the block, then Y's
     const int nW = N - (k0 + kb);
-    // CPT columns per thread (blockDim.x apart, so each load and store
-    // instruction stays coalesced); every shared-memory load of R_kk then feeds
-    // CPT independent FMA chains.
-    double w[CPT][KB];
-    double *dst[CPT];
-    int cc[CPT];
-    long long ldd[CPT];
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-        const int col = (blockIdx.x * CPT + q) * blockDim.x + threadIdx.x;
-        const double *src = nullptr;
-        long long lds = 0;
-        cc[q] = -1;
-        dst[q] = nullptr;
-        ldd[q] = 0;
-        if (col < nW) {
-            cc[q] = k0 + kb + col;
-            src = Wb; lds = ldw;
-            dst[q] = R + (long long)b * sR; ldd[q] = N;
-        } else if (col < nW + N) {
-            cc[q] = col - nW;
-            src = Y + (long long)b * sY; lds = N;
-            dst[q] = Y + (long long)b * sY; ldd[q] = N;
+    const int col = blockIdx.x * 32 + lane;
+    const bool live = col < nW + N;
+    const bool isW = col < nW;
+    const int cc = isW ? k0 + kb + col : col - nW;
+    const double *src = isW ? Wb : Y + (long long)b * sY;
+    const long long lds = isW ? ldw : N;
+    for (int r = wid; r < 32; r += 4) V[r][lane] = live && r < kb ? src[(long long)(k0 + r) * lds + cc] : 0.0;
+    __syncthreads();
+    chol32(X, root, kb, flag);
+    double *Rb = R + (long long)b * sR;
+    if (blockIdx.x == 0)
+        for (int e = threadIdx.x; e < 32 * 32; e += 128) {
+            const int r = e >> 5, c = e & 31;
+            if (r < kb && c < kb) Rb[(long long)(k0 + r) * N + k0 + c] = c > r ? X[r][c] : (c == r ? root[r] : 0.0);
         }
+    double *dst = isW ? Rb : Y + (long long)b * sY;
+    double acc[8];
 #pragma unroll
-        for (int r = 0; r < KB; ++r) w[q][r] = (cc[q] >= 0 && r < kb) ? src[(long long)(k0 + r) * lds + cc[q]] : 0.0;
+    for (int q = 0; q < 8; ++q) acc[q] = 0.0;
+    for (int l = 0; l < kb; ++l) {
+        const double v = V[l][lane];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (4 * q + wid >= l) acc[q] += X[4 * q + wid][l] * v;
     }
-    // Column-oriented order: once w[l] is final, its contribution is
-    // subtracted from every later w[r] -- up to KB - 1 independent FMAs per
-    // step.  Each w[r] receives the same operations in the same order as in
-    // the row-oriented form (r's terms l = 0, 1, ..., r - 1, then the scale).
+    if (!live) return;
 #pragma unroll
-    for (int l = 0; l < KB; ++l) {
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) w[q][l] *= rinv[l];
-#pragma unroll
-        for (int r = 0; r < KB; ++r) {
-            if (r > l) {
-                const double rl = Rk[l][r];
-#pragma unroll
-                for (int q = 0; q < CPT; ++q) w[q][r] -= rl * w[q][l];
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < CPT; ++q)
-        if (cc[q] >= 0)
-#pragma unroll
-            for (int r = 0; r < KB; ++r)
-                if (r < kb) dst[q][(long long)(k0 + r) * ldd[q] + cc[q]] = w[q][r];
+    for (int q = 0; q < 8; ++q)
+        if (4 * q + wid < kb) dst[(long long)(k0 + 4 * q + wid) * N + cc] = acc[q];
 }
 
 // D_new[k] = R_kk * D_p[k]  (R from Cholesky has a positive diagonal).
@@ -851,9 +796,7 @@ void launch_init_udv(sldqmc_ctx *c, double *Ut, double *V, int B)
     c->launches++;
 }
 
-constexpr int CHOL_CPT = 2;      // columns per thread of the panel solves
 constexpr int CHOL_BLOCK = 256;  // rows per block of the left-looking tensor-core Cholesky-QR
-constexpr int CHOL_THREADS = 128; // threads per CTA of the panel kernel
 
 static void chol_pass(sldqmc_ctx *c, double *W, long long sW, double *Y, double *R, int B)
 {
@@ -865,7 +808,7 @@ static void chol_pass(sldqmc_ctx *c, double *W, long long sW, double *Y, double 
     // and Q^T are its rows of W and Y multiplied by the inverse of the
     // diagonal block's factor (all FP64-accurate digit splitting), and that
     // product also splits the finished rows for the later panels.  Otherwise
-    // right-looking with FP64 triangular solves and trailing updates.
+    // right-looking with FP64 panels and trailing updates.
     const bool oz = c->oz_ws != nullptr;
     if (oz) {
         // blocks of CHOL_BLOCK rows: one update of the block's rows with every
@@ -889,10 +832,10 @@ static void chol_pass(sldqmc_ctx *c, double *W, long long sW, double *Y, double 
         int kb = N - k0 < 32 ? N - k0 : 32;
         int nW = N - (k0 + kb);
         {
-            dim3 grid(cdiv(nW + N, CHOL_THREADS * CHOL_CPT), B);
+            dim3 grid(cdiv(nW + N, 32), B);
             // algorithmic flops: factor of the kb x kb block, triangular solves of nW + N columns
             prof_begin(c, SLDQMC_KC_PANEL_F64, (double)B * ((double)kb * kb * kb / 3.0 + (double)(nW + N) * kb * kb), "chol_panel_f64");
-            k_chol_panel<32, CHOL_CPT><<<grid, CHOL_THREADS, 0, c->st>>>(W, sW, N, Y, nn, R, nn, N, k0, kb, c->d_flag);
+            k_chol_panel<<<grid, 128, 0, c->st>>>(W, sW, N, Y, nn, R, nn, N, k0, kb, c->d_flag);
             prof_end(c);
             c->launches++;
         }
