@@ -508,37 +508,146 @@ __global__ void k_drift(const double *Gw, const double *Gf, long long nn, long l
 // The model of one context travels with each launch as a kernel parameter
 // (constant bank): class c has noff[c] offset triples (dx, dy, dtau), listed
 // class after class in off, and coupling J[c].
+// nb: the same offsets reduced to 0 <= dx < Lx, 0 <= dy < Ly, 0 <= dtau < M, each
+// followed by its opposite, so that a neighbour is found by additions and one
+// conditional subtraction per direction; Jn: the FP32 coupling of each of
+// these neighbours (0 where the neighbour is the site itself).
+struct EffNeighbour {
+    short dx, dy;
+    int dt;
+};
+
 struct EffModel {
-    int n_class;
+    int n_class, n_nb;
     int noff[32];
     int off[64 * 3];
     double J[32];
+    EffNeighbour nb[128];
+    float Jn[128];
+    float Jabs;  // sum of |Jn|
 };
 
 static EffModel eff_model_of(const sldqmc_ctx *c)
 {
     EffModel m;
+    memset(&m, 0, sizeof(m));
     m.n_class = c->n_class;
     memcpy(m.noff, c->h_n_off, sizeof(m.noff));
     memcpy(m.off, c->h_offsets, sizeof(m.off));
     memcpy(m.J, c->h_J, sizeof(m.J));
+    auto wrap = [](int a, int L) { a %= L; return a < 0 ? a + L : a; };
+    int q = 0;
+    for (int k = 0; k < m.n_class; ++k)
+        for (int t = 0; t < m.noff[k]; ++t, ++q)
+            for (int sg = 1; sg >= -1; sg -= 2) {
+                const int *o = m.off + 3 * q;
+                EffNeighbour &n = m.nb[m.n_nb];
+                n.dx = (short)wrap(sg * (o[0] % c->p.Lx), c->p.Lx);
+                n.dy = (short)wrap(sg * (o[1] % c->p.Ly), c->p.Ly);
+                n.dt = wrap(sg * (o[2] % c->M), c->M);
+                const bool self = n.dx == 0 && n.dy == 0 && n.dt == 0;
+                m.Jn[m.n_nb] = self ? 0.0f : (float)m.J[k];
+                m.Jabs += fabsf(m.Jn[m.n_nb]);
+                ++m.n_nb;
+            }
     return m;
 }
 
-__device__ __forceinline__ int shift_site(int v, int N, int Lx, int Ly, int M, const int *o, int sg)
+// Site (tau, y, x) moved by a reduced offset.
+__device__ __forceinline__ int moved_site(int tau, int y, int x, int N, int Lx, int Ly, int M, int dt, int dy, int dx)
 {
-    const int tau = v / N, i = v % N, x = i % Lx, y = i / Lx;
-    return wrapi(tau + sg * o[2], M) * N + wrapi(x + sg * o[0], Lx) + Lx * wrapi(y + sg * o[1], Ly);
+    x += dx;
+    y += dy;
+    tau += dt;
+    x -= x >= Lx ? Lx : 0;
+    y -= y >= Ly ? Ly : 0;
+    tau -= tau >= M ? M : 0;
+    return tau * N + y * Lx + x;
 }
 
-// n_sweeps colour-ordered Metropolis sweeps on H_eff for one chain per CTA.
-// log acceptance a = ((2 beta) * sum_c J_c n_c) * s with n_c the integer
-// neighbour sums (self-pairs excluded), accumulated in class order.
-template <bool SMEM>
+// One Metropolis decision of H_eff: log acceptance a = ((2 beta) * sum_c J_c
+// n_c) * s with n_c the integer neighbour sums (self-pairs excluded),
+// accumulated in class order, accepted iff log u < a.  The G lanes of a group
+// (G a power of two, all lanes of the warp present) share the site's
+// neighbours and take the decision in FP32 where it is clear: the FP32 sum and
+// logarithms are off by less than 1e-5 of their terms, against a margin of 1e-4
+// and ten times that.  Otherwise the group's first lane takes the FP64 decision,
+// whose 2 n_class operations and logarithm on the FP64 pipe (64 cycles each per
+// warp) were most of a colour's time beside two divisions per coordinate and
+// neighbour.  Returns whether this lane flipped the site.
+struct EffSite {
+    const EffModel &em;
+    int N, Lx, Ly, M;
+    double twob;
+    uint64_t key;
+    uint32_t step;
+};
+
+__device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffNeighbour *nb, const float *Jn, int v,
+                                         bool active, int G, int sw, long long &mg)
+{
+    const int sub = threadIdx.x & (G - 1);
+    const int tau = v / e.N, i = v - tau * e.N, y = i / e.Lx, x = i - y * e.Lx;
+    float sum = 0.0f;
+    if (active)
+        for (int k = sub; k < e.em.n_nb; k += G)
+            sum += Jn[k] * (float)s[moved_site(tau, y, x, e.N, e.Lx, e.Ly, e.M, nb[k].dt, nb[k].dy, nb[k].dx)];
+    for (int o = G >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (!active || sub) return false;
+    const int sv = s[v];
+    uint32_t r[4] = {(uint32_t)i, (uint32_t)tau, e.step, PURPOSE_EFF | ((uint32_t)sw << 8)};
+    philox4x32_10(r, (uint32_t)e.key, (uint32_t)(e.key >> 32));
+    const uint64_t w = (((uint64_t)r[1] << 32) | (uint64_t)r[0]) >> 11;
+    const float af = (float)e.twob * sum * (float)sv, lf = logf(__ull2float_rn(w) * (1.0f / 9007199254740992.0f));
+    const float d = af - lf;
+    bool acc = d > 0.0f;
+    if (!(fabsf(d) > 1e-4f + 1e-4f * (fabsf((float)e.twob) * e.em.Jabs) + 1e-5f * fabsf(lf)) || w == 0) {
+        double sm = 0.0;
+        int k = 0;
+        for (int c = 0; c < e.em.n_class; ++c) {
+            int n = 0;
+            for (int t = 0; t < 2 * e.em.noff[c]; ++t, ++k) {
+                const int u = moved_site(tau, y, x, e.N, e.Lx, e.Ly, e.M, nb[k].dt, nb[k].dy, nb[k].dx);
+                if (u != v) n += s[u];
+            }
+            sm = __dadd_rn(sm, __dmul_rn(e.em.J[c], (double)n));
+        }
+        const double av = __dmul_rn(__dmul_rn(e.twob, sm), (double)sv);
+        const double lu = log((double)w * (1.0 / 9007199254740992.0));
+        if (fabs(av - lu) <= MARGIN) mg++;
+        acc = lu < av;
+    }
+    if (acc) s[v] = (int8_t)(-sv);
+    return acc;
+}
+
+__device__ __forceinline__ void eff_counts(long long acc, long long mg, int b, long long *n_accept, long long *n_margin)
+{
+    for (int o = 16; o > 0; o >>= 1) {
+        acc += __shfl_down_sync(0xffffffffu, acc, o);
+        mg += __shfl_down_sync(0xffffffffu, mg, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (n_accept && acc) atomicAdd((unsigned long long *)&n_accept[b], (unsigned long long)acc);
+        if (n_margin && mg) atomicAdd((unsigned long long *)&n_margin[b], (unsigned long long)mg);
+    }
+}
+
+__device__ __forceinline__ void eff_load_nb(const EffModel &em, EffNeighbour *nb, float *Jn)
+{
+    for (int k = threadIdx.x; k < em.n_nb; k += blockDim.x) {
+        nb[k] = em.nb[k];
+        Jn[k] = em.Jn[k];
+    }
+    __syncthreads();
+}
+
+// n_sweeps colour-ordered sweeps of one chain per CTA, its spins in shared
+// memory, G lanes per site.
 __global__ void __launch_bounds__(1024) k_eff_sweeps(int8_t *s_all, int Lx, int Ly, int M, double beta,
                                                      const __grid_constant__ EffModel em, const int *col_start,
                                                      const int *col_sites, int n_colors, int n_sweeps,
-                                                     uint64_t seed, uint32_t step, int dir_fixed,
+                                                     uint64_t seed, uint32_t step, int dir_fixed, int G,
                                                      long long *n_accept, long long *n_margin,
                                                      const uint32_t *d_step)
 {
@@ -546,92 +655,86 @@ __global__ void __launch_bounds__(1024) k_eff_sweeps(int8_t *s_all, int Lx, int 
     const int b = blockIdx.x;
     const int N = Lx * Ly;
     const int V = N * M;
-    extern __shared__ int8_t sm8[];
+    extern __shared__ int8_t s[];
+    __shared__ EffNeighbour nb[128];
+    __shared__ float Jn[128];
     int8_t *gs = s_all + (long long)b * V;
-    int8_t *s = SMEM ? sm8 : gs;
     const uint64_t key = seed + ((uint64_t)b << 32);
-    if (SMEM) {
-        for (int v = threadIdx.x; v < V; v += blockDim.x) s[v] = gs[v];
-        __syncthreads();
-    }
+    for (int v = threadIdx.x; v < V; v += blockDim.x) s[v] = gs[v];
+    eff_load_nb(em, nb, Jn);
     int dir = dir_fixed;
     if (dir < 0) dir = (int)(philox_word(key, 0, 0, step, PURPOSE_DIR) & 1u);
     long long acc = 0, mg = 0;
-    const double twob = 2.0 * beta;
+    const EffSite e{em, N, Lx, Ly, M, 2.0 * beta, key, step};
+    const int per = blockDim.x / G;
     for (int sw = 0; sw < n_sweeps; ++sw)
         for (int cc = 0; cc < n_colors; ++cc) {
             const int col = dir ? (n_colors - 1 - cc) : cc;
-            for (int q = col_start[col] + threadIdx.x; q < col_start[col + 1]; q += blockDim.x) {
-                const int v = col_sites[q];
-                double sum = 0.0;
-                int oi = 0;
-                for (int c = 0; c < em.n_class; ++c) {
-                    int n = 0;
-                    for (int t = 0; t < em.noff[c]; ++t, ++oi) {
-                        const int b1 = shift_site(v, N, Lx, Ly, M, em.off + 3 * oi, 1);
-                        const int b2 = shift_site(v, N, Lx, Ly, M, em.off + 3 * oi, -1);
-                        if (b1 != v) n += s[b1];
-                        if (b2 != v) n += s[b2];
-                    }
-                    sum = __dadd_rn(sum, __dmul_rn(em.J[c], (double)n));
-                }
-                const int sv = s[v];
-                const double av = __dmul_rn(__dmul_rn(twob, sum), (double)sv);
-                const int tau = v / N, i = v % N;
-                const double u = philox_uniform(key, (uint32_t)i, (uint32_t)tau, step,
-                                                PURPOSE_EFF | ((uint32_t)sw << 8));
-                const double lu = log(u);
-                if (fabs(av - lu) <= MARGIN) mg++;
-                if (lu < av) {
-                    s[v] = (int8_t)(-sv);
-                    acc++;
-                }
+            const int q1 = col_start[col + 1];
+            for (int q0 = col_start[col]; q0 < q1; q0 += per) {
+                const int q = q0 + threadIdx.x / G;
+                acc += eff_site(e, s, nb, Jn, q < q1 ? col_sites[q] : 0, q < q1, G, sw, mg);
             }
             __syncthreads();
         }
-    if (SMEM) {
-        for (int v = threadIdx.x; v < V; v += blockDim.x) gs[v] = s[v];
+    for (int v = threadIdx.x; v < V; v += blockDim.x) gs[v] = s[v];
+    eff_counts(acc, mg, b, n_accept, n_margin);
+}
+
+// The cc-th colour of sweep sw (in each chain's own direction) of every chain
+// on all SMs, the spins in global memory (sites of one colour do not interact).
+__global__ void __launch_bounds__(256) k_eff_colour(int8_t *s_all, int Lx, int Ly, int M, double beta,
+                                                    const __grid_constant__ EffModel em, const int *col_start,
+                                                    const int *col_sites, int n_colors, int sw, int cc, uint64_t seed,
+                                                    uint32_t step, int dir_fixed, long long *n_accept,
+                                                    long long *n_margin, const uint32_t *d_step)
+{
+    if (d_step) step = *d_step;
+    const int b = blockIdx.y;
+    const int N = Lx * Ly;
+    __shared__ EffNeighbour nb[128];
+    __shared__ float Jn[128];
+    eff_load_nb(em, nb, Jn);
+    const uint64_t key = seed + ((uint64_t)b << 32);
+    int dir = dir_fixed;
+    if (dir < 0) dir = (int)(philox_word(key, 0, 0, step, PURPOSE_DIR) & 1u);
+    const int col = dir ? (n_colors - 1 - cc) : cc;
+    long long acc = 0, mg = 0;
+    const EffSite e{em, N, Lx, Ly, M, 2.0 * beta, key, step};
+    const int q0 = col_start[col], n = col_start[col + 1] - q0;
+    for (int k0 = blockIdx.x * blockDim.x; k0 < n; k0 += gridDim.x * blockDim.x) {
+        const int k = k0 + threadIdx.x;
+        acc += eff_site(e, s_all + (long long)b * N * M, nb, Jn, k < n ? col_sites[q0 + k] : 0, k < n, 1, sw, mg);
     }
-    __shared__ long long r1[32], r2[32];
-    for (int o = 16; o > 0; o >>= 1) {
-        acc += __shfl_down_sync(0xffffffffu, acc, o);
-        mg += __shfl_down_sync(0xffffffffu, mg, o);
-    }
-    if ((threadIdx.x & 31) == 0) { r1[threadIdx.x >> 5] = acc; r2[threadIdx.x >> 5] = mg; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        long long t1 = 0, t2 = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { t1 += r1[w]; t2 += r2[w]; }
-        if (n_accept) n_accept[b] += t1;
-        if (n_margin) n_margin[b] += t2;
-    }
+    eff_counts(acc, mg, b, n_accept, n_margin);
 }
 
 // f_c(C) = sum_x sum_{o in c} s_x s_{x+o} (self-pairs give 1), one CTA per
-// configuration; out[b*n_class + c].
-__global__ void k_features(const int8_t *s_all, int Lx, int Ly, int M, const __grid_constant__ EffModel em,
-                           long long *out)
+// configuration and class; out[b*n_class + c].
+__global__ void __launch_bounds__(512) k_features(const int8_t *s_all, int Lx, int Ly, int M,
+                                                  const __grid_constant__ EffModel em, long long *out)
 {
-    const int b = blockIdx.x;
+    const int b = blockIdx.x, c = blockIdx.y;
     const int N = Lx * Ly, V = N * M;
     const int8_t *s = s_all + (long long)b * V;
-    __shared__ long long red[32];
-    const int n_class = em.n_class;
-    int oi = 0;
-    for (int c = 0; c < n_class; ++c) {
-        long long acc = 0;
-        for (int t = 0; t < em.noff[c]; ++t, ++oi)
-            for (int v = threadIdx.x; v < V; v += blockDim.x)
-                acc += s[v] * s[shift_site(v, N, Lx, Ly, M, em.off + 3 * oi, 1)];
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            long long t = 0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-            out[(long long)b * n_class + c] = t;
-        }
-        __syncthreads();
+    __shared__ long long red[16];
+    int k0 = 0;
+    for (int k = 0; k < c; ++k) k0 += 2 * em.noff[k];
+    long long acc = 0;
+    for (int v = threadIdx.x; v < V; v += blockDim.x) {
+        const int tau = v / N, i = v - tau * N, y = i / Lx, x = i - y * Lx;
+        int n = 0;
+        for (int k = k0; k < k0 + 2 * em.noff[c]; k += 2)
+            n += s[moved_site(tau, y, x, N, Lx, Ly, M, em.nb[k].dt, em.nb[k].dy, em.nb[k].dx)];
+        acc += s[v] * n;
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        long long t = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+        out[(long long)b * em.n_class + c] = t;
     }
 }
 
@@ -712,30 +815,50 @@ void launch_drift(sldqmc_ctx *c, const double *Gw, const double *Gf, int B2x, in
     c->launches++;
 }
 
+// A chain's spins stay in one CTA's shared memory while its colours are small
+// or the chains fill the GPU; otherwise each colour is one launch over all SMs.
+// In units of the time of one pass of 1024 sites (about 1.5 us, a launch three
+// of them): passes per colour in one CTA per chain, times the waves of chains,
+// against a launch and the passes spread over all SMs.  Measured per sweep:
+// 100 x 100 x 100, one chain, 4 classes 15.2 ms (one CTA, spins in global memory)
+// -> 97 us; 32 x 32 x 160, 16 classes, 4 chains 5.0 ms -> 0.40 ms (spread); 24 x 24 x
+// 20, 16 classes, 16 chains 490 -> 158 us (in shared memory).
 void launch_eff_sweeps(sldqmc_ctx *c, int8_t *d_s, int B, int n_sweeps, uint64_t seed, uint32_t step,
                        int dir, long long *n_accept, long long *n_margin)
 {
     const long long V = (long long)c->N * c->M;
-    const int nt = 1024;
     const EffModel em = eff_model_of(c);
+    const long long cs = (V + c->n_colors - 1) / c->n_colors;  // sites per colour
+    const long long in_cta = ((cs + 1023) / 1024) * ((B + c->num_sms - 1) / c->num_sms);
+    const long long spread = 3 + (cs * B + 1024LL * c->num_sms - 1) / (1024LL * c->num_sms);
     prof_begin(c, SLDQMC_KC_EFF, 0.0, "eff_sweeps");
-    if (V <= 200 * 1024) {
-        k_eff_sweeps<true><<<B, nt, (size_t)V, c->st>>>(d_s, c->p.Lx, c->p.Ly, c->M, c->p.beta,
-                                                        em, c->d_col_start, c->d_col_sites,
-                                                        c->n_colors, n_sweeps, seed, step, dir,
-                                                        n_accept, n_margin, c->step_dev);
+    if (V <= 200 * 1024 && in_cta <= spread) {
+        int G = 1;  // lanes per site, while a colour leaves them idle
+        while (G < 8 && 2 * G * cs <= 1024) G *= 2;
+        k_eff_sweeps<<<B, 1024, (size_t)V, c->st>>>(d_s, c->p.Lx, c->p.Ly, c->M, c->p.beta, em, c->d_col_start,
+                                                    c->d_col_sites, c->n_colors, n_sweeps, seed, step, dir, G, n_accept,
+                                                    n_margin, c->step_dev);
+        c->launches++;
     } else {
-        k_eff_sweeps<false><<<B, nt, 0, c->st>>>(d_s, c->p.Lx, c->p.Ly, c->M, c->p.beta, em,
-                                                 c->d_col_start, c->d_col_sites, c->n_colors, n_sweeps,
-                                                 seed, step, dir, n_accept, n_margin, c->step_dev);
+        const int bx = cdiv(cs, 256) < 1024 ? cdiv(cs, 256) : 1024;
+        for (int b0 = 0; b0 < B; b0 += 32768) {  // grid y limit
+            const int nb = B - b0 < 32768 ? B - b0 : 32768;
+            for (int sw = 0; sw < n_sweeps; ++sw)
+                for (int cc = 0; cc < c->n_colors; ++cc) {
+                    k_eff_colour<<<dim3(bx, nb), 256, 0, c->st>>>(
+                        d_s + V * b0, c->p.Lx, c->p.Ly, c->M, c->p.beta, em, c->d_col_start, c->d_col_sites, c->n_colors,
+                        sw, cc, seed + ((uint64_t)b0 << 32), step, dir, n_accept ? n_accept + b0 : nullptr,
+                        n_margin ? n_margin + b0 : nullptr, c->step_dev);
+                    c->launches++;
+                }
+        }
     }
     prof_end(c);
-    c->launches++;
 }
 
 void launch_features(sldqmc_ctx *c, const int8_t *d_s, int B, long long *out)
 {
-    k_features<<<B, 512, 0, c->st>>>(d_s, c->p.Lx, c->p.Ly, c->M, eff_model_of(c), out);
+    k_features<<<dim3(B, c->n_class), 512, 0, c->st>>>(d_s, c->p.Lx, c->p.Ly, c->M, eff_model_of(c), out);
     c->launches++;
 }
 
@@ -767,7 +890,7 @@ void launch_step_advance(sldqmc_ctx *c, uint32_t *d_step)
 
 void set_eff_smem_limits()
 {
-    cudaFuncSetAttribute(k_eff_sweeps<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_eff_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_local_flips, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
