@@ -94,7 +94,15 @@ void oz_delayed_update(sldqmc_ctx *c, double *const *G, const FlipPairs *pairs, 
 // sk); oz_similarity: dst_f = P src_f P^-1 of both flavours, P = E or, with
 // inv, E^-1, rows and columns then scaled by d_i / d_j of the field slice s
 // (null: no scaling), T_f an N x N scratch per item.
+// oz_worth: whether they are the faster way for B items; oz_full: every
+// product of the context runs there (N >= 128).  oz_chain_block: the slice
+// products of a whole block in one launch (oz_chain_fits: N <= 64).
 bool oz_have_e(sldqmc_ctx *c);
+bool oz_worth(const sldqmc_ctx *c, int B);
+bool oz_full(const sldqmc_ctx *c);
+bool oz_chain_fits(const sldqmc_ctx *c);
+void oz_chain_block(sldqmc_ctx *c, const double *Ut, const int8_t *d_s, int B, double cu, double cd, int t0, int nb,
+                    double *Xt_out);
 void oz_slice_product(sldqmc_ctx *c, const double *X, const int8_t *sk, double cu, double cd, double *Xt, int B);
 void oz_similarity(sldqmc_ctx *c, const double *const *src, double *const *T, double *const *dst, int inv,
                    const int8_t *s, const double (*ex)[2], int B);

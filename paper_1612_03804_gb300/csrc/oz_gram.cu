@@ -508,7 +508,10 @@ __device__ __forceinline__ double oz_round(long long h, long long l, int e)
         }
     const int s = __clz((int)t2);
     ex -= s;
-    if (t2 == 0u || (unsigned)(ex - 1) >= 2045u) return oz_round_fp(h, l, e);  // zero, subnormal, too large, NaN
+    if (t2 == 0u || (unsigned)(ex - 1) >= 2045u) {  // zero, subnormal, too large, NaN
+        if ((t2 | t1 | t0) == 0u && e <= OZ_NONFINITE / 2) return 0.0;
+        return oz_round_fp(h, l, e);
+    }
     const uint32_t a = __funnelshift_l(t1, t2, s), b = __funnelshift_l(t0, t1, s);
     const uint32_t rem = (b << 21) | ((t0 << s) != 0u ? 1u : 0u);  // the bits below the 53rd
     unsigned long long m = ((unsigned long long)a << 21) | (b >> 11);
@@ -875,6 +878,272 @@ __global__ void __launch_bounds__(OTHREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OTMEM) : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// The slice products of a whole stabilisation block for N <= 64: X^T <- X^T D E
+// acts on every row of X^T alone, so a CTA keeps 128 rows (of one item or of
+// several, the rows of all items lie one after another) for all slices, as
+// digit planes in shared memory (8 x 16 KB) beside E's (8 x 8 KB).  Per slice:
+// 48 MMAs into eight 64-column groups (all of tensor memory), then every
+// thread combines the groups of a row's 16 columns exactly, rounds, scales by
+// the next slice's D, and splits again.  No global memory and no launch
+// between slices.  Bound by the integer work of combining and splitting (about
+// 110 instructions per element, 16 warps) after 2.4 us of MMAs.
+// Measured at 8 x 8, 64 items: 12 us per slice (15 with FP64 rounding and scaling
+// in between); one FP64 GEMM launch per slice took 44 us.
+constexpr int CH_N = 64, CH_THREADS = 512;
+constexpr int CH_TILE_A = OBM * 128, CH_TILE_B = CH_N * 128;  // one plane: 64 BF16 (128 bytes) per row
+constexpr size_t CH_SMEM = OZ_S * (CH_TILE_A + CH_TILE_B) + 1024 + 4 * OBM * 4 + CH_N * 4 + 64;
+
+struct ChainArgs {
+    const double *U;
+    double *X;
+    const int8_t *s;
+    long long sS;
+    int rows, N, M, t0, nb;
+    double cu, cd;
+    const __nv_bfloat16 *ep;  // E's planes
+    long long eps;
+    int ldp;
+    const int *EE;
+    int *flag;
+};
+
+// A value of the row between two products: (-1)^neg m 2^(ex - 63), 2^63 <= m <
+// 2^64, or m = 0.  Scaling, the row's maximum and the splitting need no FP64
+// (a warp's FP64 instruction holds the pipe for 64 cycles) and no rounding to
+// 53 bits in between.
+struct ChValue {
+    unsigned long long m;
+    int ex, neg;
+};
+constexpr int CH_ZERO = -(1 << 24);  // exponent of zero
+
+__device__ __forceinline__ ChValue ch_from(double x, double d)
+{
+    const double y = x * d;
+    const long long u = __double_as_longlong(y);
+    const int ef = (int)((u >> 52) & 0x7FF);
+    ChValue v;
+    v.neg = u < 0;
+    v.m = ef ? (((unsigned long long)u << 11) | (1ull << 63)) : 0ull;
+    v.ex = ef == 0x7FF ? OZ_NONFINITE : ef ? ef - 1023 : CH_ZERO;
+    return v;
+}
+
+// (h + l 2^-28) 2^e times d = dm 2^(dex - 63) (2^63 <= dm)
+__device__ __forceinline__ ChValue ch_scaled(long long h, long long l, int e, unsigned long long dm, int dex)
+{
+    unsigned long long lo = ((unsigned long long)h << 28) + (unsigned long long)l;
+    long long hi = (h >> 36) + (l >> 63) + (lo < (unsigned long long)l ? 1 : 0);
+    ChValue v;
+    v.neg = hi < 0;
+    if (hi < 0) {
+        lo = 0ull - lo;
+        hi = ~hi + (lo == 0ull ? 1 : 0);
+    }
+    uint32_t t2 = (uint32_t)hi, t1 = (uint32_t)(lo >> 32), t0 = (uint32_t)lo;
+    int ex = e + 95 - 28 + dex;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (t2 == 0u) {
+            t2 = t1;
+            t1 = t0;
+            t0 = 0u;
+            ex -= 32;
+        }
+    const int s = __clz((int)t2);
+    const unsigned long long top = ((unsigned long long)__funnelshift_l(t1, t2, s) << 32) | __funnelshift_l(t0, t1, s);
+    // dm / 2^63 is in [1, 2): the product's high word is half of top dm / 2^63
+    v.m = __umul64hi(top, dm);
+    const int up = (int)(v.m >> 63);
+    v.m <<= 1 - up;
+    v.ex = t2 == 0u ? CH_ZERO : ex - s + up;
+    if (e > OZ_NONFINITE / 2) v.ex = OZ_NONFINITE;
+    return v;
+}
+
+// v 2^(57 - E) rounded to an integer, plus the bias that makes each of the
+// seven low 7-bit fields a digit + 64; |v| < 2^E.
+__device__ __forceinline__ long long ch_fixed(const ChValue &v, int E)
+{
+    const int r = E - v.ex + 63 - OZ_BITS;  // >= 7
+    long long w = 0;
+    if (r < 64) w = (long long)(((v.m >> (r - 1)) + 1ull) >> 1);
+    constexpr long long bias = 64ll * (1 + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) + (1ll << 35) + (1ll << 42));
+    return (v.neg ? -w : w) + bias;
+}
+
+// Digit p of two such values as a pair of BF16: an integer below 2^23 placed
+// in the mantissa of 2^23 (1.5 2^23 for the signed leading digit) is converted
+// by one FP32 subtraction, and BF16 is the upper half of its FP32.
+__device__ __forceinline__ uint32_t ch_pair(long long a, long long b, int p)
+{
+    float fa, fb;
+    if (p == 0) {
+        fa = __uint_as_float(0x4B400000u + (uint32_t)(int)(a >> 49)) - 12582912.0f;
+        fb = __uint_as_float(0x4B400000u + (uint32_t)(int)(b >> 49)) - 12582912.0f;
+    } else {
+        const int s = 7 * (7 - p);
+        fa = __uint_as_float(0x4B000000u | ((uint32_t)(a >> s) & 127u)) - 8388672.0f;
+        fb = __uint_as_float(0x4B000000u | ((uint32_t)(b >> s) & 127u)) - 8388672.0f;
+    }
+    return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+}
+
+// Shared-memory descriptor of a K-major operand of 128-byte rows with the
+// 128-byte swizzle (8-row atoms of 1024 bytes).
+__device__ __forceinline__ uint64_t ch_desc(uint32_t saddr)
+{
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)1u << 16) | ((uint64_t)(1024u >> 4) << 32) |
+           ((uint64_t)1u << 46) | ((uint64_t)2u << 61);
+}
+
+__global__ void __launch_bounds__(CH_THREADS, 1) k_oz_chain(ChainArgs a)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *sA = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t *sB = sA + OZ_S * CH_TILE_A;
+    int *s_ef = (int *)(sB + OZ_S * CH_TILE_B);  // [4][128]
+    int *s_ee = s_ef + 4 * OBM;                  // [64]
+    uint64_t *done = (uint64_t *)(s_ee + CH_N);
+    uint32_t *tmem_slot = (uint32_t *)(done + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        mbar_init(done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // E's planes, 16 bytes at a time, in the swizzled layout; rows beyond N zero
+    for (int e = tid; e < OZ_S * CH_N * 8; e += CH_THREADS) {
+        const int p = e >> 9, r = (e >> 3) & 63, ch = e & 7;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (r < a.N) v = *reinterpret_cast<const uint4 *>(a.ep + p * a.eps + (long long)r * a.ldp + 8 * ch);
+        *reinterpret_cast<uint4 *>(sB + p * CH_TILE_B + r * 128 + ((ch ^ (r & 7)) << 4)) = v;
+    }
+    if (tid < CH_N) s_ee[tid] = tid < a.N ? a.EE[tid] : 0;
+    // this thread's row (tensor-memory lane quarter warp % 4) and 16 columns
+    const int row = (warp & 3) * 32 + lane, cg = warp >> 2, n0 = 16 * cg;
+    const int g = blockIdx.x * OBM + row;
+    const bool live = g < a.rows;
+    const int8_t *s = a.s + (live ? (long long)(g / a.N) * a.sS : 0) + n0;
+    auto signs = [&](int slice) {  // bit j: spin of column n0 + j is up
+        uint32_t m = 0;
+        const int8_t *sl = s + (long long)slice * a.N;
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (live && n0 + j < a.N && sl[j] > 0) m |= 1u << j;
+        return m;
+    };
+    ChValue x[16];
+    int slice = a.t0;
+    uint32_t up = signs(slice);
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+        x[j] = ch_from(live && n0 + j < a.N ? a.U[(long long)g * a.N + n0 + j] : 0.0, (up >> j) & 1u ? a.cu : a.cd);
+    const unsigned long long mu = ((unsigned long long)__double_as_longlong(a.cu) << 11) | (1ull << 63),
+                             md = ((unsigned long long)__double_as_longlong(a.cd) << 11) | (1ull << 63);
+    const int eu = ((__double2hiint(a.cu) >> 20) & 0x7FF) - 1023, ed = ((__double2hiint(a.cd) >> 20) & 0x7FF) - 1023;
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tmem_slot;
+    bool ok = true;
+    for (int j = 0; j < a.nb; ++j) {
+        // split the row: its exponent over the four column groups, then the digits
+        int exm = CH_ZERO;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) exm = max(exm, x[k].ex);
+        s_ef[cg * OBM + row] = exm;
+        if (!__syncthreads_and(ok)) break;  // also: every thread has read the previous slice's tensor memory
+        exm = max(max(s_ef[row], s_ef[OBM + row]), max(s_ef[2 * OBM + row], s_ef[3 * OBM + row]));
+        // the exponent of a row of zeros is of no account; of one with an
+        // infinity or a NaN, OZ_NONFINITE (all of its other digits are then zero)
+        const int Ei = exm >= OZ_NONFINITE ? OZ_NONFINITE : exm == CH_ZERO ? 0 : exm + 1;
+#pragma unroll
+        for (int c8 = 0; c8 < 2; ++c8) {
+            if (n0 >= a.N) break;  // no MMA reads these columns
+            long long v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = ch_fixed(x[8 * c8 + k], Ei);
+            uint8_t *dst = sA + row * 128 + (((2 * cg + c8) ^ (row & 7)) << 4);
+#pragma unroll
+            for (int p = 0; p < OZ_S; ++p)
+                *reinterpret_cast<uint4 *>(dst + p * CH_TILE_A) =
+                    make_uint4(ch_pair(v[0], v[1], p), ch_pair(v[2], v[3], p), ch_pair(v[4], v[5], p), ch_pair(v[6], v[7], p));
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        fence_before();
+        __syncthreads();
+        if (tid == 0) {
+            fence_after();
+            const uint32_t ua = smem_u32(sA), ub = smem_u32(sB);
+            for (int k = 0; k < (a.N + 15) / 16; ++k)
+#pragma unroll
+                for (int p = 0; p < OZ_S; ++p)
+#pragma unroll
+                    for (int q = 0; q < OZ_S - p; q += 4) {
+                        // A's plane p times up to four of B's planes q.., into groups p + q..
+                        const int nq = OZ_S - p - q < 4 ? OZ_S - p - q : 4;
+                        mma_bf16(tmem + (uint32_t)((p + q) * CH_N), ch_desc(ua + p * CH_TILE_A + k * 32),
+                                 ch_desc(ub + q * CH_TILE_B + k * 32), oz_idesc(CH_N * nq), (k != 0 || p != 0) ? 1u : 0u);
+                    }
+            mma_commit(done);
+        }
+        if (++slice == a.M) slice = 0;
+        const bool last = j == a.nb - 1;
+        up = last ? 0u : signs(slice);
+        ok = mbar_wait(done, j & 1, a.flag);
+        fence_after();
+        const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)n0;
+#pragma unroll
+        for (int c8 = 0; c8 < 2; ++c8) {
+            if (n0 + 8 * c8 >= a.N) break;  // x stays zero
+            // Group sums below 2^22 (64 products of at most 2^16, all at that bound
+            // only for a constant row of exp(-dtau K)): with 1.5 2^23 added, the bits
+            // of the FP32 are the integer plus a constant.  Two neighbouring groups
+            // fit 32 bits (2^29), so one wide multiply-add joins four.
+            long long hl[2][8];
+#pragma unroll
+            for (int gg = 0; gg < OZ_G; gg += 4) {
+                uint32_t r[4][8];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) tmem_ld8_nowait(lane_base + (uint32_t)((gg + q) * CH_N + 8 * c8), r[q]);
+                tmem_wait_ld8x4(r[0], r[1], r[2], r[3]);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    uint32_t b[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) b[q] = __float_as_uint(__uint_as_float(r[q][k]) + 12582912.0f);
+                    const int w0 = (int)((b[0] << 7) + b[1] - 0x4B400000u * 129u), w1 = (int)((b[2] << 7) + b[3] - 0x4B400000u * 129u);
+                    hl[gg >> 2][k] = (long long)w0 * (1 << 14) + w1;
+                }
+            }
+            if (last) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int n = n0 + 8 * c8 + k;
+                    if (ok && live && n < a.N) a.X[(long long)g * a.N + n] = oz_round(hl[0][k], hl[1][k], Ei + s_ee[n] - 37);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const bool u = (up >> (8 * c8 + k)) & 1u;
+                    x[8 * c8 + k] = ch_scaled(hl[0][k], hl[1][k], Ei + s_ee[n0 + 8 * c8 + k] - 37, u ? mu : md, u ? eu : ed);
+                }
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
 struct OzWs {
     int ldp;
     long long plane_stride;
@@ -930,11 +1199,15 @@ bool encode4(CUtensorMap *map, void *ptr, int ldp, int rows, int batch, int box_
 int oz_prepare(sldqmc_ctx *c)
 {
     c->oz_ws = nullptr;
-    if (c->N < OBM) return SLDQMC_OK;  // tiles are 128 rows
+    // Below one 128-row tile only the FP64 mode's products with a propagator
+    // shared by all items (slice products, wraps), whose rows are stacked
+    const bool small = c->N < OBM;
+    if (small && c->p.prec != SLDQMC_FP64) return SLDQMC_OK;
     OzWs *w = new OzWs();
     const int N = c->N;
+    const int rows = c->cap * N < OBM ? OBM : c->cap * N;  // no fewer than a tensor-map box
     w->ldp = (N + 63) / 64 * 64;
-    w->plane_stride = (long long)c->cap * N * w->ldp;
+    w->plane_stride = (long long)rows * w->ldp;
     const size_t pbytes = (size_t)OZ_S * w->plane_stride * sizeof(__nv_bfloat16);
     const size_t ebytes = sizeof(int) * (size_t)c->cap * N;
     w->tplane_stride = (long long)c->cap * 32 * 32;
@@ -987,14 +1260,16 @@ int oz_prepare(sldqmc_ctx *c)
             return SLDQMC_ERR_CUDA;
         }
     }
-    if (!encode4(&w->mapA, w->planes, w->ldp, N, c->cap, OBM) || !encode4(&w->mapB, w->planes, w->ldp, N, c->cap, OBN) ||
-        !encode4(&w->mapRA, w->rplanes, w->ldp, N, c->cap, OBM) ||
-        !encode4(&w->mapRB, w->rplanes, w->ldp, N, c->cap, OBN) ||
-        !encode4(&w->mapT, w->tplanes, 32, 32, c->cap, OBN) ||
-        !encode4(&w->mapAS, w->planes, w->ldp, N * c->cap, 1, OBM) ||
-        !encode4(&w->mapRAS, w->rplanes, w->ldp, N * c->cap, 1, OBM) ||
-        !encode4(&w->mapL[0], w->lplanes[0], 32, N, c->cap, OBN) ||
-        !encode4(&w->mapL[1], w->lplanes[1], 32, N, c->cap, OBN)) {
+    bool mapped = encode4(&w->mapAS, w->planes, w->ldp, rows, 1, OBM) && encode4(&w->mapRAS, w->rplanes, w->ldp, rows, 1, OBM);
+    if (!small)
+        mapped = mapped && encode4(&w->mapA, w->planes, w->ldp, N, c->cap, OBM) &&
+                 encode4(&w->mapB, w->planes, w->ldp, N, c->cap, OBN) &&
+                 encode4(&w->mapRA, w->rplanes, w->ldp, N, c->cap, OBM) &&
+                 encode4(&w->mapRB, w->rplanes, w->ldp, N, c->cap, OBN) &&
+                 encode4(&w->mapT, w->tplanes, 32, 32, c->cap, OBN) &&
+                 encode4(&w->mapL[0], w->lplanes[0], 32, N, c->cap, OBN) &&
+                 encode4(&w->mapL[1], w->lplanes[1], 32, N, c->cap, OBN);
+    if (!mapped) {
         cudaFree(mem);
         delete w;
         return SLDQMC_ERR_CUDA;
@@ -1009,6 +1284,7 @@ int oz_prepare(sldqmc_ctx *c)
     cudaFuncSetAttribute(k_oz_gemm<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh);
     cudaFuncSetAttribute(k_oz_gemm<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh);
     cudaFuncSetAttribute(k_oz_gemm<false, false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh);
+    cudaFuncSetAttribute(k_oz_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CH_SMEM);
     c->oz_ws = w;
     return SLDQMC_OK;
 }
@@ -1255,7 +1531,8 @@ bool oz_e_planes(sldqmc_ctx *c)
     if (w->e_tried) return w->emem != nullptr;
     w->e_tried = 1;
     const int N = c->N;
-    w->eplane_stride = (long long)N * w->ldp;
+    const int erows = N < OBN ? OBN : N;
+    w->eplane_stride = (long long)erows * w->ldp;
     const size_t pb = (size_t)OZ_S * w->eplane_stride * sizeof(__nv_bfloat16);
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || 6.0 * (double)pb > (double)free_b ||
@@ -1268,7 +1545,7 @@ bool oz_e_planes(sldqmc_ctx *c)
     for (int e = 0; e < 2; ++e) {
         w->eplanes[e] = (__nv_bfloat16 *)((uint8_t *)w->emem + e * pb);
         w->EE[e] = (int *)((uint8_t *)w->emem + 2 * pb) + e * N;
-        if (!encode4(&w->mapE[e], w->eplanes[e], w->ldp, N, 1, OBN)) {
+        if (!encode4(&w->mapE[e], w->eplanes[e], w->ldp, erows, 1, OBN)) {
             cudaFree(w->emem);  // waits for the memset
             w->emem = nullptr;
             return false;
@@ -1404,6 +1681,33 @@ void oz_delayed_update(sldqmc_ctx *c, double *const *G, const FlipPairs *pairs, 
 }
 
 bool oz_have_e(sldqmc_ctx *c) { return c->oz_ws && oz_e_planes(c); }
+
+// A product with a propagator on the tensor cores is two launches of about
+// 5 us each at least, one of the FP64 pipe 2 N^3 B / 1.1e12 s but no less than
+// 8 us: below 128 sites (where an item fills no tile of its own) the tensor
+// cores take it from N^3 B = 8e6 (14 us of the FP64 pipe) on.  Measured at 8 x
+// 8, 64 chains, both flavours: 2 x 44 us against 10 + 15 us.
+bool oz_worth(const sldqmc_ctx *c, int B)
+{
+    return c->N >= OBM || (double)c->N * c->N * c->N * B >= 8e6;
+}
+
+bool oz_full(const sldqmc_ctx *c) { return c->oz_ws && c->N >= OBM; }
+
+bool oz_chain_fits(const sldqmc_ctx *c) { return c->N <= CH_N; }
+
+// X^T_out = U^T D_t0 E D_t0+1 E ... for nb slices (N <= 64), one launch.
+void oz_chain_block(sldqmc_ctx *c, const double *Ut, const int8_t *d_s, int B, double cu, double cd, int t0, int nb,
+                    double *Xt_out)
+{
+    OzWs *w = (OzWs *)c->oz_ws;
+    ChainArgs a{Ut, Xt_out, d_s, (long long)c->M * c->N, B * c->N, c->N, c->M, t0, nb, cu, cd, w->eplanes[0],
+                w->eplane_stride, w->ldp, w->EE[0], c->d_flag};
+    prof_begin(c, SLDQMC_KC_GEMM_OZ, 2.0 * c->N * c->N * c->N * nb * B, "oz_chain");
+    k_oz_chain<<<(a.rows + OBM - 1) / OBM, CH_THREADS, CH_SMEM, c->st>>>(a);
+    prof_end(c);
+    c->launches++;
+}
 
 // FP64-accurate slice product X^T D E for B items into Xt (which may be X
 // itself): the rows of X^T D split with their own maxima against E's planes.

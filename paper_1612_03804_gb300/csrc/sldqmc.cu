@@ -200,13 +200,17 @@ int weight_run(sldqmc_ctx *c, const int8_t *d_s, int B, int eta, int tau0, doubl
     launch_init_udv(c, Ut, c->buf[1], B);
     std::vector<int> slices;
     const bool oz = c->p.prec == SLDQMC_FP64 && c->kinetic != SLDQMC_KINETIC_SEPARABLE && oz_have_e(c);
+    const bool chain = oz && oz_chain_fits(c);
     for (int m = 0; m < M; m += c->p.n_wrap) {
         const int nb = std::min(c->p.n_wrap, M - m);
         double *Xt;
         if (c->kinetic == SLDQMC_KINETIC_SEPARABLE) {
             sep_chain_block(c, Ut, d_s, B, cu, cd, (tau0 + m) % M, nb, c->d_Einv + nn, X1);
             Xt = X1;
-        } else if (oz) {
+        } else if (chain) {
+            oz_chain_block(c, Ut, d_s, B, cu, cd, (tau0 + m) % M, nb, X1);
+            Xt = X1;
+        } else if (oz && oz_worth(c, B)) {
             for (int j = 0; j < nb; ++j)
                 oz_slice_product(c, j == 0 ? Ut : X1, d_s + (long long)((tau0 + m + j) % M) * N, cu, cd, X1, B);
             Xt = X1;
@@ -377,7 +381,7 @@ static void local_flips_slice(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s
 {
     const int N = c->N;
     double *G[2] = {Gp, Gm};
-    if (c->oz_ws) {
+    if (oz_full(c)) {
         static_assert(sizeof(FlipPairs) <= 2 * 32 * 128 * sizeof(double), "a record fits a chain's share of d_U");
         FlipPairs *pairs = reinterpret_cast<FlipPairs *>(c->d_U);
         for (int i0 = 0; i0 < N; i0 += 32) {
@@ -842,29 +846,62 @@ int sldqmc_log_bare_weight(sldqmc_ctx *c, const int8_t *s, double *log_phi)
     return SLDQMC_OK;
 }
 
-// Fresh Gt_f = E^{-1} G(tau1) E for both flavours into dst[f] (B items).
+// The twin for both flavours of a sweep's fresh Green's functions: while 2B
+// items fit in one wave of CTAs and N <= 1024, where the launches of a weight
+// are latencies rather than work; never created while the stream is being
+// captured.
+static sldqmc_ctx *fresh_twin(sldqmc_ctx *c, int B)
+{
+    if ((c->prof && c->prof->on) || 2 * B > c->num_sms || c->N > 1024) return nullptr;
+    if (!c->twin && !c->no_twin) {
+        cudaStreamCaptureStatus cs;
+        if (cudaStreamIsCapturing(c->st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return nullptr;
+        }
+    }
+    return get_twin(c);
+}
+
+// Fresh Gt_f = E^{-1} G(tau1) E for both flavours into dst[f] (B items): one
+// batch [s; -s] at eta = +1 on the twin (see get_twin), or one after the other.
 static int fresh_gt(sldqmc_ctx *c, const int8_t *d_s, int B, int tau1, double *dstp, double *dstm)
 {
     const int N = c->N;
     const long long nn = c->nn;
-    double *Gt = c->d_G[0] + 2 * (size_t)c->cap * nn;  // G(tau1) staging
-    double *T = Gt + (size_t)c->cap * nn;
+    double *Gt = c->d_G[0] + 2 * (size_t)c->cap * nn;  // staging: 2 cap items
     double *dst[2] = {dstp, dstm};
-    const bool oz = oz_have_e(c);
-    for (int f = 0; f < 2; ++f) {
-        // the tensor-core form transforms both flavours in one launch from dst itself
-        int rc = weight_run(c, d_s, B, f == 0 ? 1 : -1, tau1 % c->M, c->d_ld_tmp2, nullptr, oz ? dst[f] : Gt, 1.0, 0);
+    const double *src[2] = {Gt, Gt + (long long)B * nn};
+    sldqmc_ctx *t = fresh_twin(c, B);
+    if (t && 2 * B <= t->cap) {
+        cudaStream_t tst = t->st;
+        cudaEventRecord(c->ev_fork, c->st);
+        cudaStreamWaitEvent(tst, c->ev_fork, 0);
+        const long long n = (long long)B * c->M * N;
+        k_pair_fields<<<(int)std::min<long long>(cdiv(n, 256), 4096), 256, 0, tst>>>(d_s, t->d_s_one, n);
+        t->launches++;
+        int rc = weight_run(t, t->d_s_one, 2 * B, 1, tau1 % c->M, t->d_ld_tmp, nullptr, Gt, 1.0, 0);
         if (rc) return rc;
-        if (oz) continue;
-        GemmF64 g = gemm_desc(N, N, N, c->d_Einv, N, 0, Gt, N, nn, T, N, nn, B);
+        cudaEventRecord(c->ev_join, tst);
+        cudaStreamWaitEvent(c->st, c->ev_join, 0);
+    } else {
+        for (int f = 0; f < 2; ++f) {
+            int rc = weight_run(c, d_s, B, f == 0 ? 1 : -1, tau1 % c->M, c->d_ld_tmp2, nullptr, const_cast<double *>(src[f]),
+                                1.0, 0);
+            if (rc) return rc;
+        }
+    }
+    if (oz_have_e(c) && oz_worth(c, 2 * B)) {
+        double *Tt[2] = {Gt, Gt + (long long)B * nn};  // in place: the products read digit planes
+        oz_similarity(c, src, Tt, dst, 1, nullptr, nullptr, B);
+        return SLDQMC_OK;
+    }
+    for (int f = 0; f < 2; ++f) {
+        double *T = f == 0 ? dst[1] : Gt;  // free by then
+        GemmF64 g = gemm_desc(N, N, N, c->d_Einv, N, 0, src[f], N, nn, T, N, nn, B);
         gemm_ctx(c, g, false, false);
         GemmF64 h = gemm_desc(N, N, N, T, N, nn, c->d_E, N, 0, dst[f], N, nn, B);
         gemm_ctx(c, h, false, false);
-    }
-    if (oz) {
-        double *Tt[2] = {Gt, T};
-        const double *src[2] = {dstp, dstm};
-        oz_similarity(c, src, Tt, dst, 1, nullptr, nullptr, B);
     }
     return SLDQMC_OK;
 }
@@ -877,7 +914,7 @@ static void wrap_gt(sldqmc_ctx *c, const int8_t *d_s, int B, int tau, double *sr
     const long long nn = c->nn;
     double *T = c->d_G[0] + 3 * (size_t)c->cap * nn;
     double *src[2] = {srcp, srcm}, *dst[2] = {dstp, dstm};
-    if (oz_have_e(c)) {
+    if (oz_have_e(c) && oz_worth(c, 2 * B)) {
         double *Tt[2] = {T - (size_t)c->cap * nn, T};
         oz_similarity(c, src, Tt, dst, 0, d_s + (long long)tau * N, c->ex_scale, B);
         return;
@@ -1351,7 +1388,7 @@ int sldqmc_gram_batch_dev(sldqmc_ctx *c, const double *d_X, int B, double *d_W)
 {
     if (!c || !d_X || !d_W || B < 1 || B > c->cap) return SLDQMC_ERR_ARG;
     const int N = c->N;
-    if (c->oz_ws && c->p.prec != SLDQMC_FP64) {
+    if (oz_full(c) && c->p.prec != SLDQMC_FP64) {
         oz_gram(c, d_X, c->nn, d_W, c->nn, N, B);
     } else {
         GemmF64 g = gemm_desc(N, N, N, d_X, N, c->nn, d_X, N, c->nn, d_W, N, c->nn, B);

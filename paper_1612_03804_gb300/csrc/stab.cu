@@ -117,13 +117,15 @@ __global__ void k_gather_pivot(const double *W, long long sW, const double *Xt, 
 }
 
 // One block row of the stacked Cholesky-QR on the FP64 pipe: factor the kb x
-// kb diagonal block W_kk = R_kk^T R_kk and T = R_kk^-T (in shared memory, every
-// CTA redundantly), then T times the panel's columns: W-columns right of the
-// block give R's block row, Y-columns give Q^T's block row (in place).  A CTA
-// has 32 columns (lanes), its four warps every fourth row each: a warp's FMA
-// holds its sub-partition's FP64 pipe for 64 cycles, so a column's 528 FMAs
-// are spread over all four (4.4 us); one thread per column took 17 us of the
-// same pipe and two columns per thread 35 us, beside a factor of 45 us.
+// kb diagonal block W_kk = R_kk^T R_kk (in shared memory, every CTA
+// redundantly), then solve R_kk^T y = w for the panel's columns: W-columns right
+// of the block give R's block row, Y-columns give Q^T's block row (in place).
+// A CTA has 32 columns (lanes), its four warps every fourth row each: a warp's
+// FMA holds its sub-partition's FP64 pipe for 64 cycles, so a column's 528 FMAs
+// are spread over all four (4.4 us, a barrier per row); one thread per column
+// took 17 us of the same pipe and two columns per thread 35 us, beside a factor
+// of 45 us.  The solves substitute: a product with the factor's inverse, no
+// faster here, leaves a residual larger by the block's condition number.
 __global__ void __launch_bounds__(128) k_chol_panel(const double *W, long long sW, int ldw, double *Y, long long sY,
                                                     double *R, long long sR, int N, int k0, int kb, int *flag)
 {
@@ -153,14 +155,20 @@ __global__ void __launch_bounds__(128) k_chol_panel(const double *W, long long s
             if (r < kb && c < kb) Rb[(long long)(k0 + r) * N + k0 + c] = c > r ? X[r][c] : (c == r ? root[r] : 0.0);
         }
     double *dst = isW ? Rb : Y + (long long)b * sY;
-    double acc[8];
+    double acc[8];  // rows 4 q + wid
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q] = 0.0;
-    for (int l = 0; l < kb; ++l) {
+    for (int q = 0; q < 8; ++q) acc[q] = V[4 * q + wid][lane];
+#pragma unroll
+    for (int l = 0; l < 32; ++l) {
+        if ((l & 3) == wid) {
+            acc[l >> 2] *= X[l][l];  // 1 / R_ll
+            V[l][lane] = acc[l >> 2];
+        }
+        __syncthreads();
         const double v = V[l][lane];
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (4 * q + wid >= l) acc[q] += X[4 * q + wid][l] * v;
+        for (int q = l >> 2; q < 8; ++q)
+            if (4 * q + wid > l) acc[q] -= X[l][4 * q + wid] * v;
     }
     if (!live) return;
 #pragma unroll
@@ -809,7 +817,7 @@ static void chol_pass(sldqmc_ctx *c, double *W, long long sW, double *Y, double 
     // diagonal block's factor (all FP64-accurate digit splitting), and that
     // product also splits the finished rows for the later panels.  Otherwise
     // right-looking with FP64 panels and trailing updates.
-    const bool oz = c->oz_ws != nullptr;
+    const bool oz = oz_full(c);
     if (oz) {
         // blocks of CHOL_BLOCK rows: one update of the block's rows with every
         // earlier row (CHOL_BLOCK output columns: CHOL_BLOCK / 32 times the tiles
@@ -867,7 +875,7 @@ void stabilize(sldqmc_ctx *c, double *Xt, double *Wc, double *Y, int B, int pass
     double *W = c->buf[4];
     double *R1 = c->buf[6], *R2 = c->buf[7], *Vg = c->buf[8], *V = c->buf[1];
     // W = Xt Xt^T (upper triangle): FP64, or FP64-accurate on the tensor cores
-    if (c->oz_ws) {
+    if (oz_full(c)) {
         oz_gram(c, Xt, nn, W, 2 * nn, N, B);
     } else {
         GemmF64 g = gemm_desc(N, N, N, Xt, N, nn, Xt, N, nn, W, N, 2 * nn, B);
@@ -889,7 +897,7 @@ void stabilize(sldqmc_ctx *c, double *Xt, double *Wc, double *Y, int B, int pass
     const double *R = R1;
     if (passes == 2) {
         // second pass: W = Q1^T Q1 (as Y Y^T), upper triangle; Q = Q1 R2^{-1}, R = R2 R1
-        if (c->oz_ws) {
+        if (oz_full(c)) {
             oz_keep_bounds(c, B);
             oz_gram(c, Y, nn, W, 2 * nn, N, B);
         } else {
@@ -898,7 +906,7 @@ void stabilize(sldqmc_ctx *c, double *Xt, double *Wc, double *Y, int B, int pass
             gemm_ctx(c, g2, false, true);
         }
         chol_pass(c, W, 2 * nn, Y, R2, B);
-        if (c->oz_ws) {
+        if (oz_full(c)) {
             oz_r2r1(c, R2, R1, Xt, B);
         } else {
             GemmF64 g3 = gemm_desc(N, N, N, R2, N, nn, R1, N, nn, Xt, N, nn, B);
@@ -913,7 +921,7 @@ void stabilize(sldqmc_ctx *c, double *Xt, double *Wc, double *Y, int B, int pass
     k_new_D<<<gd, 256, 0, c->st>>>(R, nn, N, c->d_Dp, c->d_D, c->d_flag);
     prof_end(c);
     c->launches++;
-    if (c->oz_ws) {
+    if (oz_full(c)) {
         // V = (D^{-1} R D_p) P^T V, FP64-accurate on the tensor cores
         oz_update_V(c, R, V, Vg, B);
         return;
@@ -977,7 +985,7 @@ void finalize(sldqmc_ctx *c, const double *Ut, int B, double *d_ld, int *d_sign,
             prof_end(c);
             c->launches++;
             int m2 = N - (k0 + kb);
-            if (m2 > 0 && c->oz_ws) {
+            if (m2 > 0 && oz_full(c)) {
                 oz_lu_update(c, A, sItem, lda, k0, kb, B, rhs);
             } else if (m2 > 0) {
                 GemmF64 g = gemm_desc(m2, rest, kb, A + (long long)(k0 + kb) * lda + k0, lda, sItem,
@@ -998,7 +1006,7 @@ void finalize(sldqmc_ctx *c, const double *Ut, int B, double *d_ld, int *d_sign,
             k_trsm_upper_rhs<32><<<gt, 128, 0, c->st>>>(A, sItem, lda, N, k0, kb);
             prof_end(c);
             c->launches++;
-            if (k0 > 0 && c->oz_ws) {
+            if (k0 > 0 && oz_full(c)) {
                 oz_back_update(c, A, sItem, lda, k0, kb, B);
             } else if (k0 > 0) {
                 GemmF64 g = gemm_desc(k0, N, kb, A + k0, lda, sItem, A + (long long)k0 * lda + N, lda,

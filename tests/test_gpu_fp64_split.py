@@ -71,3 +71,50 @@ def test_fp64_local_sweep(Lx, Ly, rank):
         assert stats[b]["margin_events"] == 0
         np.testing.assert_array_equal(out[b], so)
         assert stats[b]["max_drift"] < TOL
+
+
+# Up to 64 sites the slice products of a block run in one launch of 128-row
+# CTAs; from there to 127 sites per slice, and wraps at all sizes, once there is
+# enough work.  Sizes: one column group and its edges (16, 17 sites), a ragged
+# last group (49, 63), exactly 64; rows that end inside a CTA and inside an
+# item; one and several CTAs; 81 sites on either side of the rule's line.
+@pytest.mark.parametrize("Lx,Ly,B", [(2, 2, 3), (4, 4, 1), (17, 1, 9), (7, 7, 3), (9, 7, 5), (8, 8, 1), (8, 8, 35),
+                                     (9, 9, 2), (9, 9, 40)])
+def test_fp64_small_weight_and_green(Lx, Ly, B):
+    import torch
+    from oracle import oracle as O
+    from paper_1612_03804_gb300 import sldqmc
+    M, N = 13, Lx * Ly
+    m = _model(Lx, Ly, M)
+    s = batch_uniform(140 + N, B, M, N)
+    with sldqmc.Context(Lx, Ly, mu=-0.5, xi=1.0, beta=M * 0.1, dtau=0.1, n_wrap=5, max_batch=B) as ctx:
+        d_s = torch.from_numpy(s).cuda()
+        ld = torch.zeros(B, dtype=torch.float64, device="cuda")
+        sg = torch.zeros(B, dtype=torch.int32, device="cuda")
+        G = torch.zeros((B, N, N), dtype=torch.float64, device="cuda")
+        ctx.green_batch_dev(d_s, 1, 9, G, ld, sg)
+        ctx.sync()
+        for b in sorted({0, 1 % B, B // 2, B - 1}):
+            ref, rs, Gr = O.weight(m, s[b], 1, tau0=9, want_G=True)
+            assert int(sg[b]) == rs
+            assert abs(float(ld[b]) - ref) <= TOL * max(1.0, abs(ref))
+            assert np.abs(G[b].cpu().numpy() - Gr).max() < TOL
+
+
+@pytest.mark.parametrize("Lx,Ly,B", [(4, 4, 3), (9, 7, 2), (8, 8, 40), (9, 9, 12), (8, 8, 80)])
+def test_fp64_small_local_sweep(Lx, Ly, B):
+    from oracle import oracle as O
+    from paper_1612_03804_gb300 import sldqmc
+    import torch
+    M, N = 7, Lx * Ly
+    m = _model(Lx, Ly, M)
+    s = batch_uniform(160 + N, B, M, N)
+    with sldqmc.Context(Lx, Ly, mu=-0.5, xi=1.0, beta=M * 0.1, dtau=0.1, n_wrap=5, max_batch=B) as ctx:
+        d_s = torch.from_numpy(s).cuda()
+        stats = ctx.local_sweep_batch_dev(d_s, 71, 0, 1)
+        out = d_s.cpu().numpy()
+    for b in sorted({0, 1, B - 1}):
+        so, st = O.local_sweep(m, s[b], 71 + (b << 32), 0, 1)
+        assert stats[b]["margin_events"] == 0
+        np.testing.assert_array_equal(out[b], so)
+        assert stats[b]["max_drift"] < TOL
