@@ -164,7 +164,8 @@ int sldqmc_local_sweep_batch_dev(sldqmc_ctx *ctx, int8_t *d_s, int B, uint64_t s
  * those of k = 1; only the rounding of the Green's function differs (the
  * decisions agree outside the 1e-8 margin).  From 128 sites on the library
  * takes blocks of 32 sites whatever k (unless their workspace would take more
- * than a third of the free device memory). */
+ * than a third of the free device memory), and up to 111 sites, where both
+ * Green's functions fit shared memory, immediate updates. */
 int sldqmc_set_local_update_rank(sldqmc_ctx *ctx, int k);
 
 /* Effective model (Eq. 2): H_eff = E0 + sum_c J_c f_c(C),

@@ -115,81 +115,150 @@ struct LocalArgs {
     long long *stats;  // per chain: accepted, proposed, margin
 };
 
+// The decision of one site: logr = -2 s (dtau J nsp + Kt ntm) + 2 log|R_+| +
+// 2 log|R_-|, accepted iff log u < logr, R_f = 1 + Delta_f (1 - G_f[i][i]).  Taken
+// in FP32 where it is clear by a thousandth and ten times the FP32 rounding of
+// its terms; otherwise by the FP64 expression, whose two logarithms are some
+// eighty instructions of the FP64 pipe at 64 cycles a warp each.
+struct FlipDecision {
+    bool acc, margin;
+    double R[2];
+};
+
+__device__ __forceinline__ FlipDecision flip_decide(const LocalArgs &a, double gp, double gm, const double (*dls)[2], int sold,
+                                                    int nsp, int ntm, double lu)
+{
+    FlipDecision o;
+    o.R[0] = __dadd_rn(1.0, __dmul_rn(dls[0][sold > 0], __dadd_rn(1.0, -gp)));
+    o.R[1] = __dadd_rn(1.0, __dmul_rn(dls[1][sold > 0], __dadd_rn(1.0, -gm)));
+    const float r0 = fabsf((float)o.R[0]), r1 = fabsf((float)o.R[1]), luf = (float)lu;
+    const float l0 = 2.0f * logf(r0), l1 = 2.0f * logf(r1);
+    const float st = -2.0f * (float)sold * ((float)a.dtauJ * (float)nsp + (float)a.Kt * (float)ntm);
+    const float d = st + l0 + l1 - luf;
+    o.acc = d > 0.0f;
+    o.margin = false;
+    if (!(fabsf(d) > 1e-3f + 1e-5f * (fabsf(st) + fabsf(l0) + fabsf(l1) + fabsf(luf))) || !(r0 > 1e-30f && r0 < 1e30f) ||
+        !(r1 > 1e-30f && r1 < 1e30f)) {
+        double logr = __dmul_rn(-2.0 * (double)sold,
+                                __dadd_rn(__dmul_rn(a.dtauJ, (double)nsp), __dmul_rn(a.Kt, (double)ntm)));
+        logr = __dadd_rn(logr, __dmul_rn(2.0, log(fabs(o.R[0]))));
+        logr = __dadd_rn(logr, __dmul_rn(2.0, log(fabs(o.R[1]))));
+        o.margin = fabs(logr - lu) <= MARGIN;
+        o.acc = lu < logr;
+    }
+    return o;
+}
+
+// Delta_f / R_f of the site decided by lane `hit`, one flavour per lane (warp-wide).
+__device__ __forceinline__ void flip_coef(const FlipDecision &d, int sold, int hit, const double (*dls)[2], double *cp,
+                                          double *cm)
+{
+    const int lane = threadIdx.x & 31;
+    const double rp = __shfl_sync(0xffffffffu, d.R[0], hit), rm = __shfl_sync(0xffffffffu, d.R[1], hit);
+    const int so = __shfl_sync(0xffffffffu, sold, hit);
+    if (lane < 2) *(lane ? cm : cp) = dls[lane][so > 0] / (lane ? rm : rp);
+}
+
+// Between two accepted flips nothing a decision depends on changes, so warp 0
+// decides up to 32 sites at once, one per lane: the lowest accepted one is the
+// next flip, the sites before it are rejected, those after it are decided
+// again.  SMEM: both Green's functions stay in shared memory (row stride N + 1)
+// for the slice; otherwise they are updated in global memory.  An accepted flip
+// is 2 N^2 FMAs of this SM's FP64 pipe (2.1 us at N = 64), spread over all
+// threads element by element.
+// Measured, 8 x 8, 64 chains, a fifth of the flips accepted: 322 us per slice
+// when every site was decided in FP64 in turn, 94 now.
+template <bool SMEM>
 __global__ void __launch_bounds__(512) k_local_flips(LocalArgs a)
 {
     const int b = blockIdx.x;
-    const int N = a.Lx * a.Ly;
-    double *G[2] = {a.Gp + (long long)b * a.nn, a.Gm + (long long)b * a.nn};
+    const int N = a.Lx * a.Ly, tid = threadIdx.x, lane = tid & 31;
+    const int ld = SMEM ? N + 1 : N;
     int8_t *s = a.s + (long long)b * a.M * N;
     extern __shared__ double sh[];
-    double *col = sh;           // 2N
-    double *row = sh + 2 * N;   // 2N
+    double *col = sh;           // 2N: coef * G[:, i]
+    double *row = sh + 2 * N;   // 2N: e_i - G[i, :]
     double *lus = sh + 4 * N;   // N: log u of every site of the slice
+    double *gG[2] = {a.Gp + (long long)b * a.nn, a.Gm + (long long)b * a.nn};
+    double *G[2] = {SMEM ? sh + 5 * N : gG[0], SMEM ? sh + 5 * N + (long long)N * ld : gG[1]};
+    // the slice's spins, and the sums of their neighbours in time
+    int8_t *sp = SMEM ? reinterpret_cast<int8_t *>(sh + 5 * N + 2LL * N * ld) : s + (long long)a.tau * N, *nt = sp + N;
     __shared__ double coef[2], dls[2][2];
-    __shared__ int accept;
+    __shared__ int s_hit;
     const uint64_t seed = a.seed + ((uint64_t)b << 32);
-    long long n_acc = 0, n_mg = 0;
-    const int tau = a.tau;
+    const int tau = a.tau, nn = N * N;
+    if (SMEM) {
+        for (int e = tid; e < 2 * nn; e += blockDim.x) {
+            const int f = e >= nn, q = e - f * nn, r = q / N;
+            G[f][r * ld + (q - r * N)] = gG[f][q];
+        }
+        for (int i = tid; i < N; i += blockDim.x) {
+            sp[i] = s[tau * N + i];
+            nt[i] = (int8_t)(s[wrapi(tau + 1, a.M) * N + i] + s[wrapi(tau - 1, a.M) * N + i]);
+        }
+    }
     // off the serial chain: the uniforms of all sites, and Delta_f for both field values
-    for (int i = threadIdx.x; i < N; i += blockDim.x)
+    for (int i = tid; i < N; i += blockDim.x)
         lus[i] = log(philox_uniform(seed, (uint32_t)i, (uint32_t)tau, a.sweep, PURPOSE_LOCAL));
-    if (threadIdx.x < 4) {
-        const int f = threadIdx.x >> 1, sp = threadIdx.x & 1;
-        const double eta = f == 0 ? 1.0 : -1.0;
-        dls[f][sp] = exp(-2.0 * eta * a.dtxi * (sp ? 1.0 : -1.0)) - 1.0;
+    if (tid < 4) {
+        const int f = tid >> 1, sp = tid & 1;
+        dls[f][sp] = exp(-2.0 * (f == 0 ? 1.0 : -1.0) * a.dtxi * (sp ? 1.0 : -1.0)) - 1.0;
     }
     __syncthreads();
-    for (int i = 0; i < N; ++i) {
-        if (threadIdx.x == 0) {
-            const int sold = s[tau * N + i];
-            const int x = i % a.Lx, y = i / a.Lx;
-            int nsp = 0;
-            if (a.Lx > 1) nsp += s[tau * N + wrapi(x + 1, a.Lx) + a.Lx * y] + s[tau * N + wrapi(x - 1, a.Lx) + a.Lx * y];
-            if (a.Ly > 1) nsp += s[tau * N + x + a.Lx * wrapi(y + 1, a.Ly)] + s[tau * N + x + a.Lx * wrapi(y - 1, a.Ly)];
-            const int ntm = s[wrapi(tau + 1, a.M) * N + i] + s[wrapi(tau - 1, a.M) * N + i];
-            double logr = __dmul_rn(-2.0 * (double)sold,
-                                    __dadd_rn(__dmul_rn(a.dtauJ, (double)nsp), __dmul_rn(a.Kt, (double)ntm)));
-            double R[2], Dl[2];
-            for (int f = 0; f < 2; ++f) {
-                Dl[f] = dls[f][sold > 0];
-                R[f] = __dadd_rn(1.0, __dmul_rn(Dl[f], __dadd_rn(1.0, -G[f][(long long)i * N + i])));
-                logr = __dadd_rn(logr, __dmul_rn(2.0, log(fabs(R[f]))));
+    int q = 0, n_acc = 0, n_mg = 0;  // warp 0: the next site to decide
+    for (;;) {
+        if (tid < 32) {
+            int hit = N;
+            while (q < N && hit == N) {
+                const int i = q + lane;
+                FlipDecision d{false, false, {1.0, 1.0}};
+                int sold = 1;
+                if (i < N) {
+                    sold = sp[i];
+                    const int y = i / a.Lx, x = i - y * a.Lx;
+                    int nsp = 0;
+                    if (a.Lx > 1) nsp += sp[x + 1 < a.Lx ? i + 1 : i + 1 - a.Lx] + sp[x > 0 ? i - 1 : i - 1 + a.Lx];
+                    if (a.Ly > 1) nsp += sp[y + 1 < a.Ly ? i + a.Lx : x] + sp[y > 0 ? i - a.Lx : i - a.Lx + N];
+                    const int ntm = SMEM ? nt[i] : s[wrapi(tau + 1, a.M) * N + i] + s[wrapi(tau - 1, a.M) * N + i];
+                    d = flip_decide(a, G[0][(long long)i * ld + i], G[1][(long long)i * ld + i], dls, sold, nsp, ntm, lus[i]);
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, d.acc);
+                const int first = m ? __ffs(m) - 1 : 32;  // lanes up to it are decided
+                n_mg += __popc(__ballot_sync(0xffffffffu, d.margin && lane <= first));
+                if (m) {
+                    hit = q + first;
+                    flip_coef(d, sold, first, dls, coef, coef + 1);
+                    if (lane == first) sp[i] = (int8_t)(-sold);
+                    __syncwarp();
+                    n_acc++;
+                }
+                q += first + 1 < 32 ? first + 1 : 32;
             }
-            const double lu = lus[i];
-            if (fabs(logr - lu) <= MARGIN) n_mg++;
-            const int acc = lu < logr;
-            accept = acc;
-            if (acc) {
-                coef[0] = Dl[0] / R[0];
-                coef[1] = Dl[1] / R[1];
-                s[tau * N + i] = (int8_t)(-sold);
-                n_acc++;
-            }
+            if (lane == 0) s_hit = hit;
         }
         __syncthreads();
-        const int acc_i = accept;
-        __syncthreads();  // every thread has read the decision before thread 0 writes the next
-        if (acc_i) {
-            for (int e = threadIdx.x; e < 2 * N; e += blockDim.x) {
-                const int f = e / N, k = e % N;
-                col[e] = G[f][(long long)k * N + i];
-                row[e] = (k == i ? 1.0 : 0.0) - G[f][(long long)i * N + k];
-            }
-            __syncthreads();
-            // warp w takes rows w, w + nwarps, ...; its lanes walk the row's
-            // columns (coalesced, no index division)
-            const int nwarps = blockDim.x >> 5, wl = threadIdx.x & 31;
-            for (int fr = threadIdx.x >> 5; fr < 2 * N; fr += nwarps) {
-                const int f = fr >= N, rr = fr - f * N;
-                const double cf = coef[f] * col[f * N + rr];
-                double *g = G[f] + (long long)rr * N;
-                const double *rw = row + f * N;
-                for (int k = wl; k < N; k += 32) g[k] -= cf * rw[k];
-            }
-            __syncthreads();
+        const int i = s_hit;
+        if (i >= N) break;
+        for (int e = tid; e < 2 * N; e += blockDim.x) {
+            const int f = e >= N, k = e - f * N;
+            col[e] = coef[f] * G[f][(long long)k * ld + i];
+            row[e] = (k == i ? 1.0 : 0.0) - G[f][(long long)i * ld + k];
         }
+        __syncthreads();
+        for (int e = tid; e < 2 * nn; e += blockDim.x) {
+            const int f = e >= nn, p = e - f * nn, r = p / N, k = p - r * N;
+            G[f][(long long)r * ld + k] -= col[f * N + r] * row[f * N + k];
+        }
+        __syncthreads();
     }
-    if (threadIdx.x == 0) {
+    if (SMEM) {
+        for (int e = tid; e < 2 * nn; e += blockDim.x) {
+            const int f = e >= nn, p = e - f * nn, r = p / N;
+            gG[f][p] = G[f][r * ld + (p - r * N)];
+        }
+        for (int i = tid; i < N; i += blockDim.x) s[tau * N + i] = sp[i];
+    }
+    if (tid == 0) {
         a.stats[b * 4 + 0] += n_acc;
         a.stats[b * 4 + 1] += N;
         a.stats[b * 4 + 2] += n_mg;
@@ -327,13 +396,11 @@ __global__ void __launch_bounds__(512) k_local_flips_delayed(DelayArgs d)
 // i0..i0+ns-1, so the block's serial chain runs on those alone, in shared
 // memory, and what the accepted flips do to the other rows and columns is
 // formed afterwards on all SMs (k_flip_pairs and a rank-32 product,
-// oz_gram.cu).  One CTA per chain.  Warp 0 walks the sites up to the next
-// accepted one; then all warps subtract its pair from the rows still to
-// come.  The chain is bound by the latency of dependent FP64 operations, of
-// which the two logarithms of a decision were most: the decision is taken in
-// FP32 where it is clear by a thousandth (its rounding is below 1e-5 of the
-// terms), and otherwise, and near the margin, by the FP64 expression.
-// A block of 32 sites of 8 chains at N = 576: 29 us, and 29 us for the pairs;
+// oz_gram.cu).  One CTA per chain.  Warp 0 decides all sites still to come at
+// once (see k_local_flips); then all warps subtract the accepted one's pair from
+// the rows below.  Bound by the latency of dependent FP64 operations per
+// accepted flip.
+// A block of 32 sites of 8 chains at N = 576: 25 us, and 23 us for the pairs;
 // 247 us when every pair was formed for all rows and columns inside the chain,
 // and 651 us per 32 sites of 16 chains at N = 256 with immediate updates on one
 // SM per chain (2 N^2 FMAs of the FP64 pipe per accepted flip and flavour).
@@ -370,42 +437,16 @@ __global__ void __launch_bounds__(256) k_flip_block(LocalArgs a, FlipPairs *out,
         dls[f][sp] = exp(-2.0 * (f == 0 ? 1.0 : -1.0) * a.dtxi * (sp ? 1.0 : -1.0)) - 1.0;
     }
     __syncthreads();
-    long long n_mg = 0;
-    int q = 0, n = 0;
+    int n_mg = 0, q = 0, n = 0;
     for (;;) {
         if (wid == 0) {
-            int hit = ns;
-            for (; q < ns; ++q) {
-                const int f = lane & 1;  // flavour f on the lanes of its parity
-                const int so = __shfl_sync(0xffffffffu, sold, q);
-                const int np = __shfl_sync(0xffffffffu, nsp, q), nt = __shfl_sync(0xffffffffu, ntm, q);
-                const double Dl = dls[f][so > 0];
-                const double R = __dadd_rn(1.0, __dmul_rn(Dl, __dadd_rn(1.0, -g[f][q][q])));
-                const double lu = lus[q];
-                const float Rf = fabsf((float)R), luf = (float)lu;
-                const float lr = 2.0f * logf(Rf);
-                const float st = -2.0f * (float)so * ((float)a.dtauJ * (float)np + (float)a.Kt * (float)nt);
-                const float lro = __shfl_xor_sync(0xffffffffu, lr, 1);
-                const float d = st + lr + lro - luf;
-                bool clear = fabsf(d) > 1e-3f + 1e-5f * (fabsf(st) + fabsf(lr) + fabsf(lro) + fabsf(luf)) &&
-                             Rf > 1e-30f && Rf < 1e30f;
-                clear = __all_sync(0xffffffffu, clear);
-                bool acc = d > 0.0f;
-                if (!clear) {
-                    const double lR = log(fabs(R)), lRo = __shfl_xor_sync(0xffffffffu, lR, 1);
-                    double logr = __dmul_rn(-2.0 * (double)so,
-                                            __dadd_rn(__dmul_rn(a.dtauJ, (double)np), __dmul_rn(a.Kt, (double)nt)));
-                    logr = __dadd_rn(logr, __dmul_rn(2.0, f ? lRo : lR));
-                    logr = __dadd_rn(logr, __dmul_rn(2.0, f ? lR : lRo));
-                    if (fabs(logr - lu) <= MARGIN) n_mg++;
-                    acc = lu < logr;
-                }
-                if (acc) {
-                    if (lane < 2) coef[f][n] = Dl / R;
-                    hit = q;
-                    break;
-                }
-            }
+            // all sites from q on at once: the lowest accepted one is the next flip
+            FlipDecision d{false, false, {1.0, 1.0}};
+            if (lane >= q && lane < ns) d = flip_decide(a, g[0][lane][lane], g[1][lane][lane], dls, sold, nsp, ntm, lus[lane]);
+            const unsigned m = __ballot_sync(0xffffffffu, d.acc);
+            const int hit = m ? __ffs(m) - 1 : ns;
+            n_mg += __popc(__ballot_sync(0xffffffffu, d.margin && lane <= hit));
+            if (m) flip_coef(d, sold, hit, dls, &coef[0][n], &coef[1][n]);
             if (lane == 0) {
                 s_q = hit;
                 if (hit < ns) sites[n] = hit;
@@ -793,6 +834,10 @@ void launch_log_bare(sldqmc_ctx *c, const int8_t *d_s, int B, double *out, int a
     c->launches++;
 }
 
+// Both Green's functions and the vectors of a slice within 200 KB (N <= 111).
+static size_t resident_bytes(int N) { return sizeof(double) * ((size_t)5 * N + (size_t)2 * N * (N + 1)) + 2 * (size_t)N; }
+bool local_flips_resident(int N) { return resident_bytes(N) <= 200 * 1024; }
+
 void launch_local_flips(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s, int B, int tau,
                         uint32_t sweep, uint64_t seed, long long *stats)
 {
@@ -803,7 +848,8 @@ void launch_local_flips(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s, int 
     size_t sh = sizeof(double) * 5 * (size_t)c->N;
     int nt = c->N * c->N >= 512 ? 512 : 256;
     prof_begin(c, SLDQMC_KC_LOCAL, 0.0, "local_flips");
-    k_local_flips<<<B, nt, sh, c->st>>>(a);
+    if (local_flips_resident(c->N)) k_local_flips<true><<<B, nt, resident_bytes(c->N), c->st>>>(a);
+    else k_local_flips<false><<<B, nt, sh, c->st>>>(a);
     prof_end(c);
     c->launches++;
 }
@@ -891,7 +937,8 @@ void launch_step_advance(sldqmc_ctx *c, uint32_t *d_step)
 void set_eff_smem_limits()
 {
     cudaFuncSetAttribute(k_eff_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_local_flips, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_local_flips<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_local_flips<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
 }  // namespace sldqmc

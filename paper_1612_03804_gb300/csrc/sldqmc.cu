@@ -25,6 +25,7 @@ void launch_check_field(sldqmc_ctx *c, const int8_t *d_s, long long n);
 void launch_log_bare(sldqmc_ctx *c, const int8_t *d_s, int B, double *out, int accumulate);
 void launch_local_flips(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s, int B, int tau,
                         uint32_t sweep, uint64_t seed, long long *stats);
+bool local_flips_resident(int N);
 void launch_drift(sldqmc_ctx *c, const double *Gw, const double *Gf, int B2x, int B, long long *stats);
 void launch_local_flips_delayed(sldqmc_ctx *c, double *Gp, double *Gm, double *U, double *V, int8_t *d_s, int B,
                                 int tau, int i0, int ns, uint32_t sweep, uint64_t seed, long long *stats);
@@ -373,7 +374,8 @@ int ensure_local_buffers(sldqmc_ctx *c)
 // The flips of slice tau.  From 128 sites on, blocks of 32 sites whatever
 // local_rank says: the decisions on the block's own rows and columns, then the
 // rank-32 correction of both flavours on the tensor cores.  Below: one launch
-// of immediate rank-1 updates, or blocks of local_rank sites whose pending
+// of immediate rank-1 updates, always where the Green's functions fit shared
+// memory (8 x 8, 64 chains: a third of the time of blocks of 32), or blocks of local_rank sites whose pending
 // corrections G -= U V are applied by one batched GEMM per flavour after each
 // block.
 static void local_flips_slice(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s, int B, int tau, uint32_t sweep,
@@ -390,7 +392,7 @@ static void local_flips_slice(sldqmc_ctx *c, double *Gp, double *Gm, int8_t *d_s
         }
         return;
     }
-    if (c->local_rank <= 1) {
+    if (c->local_rank <= 1 || local_flips_resident(N)) {
         launch_local_flips(c, Gp, Gm, d_s, B, tau, sweep, seed, c->d_stats);
         return;
     }
