@@ -43,8 +43,9 @@ __device__ __forceinline__ void chol32_finalise(double (*X)[33], double *root, i
 }
 
 // W = R^T R of the block W (X[r][c], c >= r; X[r][c] = 0 below the diagonal;
-// rows and columns kb..31 the identity), by all warps of the CTA.  On return
-// X holds R above the diagonal and T = R^-T on and below it, root[j] = R_jj.
+// rows and columns kb..31 the identity, which stay as they are), by all warps
+// of the CTA.  On return X holds R above the diagonal and T = R^-T on and below
+// it, root[j] = R_jj (j < kb).
 // Right-looking, with R's and T's rows (T by forward substitution of R^T T =
 // 1) in one array: at step j row r > j loses X[j][r] times row j in the lanes
 // c >= r (R) and c <= j (T), one FMA per row.  Warp 0 updates row j + 1 and
@@ -58,7 +59,7 @@ __device__ __forceinline__ void chol32(double (*X)[33], double *root, int kb, in
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (wid == 0) chol32_finalise(X, root, 0, lane, X[0][lane], kb, flag);
     __syncthreads();
-    for (int j = 0; j < 31; ++j) {
+    for (int j = 0; j < kb - 1; ++j) {
         if (wid == 0) {
             const int r = j + 1;
             double v = X[r][lane];
@@ -67,13 +68,13 @@ __device__ __forceinline__ void chol32(double (*X)[33], double *root, int kb, in
             chol32_finalise(X, root, r, lane, v, kb, flag);
         } else {
             const double xj = X[j][lane];
-            for (int r = j + 1 + wid; r < 32; r += nw - 1)
+            for (int r = j + 1 + wid; r < kb; r += nw - 1)
                 if (lane >= r || lane <= j) X[r][lane] -= X[j][r] * xj;
         }
         __syncthreads();
     }
     // R_jj = d y
-    if (threadIdx.x < 32) root[threadIdx.x] *= X[threadIdx.x][threadIdx.x];
+    if (threadIdx.x < kb) root[threadIdx.x] *= X[threadIdx.x][threadIdx.x];
     __syncthreads();
 }
 

@@ -94,11 +94,11 @@ void oz_delayed_update(sldqmc_ctx *c, double *const *G, const FlipPairs *pairs, 
 // sk); oz_similarity: dst_f = P src_f P^-1 of both flavours, P = E or, with
 // inv, E^-1, rows and columns then scaled by d_i / d_j of the field slice s
 // (null: no scaling), T_f an N x N scratch per item.
-// oz_worth: whether they are the faster way for B items; oz_full: every
+// oz_worth: whether they are the faster way for `times` plan_cap items; oz_full: every
 // product of the context runs there (N >= 128).  oz_chain_block: the slice
 // products of a whole block in one launch (oz_chain_fits: N <= 64).
 bool oz_have_e(sldqmc_ctx *c);
-bool oz_worth(const sldqmc_ctx *c, int B);
+bool oz_worth(const sldqmc_ctx *c, int times);
 bool oz_full(const sldqmc_ctx *c);
 bool oz_chain_fits(const sldqmc_ctx *c);
 void oz_chain_block(sldqmc_ctx *c, const double *Ut, const int8_t *d_s, int B, double cu, double cd, int t0, int nb,
@@ -114,6 +114,12 @@ void oz_keep_bounds(sldqmc_ctx *c, int B);
 // triangular; D, D_p, P from the context; Ts an N x N FP64 scratch per item).
 void oz_update_V(sldqmc_ctx *c, const double *R, double *V, double *Ts, int B);
 void oz_r2r1(sldqmc_ctx *c, const double *R2, const double *R1, double *R, int B);
+
+// The whole weight of a configuration in one CTA (small.cu: FP64 mode, dense
+// propagator, N <= 32).
+bool small_fits(const sldqmc_ctx *c);
+void small_weight(sldqmc_ctx *c, const int8_t *d_s, int B, double cu, double cd, int tau0, double *d_ld, int *d_sign,
+                  double *d_G, double scale, int accumulate);
 
 // Slice products with the separable exp(-dtau K) (sep.cu): X^T_out =
 // U^T D_t0 E D_t0+1 E ... for nb slices, one row per CTA in shared memory.
@@ -168,6 +174,8 @@ struct sldqmc_ctx {
     double dtauJ, Ktau;          // bare-weight constants
     // stabilisation workspace, cap items each
     int cap;
+    int plan_cap;      // items per call that a choice between two ways of a product goes by: the caller's
+                       // max_batch also on the twin, so that both give the same bits
     long long nn;      // N*N
     double *buf[9];    // Ut, V, X1, X2, W(2*nn), Y, R1, R2, Vg
     double *d_D, *d_Dp, *d_logacc;

@@ -123,7 +123,7 @@ extern "C" int sldqmc_weight_noalloc(const sldqmc_params *p, void *stream, const
     c.M = (int)M;
     c.p.beta = (double)M * p->dtau;
     c.st = (cudaStream_t)stream;
-    c.cap = B;
+    c.cap = c.plan_cap = B;
     c.nn = N * N;
     for (int e = 0; e < 2; ++e) {
         const double et = e == 0 ? 1.0 : -1.0;

@@ -1687,9 +1687,9 @@ bool oz_have_e(sldqmc_ctx *c) { return c->oz_ws && oz_e_planes(c); }
 // 8 us: below 128 sites (where an item fills no tile of its own) the tensor
 // cores take it from N^3 B = 8e6 (14 us of the FP64 pipe) on.  Measured at 8 x
 // 8, 64 chains, both flavours: 2 x 44 us against 10 + 15 us.
-bool oz_worth(const sldqmc_ctx *c, int B)
+bool oz_worth(const sldqmc_ctx *c, int times)
 {
-    return c->N >= OBM || (double)c->N * c->N * c->N * B >= 8e6;
+    return c->N >= OBM || (double)c->N * c->N * c->N * c->plan_cap * times >= 8e6;
 }
 
 bool oz_full(const sldqmc_ctx *c) { return c->oz_ws && c->N >= OBM; }

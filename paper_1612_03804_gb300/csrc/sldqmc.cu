@@ -197,6 +197,10 @@ int weight_run(sldqmc_ctx *c, const int8_t *d_s, int B, int eta, int tau0, doubl
     const int N = c->N, M = c->M;
     const long long nn = c->nn;
     const double cu = c->ex_scale[eta < 0][0], cd = c->ex_scale[eta < 0][1];
+    if (small_fits(c)) {
+        small_weight(c, d_s, B, cu, cd, tau0, d_ld, d_sign, d_G, scale, accumulate);
+        return SLDQMC_OK;
+    }
     double *Ut = c->buf[0], *Yb = c->buf[5], *X1 = c->buf[2], *X2 = c->buf[3];
     launch_init_udv(c, Ut, c->buf[1], B);
     std::vector<int> slices;
@@ -211,7 +215,7 @@ int weight_run(sldqmc_ctx *c, const int8_t *d_s, int B, int eta, int tau0, doubl
         } else if (chain) {
             oz_chain_block(c, Ut, d_s, B, cu, cd, (tau0 + m) % M, nb, X1);
             Xt = X1;
-        } else if (oz && oz_worth(c, B)) {
+        } else if (oz && oz_worth(c, 1)) {
             for (int j = 0; j < nb; ++j)
                 oz_slice_product(c, j == 0 ? Ut : X1, d_s + (long long)((tau0 + m + j) % M) * N, cu, cd, X1, B);
             Xt = X1;
@@ -287,6 +291,7 @@ sldqmc_ctx *get_twin(sldqmc_ctx *c)
         return nullptr;
     }
     t->no_twin = 1;
+    t->plan_cap = c->cap;
     t->kinetic = c->kinetic;
     if (c->tile_n == 128) tc_set_tile_n(t, 128);
     t->tile_n = c->tile_n;
@@ -630,7 +635,7 @@ int sldqmc_create(const sldqmc_params *p, void *stream, sldqmc_ctx **out)
     c->M = (int)M;
     c->p.beta = (double)M * p->dtau;
     c->st = (cudaStream_t)stream;
-    c->cap = p->max_batch;
+    c->cap = c->plan_cap = p->max_batch;
     c->nn = N * N;
     {
         int dev = 0;
@@ -893,7 +898,7 @@ static int fresh_gt(sldqmc_ctx *c, const int8_t *d_s, int B, int tau1, double *d
             if (rc) return rc;
         }
     }
-    if (oz_have_e(c) && oz_worth(c, 2 * B)) {
+    if (oz_have_e(c) && oz_worth(c, 2)) {
         double *Tt[2] = {Gt, Gt + (long long)B * nn};  // in place: the products read digit planes
         oz_similarity(c, src, Tt, dst, 1, nullptr, nullptr, B);
         return SLDQMC_OK;
@@ -916,7 +921,7 @@ static void wrap_gt(sldqmc_ctx *c, const int8_t *d_s, int B, int tau, double *sr
     const long long nn = c->nn;
     double *T = c->d_G[0] + 3 * (size_t)c->cap * nn;
     double *src[2] = {srcp, srcm}, *dst[2] = {dstp, dstm};
-    if (oz_have_e(c) && oz_worth(c, 2 * B)) {
+    if (oz_have_e(c) && oz_worth(c, 2)) {
         double *Tt[2] = {T - (size_t)c->cap * nn, T};
         oz_similarity(c, src, Tt, dst, 0, d_s + (long long)tau * N, c->ex_scale, B);
         return;

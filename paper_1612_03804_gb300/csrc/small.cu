@@ -1,0 +1,320 @@
+// small.cu -- the whole stabilised weight of a configuration in one CTA, for
+// lattices of up to 32 sites.
+//
+// A weight of such a lattice is a chain of some forty dependent steps (slice
+// products, Gram matrix, pivot sort, Cholesky, V update per block, then the LU),
+// each of a few microseconds of launch latency and almost no work: 4 x 4, 20
+// slices 675 us as 42 launches, 107 us here.  All matrices live in shared memory (five
+// of 32 x 33 doubles), a step costs a barrier instead of a launch, and the FP64
+// pipe is the bound: a warp's instruction holds it for 64 cycles, so elements
+// are dealt to threads without gaps (thread e, e + 256, ... of the N x N).
+// The method and its error flags are those of stab.cu: X^T <- X^T D E per
+// slice; per block pre-pivoted Cholesky-QR (twice in the last block), D, V;
+// then M_mid = D_b^-1 U^T + D_s V, LU with partial pivoting, G by substitution.
+#include <cuda_runtime.h>
+#include <math.h>
+
+#include "chol32.cuh"
+#include "internal.h"
+
+namespace sldqmc {
+
+namespace {
+
+constexpr int SM_N = 32, SM_LD = 33, SM_THREADS = 256;
+typedef double (*Mat)[SM_LD];
+
+struct SmallArgs {
+    const double *E;
+    const int8_t *s;
+    int N, M, n_wrap, tau0;
+    double cu, cd;
+    double *ld;
+    int *sign;
+    double *G;
+    double scale;
+    int accumulate;
+    int *flag;
+};
+
+// C = A B (sum over k0(r) <= k < k1(c)) for N x N matrices, C distinct from both.
+template <class K0, class K1, class Load>
+__device__ __forceinline__ void sm_product(Mat C, int N, K0 k0, K1 k1, Load ab)
+{
+    for (int e = threadIdx.x; e < N * N; e += SM_THREADS) {
+        const int r = e / N, c = e - r * N;
+        double a0 = 0.0, a1 = 0.0;  // two chains
+        int k = k0(r);
+        const int kend = k1(c);
+        for (; k + 1 < kend; k += 2) {
+            a0 = ab(a0, r, k, c);
+            a1 = ab(a1, r, k + 1, c);
+        }
+        if (k < kend) a0 = ab(a0, r, k, c);
+        C[r][c] = a0 + a1;
+    }
+    __syncthreads();
+}
+
+// W <- R^-T W for the N rows of W, R above the diagonal of F, 1 / R_jj on it.
+__device__ __forceinline__ void sm_solve(Mat W, Mat F, int N)
+{
+    for (int l = 0; l < N; ++l) {
+        for (int c = threadIdx.x; c < N; c += SM_THREADS) W[l][c] *= F[l][l];
+        __syncthreads();
+        for (int e = threadIdx.x; e < (N - 1 - l) * N; e += SM_THREADS) {
+            const int q = e / N, r = l + 1 + q, c = e - q * N;
+            W[r][c] -= F[l][r] * W[l][c];
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(SM_THREADS) k_small_weight(SmallArgs a)
+{
+    __shared__ double buf[5][SM_N][SM_LD];
+    __shared__ double D[SM_N], Dp[SM_N], root[SM_N], piv[SM_N], part[SM_N];
+    __shared__ unsigned long long key[SM_N];
+    __shared__ int perm[SM_N], s_p;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int N = a.N;
+    const int8_t *s = a.s + (long long)b * a.M * N;
+    Mat E = buf[0], U = buf[1], F = buf[2], V = buf[3], W = buf[4];
+    for (int e = tid; e < N * N; e += SM_THREADS) {
+        const int r = e / N, c = e - r * N;
+        E[r][c] = a.E[e];
+        U[r][c] = V[r][c] = r == c ? 1.0 : 0.0;
+    }
+    if (tid < N) D[tid] = 1.0;
+    int sgn = 1;  // warp 0
+    __syncthreads();
+    const auto from0 = [](int) { return 0; };
+    const auto toN = [N](int) { return N; };
+    int slice = a.tau0;
+    for (int m = 0; m < a.M; m += a.n_wrap) {
+        const int nb = a.n_wrap < a.M - m ? a.n_wrap : a.M - m;
+        const int passes = m + nb >= a.M ? 2 : 1;
+        for (int j = 0; j < nb; ++j) {
+            const int8_t *sl = s + (long long)slice * N;
+            for (int e = tid; e < N * N; e += SM_THREADS) {
+                const int r = e / N, c = e - r * N;
+                U[r][c] *= sl[c] > 0 ? a.cu : a.cd;
+            }
+            __syncthreads();
+            sm_product(F, N, from0, toN, [=](double x, int r, int k, int c) { return fma(U[r][k], E[k][c], x); });
+            Mat t = U;
+            U = F;
+            F = t;
+            if (++slice == a.M) slice = 0;
+        }
+        // Gram matrix of the rows of U = X^T
+        sm_product(W, N, from0, toN, [=](double x, int r, int k, int c) { return fma(U[r][k], U[c][k], x); });
+        // sort by sqrt(W_jj) D_j, largest first (non-negative doubles order like
+        // their bit patterns); the parity of the permutation by its inversions
+        if (wid == 0) {
+            if (lane < N) key[lane] = (unsigned long long)__double_as_longlong(sqrt(W[lane][lane]) * D[lane]);
+            __syncwarp();
+            int rank = 0;
+            if (lane < N) {
+                for (int i = 0; i < N; ++i) rank += key[i] > key[lane] || (key[i] == key[lane] && i < lane);
+                perm[rank] = lane;
+            }
+            int inv = 0;
+            for (int i = 0; i < N; ++i) {
+                const int ri = __shfl_sync(0xffffffffu, rank, i);
+                inv += lane < N && i < lane && ri > rank;
+            }
+            if (__popc(__ballot_sync(0xffffffffu, inv & 1)) & 1) sgn = -sgn;
+            __syncwarp();
+            if (lane < N) Dp[lane] = D[perm[lane]];
+        }
+        __syncthreads();
+        // the permuted Gram matrix for the factor, then the permuted rows in its place
+        for (int e = tid; e < SM_N * SM_N; e += SM_THREADS) {
+            const int r = e >> 5, c = e & 31;
+            F[r][c] = r < N && c < N ? (c >= r ? W[perm[r]][perm[c]] : 0.0) : (r == c ? 1.0 : 0.0);
+        }
+        __syncthreads();
+        for (int e = tid; e < N * N; e += SM_THREADS) {
+            const int r = e / N, c = e - r * N;
+            W[r][c] = U[perm[r]][c];
+        }
+        chol32(F, root, N, a.flag);
+        sm_solve(W, F, N);
+        if (tid < N) F[tid][tid] = root[tid];
+        __syncthreads();
+        if (passes == 2) {
+            // W = Q1^T: its Gram matrix into U, factor R2, solve, R = R2 R1
+            for (int e = tid; e < SM_N * SM_N; e += SM_THREADS) {
+                const int r = e >> 5, c = e & 31;
+                double x = r == c ? 1.0 : 0.0;
+                if (r < N && c < N) {
+                    x = 0.0;
+                    if (c >= r)
+                        for (int k = 0; k < N; ++k) x = fma(W[r][k], W[c][k], x);
+                }
+                U[r][c] = x;
+            }
+            __syncthreads();
+            chol32(U, root, N, a.flag);
+            sm_solve(W, U, N);
+            if (tid < N) U[tid][tid] = root[tid];
+            __syncthreads();
+            double x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int e = tid + q * SM_THREADS, r = e / N, c = e - r * N;
+                x[q] = 0.0;
+                if (e < N * N)
+                    for (int k = r; k <= c; ++k) x[q] = fma(U[r][k], F[k][c], x[q]);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int e = tid + q * SM_THREADS, r = e / N, c = e - r * N;
+                if (e < N * N && c >= r) F[r][c] = x[q];
+            }
+            __syncthreads();
+        }
+        if (tid < N) {
+            double d = F[tid][tid] * Dp[tid];
+            if (!(d > 0.0) || !isfinite(d)) {
+                atomicOr(a.flag, FLAG_NUMERICAL);
+                d = 1.0;
+            }
+            D[tid] = d;
+            part[tid] = 1.0 / d;
+        }
+        __syncthreads();
+        // V <- (D^-1 R D_p) P^T V: the factor's upper triangle in place, V into U
+        for (int e = tid; e < N * N; e += SM_THREADS) {
+            const int r = e / N, c = e - r * N;
+            if (c >= r) F[r][c] = F[r][c] * Dp[c] * part[r];
+        }
+        __syncthreads();
+        sm_product(U, N, [](int r) { return r; }, toN,
+                   [=](double x, int r, int k, int c) { return fma(F[r][k], V[perm[k]][c], x); });
+        Mat t = V;  // V <- U, U <- W (= Q^T)
+        V = U;
+        U = W;
+        W = t;
+    }
+    // M_mid = D_b^-1 U^T + D_s V in W, its right-hand side D_b^-1 U^T in U
+    if (tid < N) {
+        const double d = D[tid];
+        part[tid] = d > 1.0 ? log(d) : 0.0;
+        Dp[tid] = d > 1.0 ? 1.0 / d : 1.0;
+    }
+    __syncthreads();
+    for (int e = tid; e < N * N; e += SM_THREADS) {
+        const int r = e / N, c = e - r * N;
+        const double u = U[r][c] * Dp[r], d = D[r];
+        U[r][c] = u;
+        W[r][c] = u + (d > 1.0 ? 1.0 : d) * V[r][c];
+    }
+    __syncthreads();
+    const int cols = a.G ? 2 * N : N;
+    for (int j = 0; j < N; ++j) {
+        if (wid == 0) {
+            // the largest |entry| of the column, the lowest row on ties
+            unsigned long long bk = lane >= j && lane < N ? (unsigned long long)__double_as_longlong(fabs(W[lane][j])) : 0ull;
+            int bi = lane >= j && lane < N ? lane : N;
+            for (int o = 16; o > 0; o >>= 1) {
+                const unsigned long long ok = __shfl_xor_sync(0xffffffffu, bk, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (oi < N && (bi >= N || ok > bk || (ok == bk && oi < bi))) {
+                    bk = ok;
+                    bi = oi;
+                }
+            }
+            if (bi != j) sgn = -sgn;
+            double v = W[bi][j];
+            if (v == 0.0 || !isfinite(v)) {
+                if (lane == 0) atomicOr(a.flag, FLAG_NUMERICAL);
+                v = 1.0;
+            }
+            if (v < 0.0) sgn = -sgn;
+            if (lane == 0) {
+                s_p = bi;
+                piv[j] = v;
+                root[j] = 1.0 / v;
+            }
+        }
+        __syncthreads();
+        const int p = s_p;
+        // rows j and p change places (row j holds U12 from now on)
+        for (int c = tid; c < cols; c += SM_THREADS) {
+            double *x = c < N ? &W[j][c] : &U[j][c - N], *y = c < N ? &W[p][c] : &U[p][c - N];
+            if (p != j) {
+                const double t = *x;
+                *x = *y;
+                *y = t;
+            }
+            if (c == j) *x = piv[j];
+        }
+        __syncthreads();
+        const double rv = root[j];
+        const int nc = cols - 1 - j;
+        for (int e = tid; e < (N - 1 - j) * nc; e += SM_THREADS) {
+            const int q = e / nc, r = j + 1 + q, c = j + 1 + (e - q * nc);
+            const double f = W[r][j] * rv;
+            if (c < N) W[r][c] -= f * W[j][c];
+            else U[r][c - N] -= f * U[j][c - N];
+        }
+        __syncthreads();
+    }
+    if (a.G) {
+        // back substitution: X_r = (Y_r - sum_{l > r} U_rl X_l) / U_rr
+        for (int r = N - 1; r >= 0; --r) {
+            for (int c = tid; c < N; c += SM_THREADS) U[r][c] *= root[r];
+            __syncthreads();
+            for (int e = tid; e < r * N; e += SM_THREADS) {
+                const int q = e / N, c = e - q * N;
+                U[q][c] -= W[q][r] * U[r][c];
+            }
+            __syncthreads();
+        }
+        for (int e = tid; e < N * N; e += SM_THREADS) {
+            const int r = e / N, c = e - r * N;
+            a.G[(long long)b * N * N + e] = U[r][c];
+        }
+    }
+    if (wid == 0) {
+        double x = lane < N ? part[lane] + log(fabs(piv[lane])) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) {
+            if (a.accumulate) {
+                a.ld[b] += a.scale * x;
+            } else {
+                a.ld[b] = a.scale * x;
+                if (a.sign) a.sign[b] = sgn;
+            }
+        }
+    }
+}
+
+}  // namespace
+
+// A CTA per item does N^3 FMAs per slice on one SM's FP64 pipe, so with several
+// items per SM the launches over all items win from 26 sites on.  Measured, 40
+// slices, one CTA per item against launches: 4 x 4, 1 / 1024 items 179 / 623 us
+// against 635 / 1348; 5 x 5, 1024 items 1813 against 2093; 4 x 7, 128 / 512 items
+// 585 / 1576 against 897 / 1247; 8 x 4, 128 / 512 items 670 / 2079 against 916 / 1277.
+bool small_fits(const sldqmc_ctx *c)
+{
+    const double n3 = (double)c->N * c->N * c->N;
+    return c->N <= SM_N && c->p.prec == SLDQMC_FP64 && c->kinetic != SLDQMC_KINETIC_SEPARABLE &&
+           (c->N <= 25 || n3 * c->plan_cap <= 7.5e6);
+}
+
+void small_weight(sldqmc_ctx *c, const int8_t *d_s, int B, double cu, double cd, int tau0, double *d_ld, int *d_sign,
+                  double *d_G, double scale, int accumulate)
+{
+    const SmallArgs a{c->d_E, d_s, c->N, c->M, c->p.n_wrap, tau0, cu, cd, d_ld, d_sign, d_G, scale, accumulate, c->d_flag};
+    prof_begin(c, SLDQMC_KC_PANEL_F64, 2.0 * c->N * c->N * c->N * c->M * B, "small_weight");
+    k_small_weight<<<B, SM_THREADS, 0, c->st>>>(a);
+    prof_end(c);
+    c->launches++;
+}
+
+}  // namespace sldqmc

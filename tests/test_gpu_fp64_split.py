@@ -118,3 +118,32 @@ def test_fp64_small_local_sweep(Lx, Ly, B):
         assert stats[b]["margin_events"] == 0
         np.testing.assert_array_equal(out[b], so)
         assert stats[b]["max_drift"] < TOL
+
+
+# Up to 25 sites, and to 32 with few configurations, a whole weight runs in one
+# CTA; 27 and 32 sites with a capacity beyond that take the launches.
+@pytest.mark.parametrize("Lx,Ly,B,cap", [(1, 1, 2, 2), (3, 1, 3, 3), (5, 5, 3, 3), (9, 3, 2, 2), (9, 3, 2, 512), (8, 4, 3, 3),
+                                         (8, 4, 3, 400), (11, 3, 2, 2)])
+def test_fp64_one_cta_weight(Lx, Ly, B, cap):
+    import torch
+    from oracle import oracle as O
+    from paper_1612_03804_gb300 import sldqmc
+    M, N = 11, Lx * Ly
+    m = _model(Lx, Ly, M, n_wrap=4)
+    s = batch_uniform(180 + N, B, M, N)
+    with sldqmc.Context(Lx, Ly, mu=-0.5, xi=1.0, beta=M * 0.1, dtau=0.1, n_wrap=4, max_batch=cap) as ctx:
+        d_s = torch.from_numpy(s).cuda()
+        G = torch.zeros((B, N, N), dtype=torch.float64, device="cuda")
+        ld = torch.zeros(B, dtype=torch.float64, device="cuda")
+        sg = torch.zeros(B, dtype=torch.int32, device="cuda")
+        lw = torch.zeros(B, dtype=torch.float64, device="cuda")
+        ctx.green_batch_dev(d_s, -1, 6, G, ld, sg)
+        ctx.log_weight_batch_dev(d_s, lw)
+        ctx.sync()
+        for b in range(B):
+            ref, rs, Gr = O.weight(m, s[b], -1, tau0=6, want_G=True)
+            assert int(sg[b]) == rs
+            assert abs(float(ld[b]) - ref) <= TOL * max(1.0, abs(ref))
+            assert np.abs(G[b].cpu().numpy() - Gr).max() < TOL
+            both = 2.0 * (O.weight(m, s[b], 1)[0] + O.weight(m, s[b], -1)[0]) + ctx.log_bare_weight(s[b])
+            assert abs(float(lw[b]) - both) <= TOL * max(1.0, abs(both))
