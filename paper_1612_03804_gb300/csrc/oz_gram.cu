@@ -40,7 +40,7 @@
 // two parts with their own A rows and outputs): warp 0 streams the 8 + 8
 // digit-plane tiles of a 32-wide K-block by TMA (64-byte swizzle), warp 1
 // issues the 36 digit products per 16-wide K-step as eight MMAs (A's plane p
-// against B's planes 0..7-p at once), and eight epilogue warps drain one
+// against B's planes 0..7-p at once), and sixteen epilogue warps drain one
 // of two tensor-memory buffers (8 groups x 32 columns each) while the next
 // tile accumulates into the other.  Every mbarrier wait is bounded; a wait
 // that runs out raises the context's timeout flag and the CTA frees its
@@ -71,7 +71,8 @@ constexpr int OSTAGES = 2;
 constexpr int OTILE_A = OBM * 64;  // one digit plane of A per stage
 constexpr int OTILE_B = OBN * 64;
 constexpr int OSTAGE = OZ_S * (OTILE_A + OTILE_B);
-constexpr int OEPI = 8;            // epilogue warps, two per TMEM lane quarter
+constexpr int OEPI = 16;           // epilogue warps, four per TMEM lane quarter
+constexpr int OCOL = OBN * 4 / OEPI;  // accumulator columns drained by one of them
 constexpr int OTHREADS = 64 + 32 * OEPI;
 constexpr int OTMEM = 2 * OZ_G * OBN;  // two buffers of eight 32-column accumulators
 
@@ -113,36 +114,44 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, 
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
-// Balanced base-2^7 digits of v = round(|x| 2^(57 - E)) < 2^57 for a double x
-// with |x| < 2^E (E the frexp exponent of its row's maximum, ef_max its
-// biased exponent, 0 for a row of zeros or subnormals): x 2^-E = sum_p
-// dg[p] 2^-(7p+8), p = 0..7.
-__device__ __forceinline__ void oz_digits(double x, int E, int ef_max, int dg[OZ_S])
+// The balanced base-2^7 digits of x 2^-E = sum_p dg[p] 2^-(7p+8), p = 0..7, for
+// |x| < 2^E (E the frexp exponent of its row's maximum, or a bound; subnormals
+// count as zero): v = x 2^(57-E) rounded to an integer, plus the bias that makes
+// each of the seven low 7-bit fields a digit + 64, so that the digits are
+// fields, without carries.
+__device__ __forceinline__ long long oz_fixed(double x, int E)
 {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const long long u = __double_as_longlong(x);
     const int ef = (int)((u >> 52) & 0x7FF);
+    const unsigned long long m = ((unsigned long long)u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const int r = E - ef + 1075 - OZ_BITS;  // x = m 2^(ef - 1075); r >= -4 since |x| < 2^E
     long long v = 0;
-    if (ef > 0 && ef_max > 0) {
-        // x = m 2^(ef - 1075)
-        const unsigned long long m = (u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-        const int sh = ef - 1075 + OZ_BITS - E;
-        if (sh >= 0) v = (long long)(m << sh);  // sh <= 4 since |x| < 2^E
-        else if (sh > -60) v = (long long)((m + (1ull << (-sh - 1))) >> (-sh));
+    if (ef > 0 && r < 60) v = r <= 0 ? (long long)(m << (r < -4 ? 4 : -r)) : (long long)((m + (1ull << (r - 1))) >> r);
+    constexpr long long bias = 64ll * (1 + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) + (1ll << 35) + (1ll << 42));
+    return (u < 0 ? -v : v) + bias;
+}
+
+// Digit p of two such values as a pair of BF16: an integer below 2^23 placed
+// in the mantissa of 2^23 (1.5 2^23 for the signed leading digit) is converted
+// by one FP32 subtraction, and BF16 is the upper half of its FP32.
+__device__ __forceinline__ uint32_t oz_pair(long long a, long long b, int p)
+{
+    float fa, fb;
+    if (p == 0) {
+        fa = __uint_as_float(0x4B400000u + (uint32_t)(int)(a >> 49)) - 12582912.0f;
+        fb = __uint_as_float(0x4B400000u + (uint32_t)(int)(b >> 49)) - 12582912.0f;
+    } else {
+        const int s = 7 * (7 - p);
+        fa = __uint_as_float(0x4B000000u | ((uint32_t)(a >> s) & 127u)) - 8388672.0f;
+        fb = __uint_as_float(0x4B000000u | ((uint32_t)(b >> s) & 127u)) - 8388672.0f;
     }
-#pragma unroll
-    for (int p = OZ_S - 1; p >= 1; --p) {
-        int d = (int)(v & ((1 << OZ_BETA) - 1));
-        v >>= OZ_BETA;
-        if (d >= (1 << (OZ_BETA - 1))) {
-            d -= 1 << OZ_BETA;
-            v += 1;
-        }
-        dg[p] = d;
-    }
-    dg[0] = (int)v;  // 0..256
-    if (u >> 63)
-#pragma unroll
-        for (int p = 0; p < OZ_S; ++p) dg[p] = -dg[p];
+    return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+}
+
+// Plane p of eight values, 16 bytes.
+__device__ __forceinline__ uint4 oz_pair8(const long long (&v)[8], int p)
+{
+    return make_uint4(oz_pair(v[0], v[1], p), oz_pair(v[2], v[3], p), oz_pair(v[4], v[5], p), oz_pair(v[6], v[7], p));
 }
 
 // Digits of the rows of one or two matrices (rows x cols, row stride ld, item
@@ -193,13 +202,10 @@ __global__ void __launch_bounds__(256) k_oz_slice(OzRows a, long long sX, int ro
     if (lane == 0) (blockIdx.z ? a.E[1] : a.E[0])[(long long)b * prow + i] = Ei;
     __nv_bfloat16 *row = (blockIdx.z ? a.planes[1] : a.planes[0]) + ((long long)b * prow + i) * ldp;
     for (int k = 2 * lane; k < N; k += 64) {
-        int d0[OZ_S], d1[OZ_S];
-        oz_digits(at(k), Ei, ef_max, d0);
-        oz_digits(k + 1 < N ? at(k + 1) : 0.0, Ei, ef_max, d1);
+        const long long v0 = oz_fixed(at(k), Ei), v1 = oz_fixed(k + 1 < N ? at(k + 1) : 0.0, Ei);
 #pragma unroll
         for (int p = 0; p < OZ_S; ++p)
-            *reinterpret_cast<__nv_bfloat162 *>(row + (long long)p * plane_stride + k) =
-                __floats2bfloat162_rn((float)d0[p], (float)d1[p]);
+            *reinterpret_cast<uint32_t *>(row + (long long)p * plane_stride + k) = oz_pair(v0, v1, p);
     }
 }
 
@@ -236,7 +242,7 @@ __device__ __forceinline__ void oz_slice_block(int bx, const double *src, long l
     __syncthreads();
     const int r = threadIdx.x >> 3, q = threadIdx.x & 7;
     const int j = c0 + r;
-    int dg[4][OZ_S];
+    long long v4[4];
     if (LOCAL) {
         // the row's largest |entry| over its eight threads (lanes 8r'..8r'+7)
         unsigned long long mx = 0;
@@ -256,7 +262,7 @@ __device__ __forceinline__ void oz_slice_block(int bx, const double *src, long l
         const int E = oz_exponent(ef_max);
         if (q == 0) Ej[(long long)b * sE + j] = E;
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) oz_digits(tile[4 * q + jj][r], E, ef_max, dg[jj]);
+        for (int jj = 0; jj < 4; ++jj) v4[jj] = oz_fixed(tile[4 * q + jj][r], E);
     } else {
         if (j >= Nc) return;
         const int E = Ej[(long long)b * sE + j];
@@ -266,17 +272,15 @@ __device__ __forceinline__ void oz_slice_block(int bx, const double *src, long l
         for (int jj = 0; jj < 4; ++jj) {
             const double x = tile[4 * q + jj][r];
             over |= ((unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull) >= bound;
-            oz_digits(x, E, 1, dg[jj]);
+            v4[jj] = oz_fixed(x, E);
         }
         if (over) atomicOr(flag, FLAG_NUMERICAL);
     }
     const long long row = ((long long)b * rows_cap + j) * ldk + koff + 4 * q;
 #pragma unroll
-    for (int p = 0; p < OZ_S; ++p) {
-        __nv_bfloat162 h2[2] = {__floats2bfloat162_rn((float)dg[0][p], (float)dg[1][p]),
-                                __floats2bfloat162_rn((float)dg[2][p], (float)dg[3][p])};
-        *reinterpret_cast<uint2 *>(planes + (long long)p * plane_stride + row) = *reinterpret_cast<const uint2 *>(h2);
-    }
+    for (int p = 0; p < OZ_S; ++p)
+        *reinterpret_cast<uint2 *>(planes + (long long)p * plane_stride + row) =
+            make_uint2(oz_pair(v4[0], v4[1], p), oz_pair(v4[2], v4[3], p));
 }
 
 __global__ void __launch_bounds__(256) k_oz_slice_fixed(const double *src, long long sS, long long ld, int j0, int Nc,
@@ -435,16 +439,14 @@ __global__ void __launch_bounds__(256) k_oz_panel_prep(OzPanelPrep f, OzPanelSli
     const int ef_max = (int)(mx >> 52);
     const int E = oz_exponent(ef_max);
     if (q == 0) f.ET[b * 32 + r] = E;
-    int dg[4][OZ_S];
+    long long v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) oz_digits(tv[i], E, ef_max, dg[i]);
+    for (int i = 0; i < 4; ++i) v[i] = oz_fixed(tv[i], E);
     const long long row = ((long long)b * 32 + r) * 32 + 4 * q;
 #pragma unroll
-    for (int p = 0; p < OZ_S; ++p) {
-        __nv_bfloat162 h2[2] = {__floats2bfloat162_rn((float)dg[0][p], (float)dg[1][p]),
-                                __floats2bfloat162_rn((float)dg[2][p], (float)dg[3][p])};
-        *reinterpret_cast<uint2 *>(f.tplanes + (long long)p * f.tps + row) = *reinterpret_cast<const uint2 *>(h2);
-    }
+    for (int p = 0; p < OZ_S; ++p)
+        *reinterpret_cast<uint2 *>(f.tplanes + (long long)p * f.tps + row) =
+            make_uint2(oz_pair(v[0], v[1], p), oz_pair(v[2], v[3], p));
 }
 
 // One part of a product's rows: rows m of C (rows of A, starting at plane row
@@ -755,9 +757,9 @@ __global__ void __launch_bounds__(OTHREADS, 1)
             }
         }
     } else {
-        // epilogue: warp w drains lane quarter w % 4, columns [hc, hc + 16)
+        // epilogue: warp w drains lane quarter w % 4, columns [hc, hc + OCOL)
         const int q4 = warp & 3;
-        const int hc = ((warp - 2) >> 2) * 16;
+        const int hc = ((warp - 2) >> 2) * OCOL;
         int cc = 0;  // chunk counter, in step with the MMA thread's
         bool ok = true;
         for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
@@ -778,20 +780,20 @@ __global__ void __launch_bounds__(OTHREADS, 1)
             const long long cs = TRANS ? ldc : 1;
             const int nb = n0 + hc;
             const int *eb = (part ? a.pt[1].EB : a.pt[0].EB) + (a.b_shared ? 0 : (long long)b * (part ? a.pt[1].sEB : a.pt[0].sEB));
-            double cold[16];
+            double cold[OCOL];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) cold[j] = (SUB && mm < M && nb + j < a.Nn) ? o[(nb + j) * cs] : 0.0;
+            for (int j = 0; j < OCOL; ++j) cold[j] = (SUB && mm < M && nb + j < a.Nn) ? o[(nb + j) * cs] : 0.0;
             // the columns' exponents, also fetched while the MMAs run (not for an
             // update, whose old values already take those registers)
-            int ebv[16];
+            int ebv[OCOL];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) ebv[j] = (!SUB && nb + j < a.Nn) ? eb[nb + j] : 0;
+            for (int j = 0; j < OCOL; ++j) ebv[j] = (!SUB && nb + j < a.Nn) ? eb[nb + j] : 0;
             // The group sums as exact integers, folded as they arrive and added
             // over the K-chunks (|h| <= K 2^37): groups 0..3 (p + q = 2..5) into h,
             // 4..7 (6..9) into l, so that sum_g acc_g 2^-(7(g+2)+2) = h 2^-37 + l 2^-65
-            long long h[16], l[16];
+            long long h[OCOL], l[OCOL];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) h[j] = l[j] = 0;
+            for (int j = 0; j < OCOL; ++j) h[j] = l[j] = 0;
             int k_lo, k_hi;
             oz_krange(a, m0, n0, k_lo, k_hi);
             for (int kc0 = k_lo; kc0 < k_hi; kc0 += OZ_KCHUNK, ++cc) {
@@ -800,19 +802,16 @@ __global__ void __launch_bounds__(OTHREADS, 1)
                 fence_after();
                 const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(u * OZ_G * OBN + hc);
 #pragma unroll
-                for (int c8 = 0; c8 < 16; c8 += 8) {
+                for (int gg = 0; gg < OZ_G; gg += 4) {
+                    uint32_t r[4][OCOL];
 #pragma unroll
-                    for (int gg = 0; gg < OZ_G; gg += 4) {
-                        uint32_t r[4][8];
+                    for (int g = 0; g < 4; ++g) tmem_ld8_nowait(lane_base + (uint32_t)((gg + g) * OBN), r[g]);
+                    tmem_wait_ld8x4(r[0], r[1], r[2], r[3]);
 #pragma unroll
-                        for (int g = 0; g < 4; ++g) tmem_ld8_nowait(lane_base + (uint32_t)((gg + g) * OBN + c8), r[g]);
-                        tmem_wait_ld8x4(r[0], r[1], r[2], r[3]);
+                    for (int j = 0; j < OCOL; ++j)
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
-#pragma unroll
-                            for (int g = 0; g < 4; ++g)
-                                oz_fold(gg ? l[c8 + j] : h[c8 + j], __float2int_rn(__uint_as_float(r[g][j])), OZ_BETA * (3 - g));
-                    }
+                        for (int g = 0; g < 4; ++g)
+                            oz_fold(gg ? l[j] : h[j], __float2int_rn(__uint_as_float(r[g][j])), OZ_BETA * (3 - g));
                 }
                 fence_before();
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tmem_free[u])) : "memory");
@@ -823,7 +822,7 @@ __global__ void __launch_bounds__(OTHREADS, 1)
             const int8_t *sg = (TRANS && !SUB && !SLICE && a.sgn) ? a.sgn + (long long)item * a.sSgn : nullptr;
             const bool up = sg && sg[mi] > 0;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
+            for (int j = 0; j < OCOL; ++j) {
                 const int n = nb + j;
                 double v = 0.0;
                 if (n < a.Nn) {
@@ -848,25 +847,15 @@ __global__ void __launch_bounds__(OTHREADS, 1)
                 // eight K positions per 16-byte store: each lane writes its own plane row,
                 // so the stores cannot coalesce across lanes; wider stores halve the
                 // sector writes
+                long long v8[OCOL];
 #pragma unroll
-                for (int g8 = 0; g8 < 2; ++g8) {
-                    int dg[8][OZ_S];
-#pragma unroll
-                    for (int jj = 0; jj < 8; ++jj) {
-                        const double x = __longlong_as_double(h[8 * g8 + jj]);
-                        over |= ((unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull) >= bound;
-                        oz_digits(x, E, 1, dg[jj]);
-                    }
-#pragma unroll
-                    for (int p = 0; p < OZ_S; ++p) {
-                        __nv_bfloat162 h2[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i)
-                            h2[i] = __floats2bfloat162_rn((float)dg[2 * i][p], (float)dg[2 * i + 1][p]);
-                        *reinterpret_cast<uint4 *>(dst + (long long)p * a.splane_stride + 8 * g8) =
-                            *reinterpret_cast<const uint4 *>(h2);
-                    }
+                for (int jj = 0; jj < OCOL; ++jj) {
+                    over |= ((unsigned long long)h[jj] & 0x7FFFFFFFFFFFFFFFull) >= bound;
+                    v8[jj] = oz_fixed(__longlong_as_double(h[jj]), E);
                 }
+#pragma unroll
+                for (int p = 0; p < OZ_S; ++p)
+                    *reinterpret_cast<uint4 *>(dst + (long long)p * a.splane_stride) = oz_pair8(v8, p);
                 if (over) atomicOr(a.flag, FLAG_NUMERICAL);
             }
         }
@@ -962,8 +951,7 @@ __device__ __forceinline__ ChValue ch_scaled(long long h, long long l, int e, un
     return v;
 }
 
-// v 2^(57 - E) rounded to an integer, plus the bias that makes each of the
-// seven low 7-bit fields a digit + 64; |v| < 2^E.
+// As oz_fixed; |v| < 2^E.
 __device__ __forceinline__ long long ch_fixed(const ChValue &v, int E)
 {
     const int r = E - v.ex + 63 - OZ_BITS;  // >= 7
@@ -971,23 +959,6 @@ __device__ __forceinline__ long long ch_fixed(const ChValue &v, int E)
     if (r < 64) w = (long long)(((v.m >> (r - 1)) + 1ull) >> 1);
     constexpr long long bias = 64ll * (1 + (1ll << 7) + (1ll << 14) + (1ll << 21) + (1ll << 28) + (1ll << 35) + (1ll << 42));
     return (v.neg ? -w : w) + bias;
-}
-
-// Digit p of two such values as a pair of BF16: an integer below 2^23 placed
-// in the mantissa of 2^23 (1.5 2^23 for the signed leading digit) is converted
-// by one FP32 subtraction, and BF16 is the upper half of its FP32.
-__device__ __forceinline__ uint32_t ch_pair(long long a, long long b, int p)
-{
-    float fa, fb;
-    if (p == 0) {
-        fa = __uint_as_float(0x4B400000u + (uint32_t)(int)(a >> 49)) - 12582912.0f;
-        fb = __uint_as_float(0x4B400000u + (uint32_t)(int)(b >> 49)) - 12582912.0f;
-    } else {
-        const int s = 7 * (7 - p);
-        fa = __uint_as_float(0x4B000000u | ((uint32_t)(a >> s) & 127u)) - 8388672.0f;
-        fb = __uint_as_float(0x4B000000u | ((uint32_t)(b >> s) & 127u)) - 8388672.0f;
-    }
-    return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
 }
 
 // Shared-memory descriptor of a K-major operand of 128-byte rows with the
@@ -1073,8 +1044,7 @@ __global__ void __launch_bounds__(CH_THREADS, 1) k_oz_chain(ChainArgs a)
             uint8_t *dst = sA + row * 128 + (((2 * cg + c8) ^ (row & 7)) << 4);
 #pragma unroll
             for (int p = 0; p < OZ_S; ++p)
-                *reinterpret_cast<uint4 *>(dst + p * CH_TILE_A) =
-                    make_uint4(ch_pair(v[0], v[1], p), ch_pair(v[2], v[3], p), ch_pair(v[4], v[5], p), ch_pair(v[6], v[7], p));
+                *reinterpret_cast<uint4 *>(dst + p * CH_TILE_A) = oz_pair8(v, p);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         fence_before();
@@ -1640,16 +1610,11 @@ __global__ void __launch_bounds__(128) k_flip_pairs(PairArgs a)
     const long long ps = right ? a.rps : a.lps;
 #pragma unroll
     for (int k8 = 0; k8 < 32; k8 += 8) {
-        int dg[8][OZ_S];
+        long long v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) oz_digits(x[k8 + k], E, ef_max, dg[k]);
+        for (int k = 0; k < 8; ++k) v[k] = oz_fixed(x[k8 + k], E);
 #pragma unroll
-        for (int q = 0; q < OZ_S; ++q) {
-            __nv_bfloat162 h2[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) h2[k] = __floats2bfloat162_rn((float)dg[2 * k][q], (float)dg[2 * k + 1][q]);
-            *reinterpret_cast<uint4 *>(dst + q * ps + k8) = *reinterpret_cast<const uint4 *>(h2);
-        }
+        for (int q = 0; q < OZ_S; ++q) *reinterpret_cast<uint4 *>(dst + q * ps + k8) = oz_pair8(v, q);
     }
 }
 
