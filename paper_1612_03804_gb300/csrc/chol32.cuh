@@ -8,73 +8,90 @@
 
 namespace sldqmc {
 
-// 1/sqrt(d) of a pivot: the FP32 value y (relative error 2^-22) and one step of
-// third order, y + y e (1/2 + 3/8 e) with e = 1 - d y^2, whose remainder is below
-// 2^-66: five FP64 operations, four of them in sequence.  Conversions and
-// comparisons would take the FP64 pipe as well, so they are made on the bits:
-// one integer comparison tells a positive d of binary exponent -100 .. 99, and
-// for those d truncated to FP32 and y as a double are shifts.  Otherwise the
-// library's function; a pivot that is not positive and finite raises the
-// flag and counts as 1 (d is set to it).
-__device__ __forceinline__ double chol_rsqrt(double &d, bool real, int *flag)
+// Scratch of chol32.
+struct CholScratch {
+    double mult[2][32];  // row j over its pivot, for the step j's updates
+    double pivot[32];
+};
+
+// 1/d of a pivot by integers (an FP64 operation of a warp takes some 100 cycles
+// of the chain of pivots, an integer one 5).  With d = M 2^k, M of 53 bits, and
+// the FP32 reciprocal R0 2^-24 of M 2^-52 rounded to FP32, the remainder e = 1 - M
+// R0 2^-76 is below 3 2^-24, so its integer is the low 64 bits of -M R0, and 1/d =
+// R0 (1 + e + e^2) 2^.. (e^3 is below 2^-67), within 0.9 units in the last place.  A pivot that
+// is not positive and finite raises the flag and counts as 1 (d is set to
+// it); binary exponents beyond -500 .. 499 take the division.
+__device__ __forceinline__ double chol_reciprocal(double &d, bool real, int *flag)
 {
-    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
-    if (hi - (923u << 20) >= (200u << 20)) {
+    const long long u = __double_as_longlong(d);
+    const int ef = (int)(u >> 52);  // negative for negative d
+    if ((unsigned)(ef - 523) >= 1000u) {
         if (!(d > 0.0) || !isfinite(d)) {
             if (real) atomicOr(flag, FLAG_NUMERICAL);
             d = 1.0;
         }
-        return rsqrt(d);
+        return 1.0 / d;
     }
-    const float f = rsqrtf(__uint_as_float(((hi << 3) | (lo >> 29)) - (896u << 23)));
-    const double y = __longlong_as_double(((long long)__float_as_uint(f) << 29) + (896ll << 52));
-    const double e = fma(-(d * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
-// The row X[j][lane] = v with its pivot in lane j is final once scaled by y =
-// 1/sqrt(pivot); lane j then holds y, the diagonal of the inverse.
-__device__ __forceinline__ void chol32_finalise(double (*X)[33], double *root, int j, int lane, double v, int kb, int *flag)
-{
-    double d = __shfl_sync(0xffffffffu, v, j);
-    const double y = chol_rsqrt(d, lane == 0 && j < kb, flag);
-    X[j][lane] = lane == j ? y : v * y;
-    if (lane == 0) root[j] = d;
+    const unsigned long long M = ((unsigned long long)u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const float f = __uint_as_float(0x3F800000u + (uint32_t)((M - (1ull << 52) + (1ull << 28)) >> 29));  // in [1, 2]
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+    const uint32_t rb = __float_as_uint(r);
+    const uint32_t R0 = rb >= 0x3F800000u ? 1u << 24 : (rb & 0x7FFFFFu) | 0x800000u;  // r in [1/2, 1]
+    const long long e = -(long long)(M * (unsigned long long)R0);                     // units of 2^-76
+    const long long s = e >> 40;
+    const long long R = ((long long)R0 << 31) + (((e >> 15) * (long long)R0 + (1ll << 29)) >> 30) +
+                        ((s * s * (long long)R0 + (1ll << 40)) >> 41);  // units of 2^-55
+    return __longlong_as_double(((long long)(2044 - ef) << 52) + ((R + 2) >> 2));
 }
 
 // W = R^T R of the block W (X[r][c], c >= r; X[r][c] = 0 below the diagonal;
 // rows and columns kb..31 the identity, which stay as they are), by all warps
 // of the CTA.  On return X holds R above the diagonal and T = R^-T on and below
 // it, root[j] = R_jj (j < kb).
-// Right-looking, with R's and T's rows (T by forward substitution of R^T T =
-// 1) in one array: at step j row r > j loses X[j][r] times row j in the lanes
-// c >= r (R) and c <= j (T), one FMA per row.  Warp 0 updates row j + 1 and
-// finalises it while the others update the rows below, so a step costs one
-// barrier, and the chain of pivots is what bounds the kernel: a warp's FP64
-// instruction holds its sub-partition's pipe for 64 cycles however few lanes
-// work, and a step has seven in sequence or nearly.
-// All threads of the CTA call it between barriers; blockDim.x a multiple of 32.
-__device__ __forceinline__ void chol32(double (*X)[33], double *root, int kb, int *flag)
+// Right-looking without square roots (W = L D L^T), L^-1 formed with it (by
+// forward substitution) in the same array: at step j row r > j loses
+// X[j][r] / d_j times row j in the lanes c >= r (D L^T) and c <= j (L^-1, whose
+// diagonal is 1), one FMA per row; the rows are scaled by 1 / sqrt(d_j) at the
+// end, all pivots at once.  Warp 0 updates row j + 1, divides it by its pivot
+// and leaves it to the next step while the others update the rows below, so a
+// step costs one barrier and two FP64 operations in sequence (seven when the
+// rows were scaled by 1 / sqrt as they went; a panel's preparation 20.4 -> 18.7
+// us by events, 32 x 32, 4 items).
+// All threads of the CTA call it between barriers; blockDim.x a multiple of 32
+// (at least 64).
+__device__ __forceinline__ void chol32(double (*X)[33], double *root, CholScratch &sc, int kb, int *flag)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (wid == 0) chol32_finalise(X, root, 0, lane, X[0][lane], kb, flag);
-    __syncthreads();
-    for (int j = 0; j < kb - 1; ++j) {
+    double m = 0.0;  // warp 0: the current row over its pivot
+    for (int j = -1; j < kb - 1; ++j) {
         if (wid == 0) {
             const int r = j + 1;
             double v = X[r][lane];
-            const double xj = X[j][lane], xr = X[j][r];
-            if (lane >= r || lane <= j) v -= xr * xj;
-            chol32_finalise(X, root, r, lane, v, kb, flag);
-        } else {
+            if (j >= 0) {
+                const double mr = __shfl_sync(0xffffffffu, m, r), xj = X[j][lane];
+                if (lane >= r || lane <= j) v -= mr * xj;
+            }
+            double d = __shfl_sync(0xffffffffu, v, r);
+            const double inv = chol_reciprocal(d, lane == 0, flag);
+            m = v * inv;
+            X[r][lane] = lane == r ? 1.0 : v;
+            sc.mult[r & 1][lane] = m;
+            if (lane == 0) sc.pivot[r] = d;
+        } else if (j >= 0) {
             const double xj = X[j][lane];
             for (int r = j + 1 + wid; r < kb; r += nw - 1)
-                if (lane >= r || lane <= j) X[r][lane] -= X[j][r] * xj;
+                if (lane >= r || lane <= j) X[r][lane] -= sc.mult[j & 1][r] * xj;
         }
         __syncthreads();
     }
-    // R_jj = d y
-    if (threadIdx.x < kb) root[threadIdx.x] *= X[threadIdx.x][threadIdx.x];
+    if (wid == 0 && lane < kb) {
+        const double d = sc.pivot[lane], y = rsqrt(d);
+        sc.pivot[lane] = y;
+        root[lane] = d * y;
+    }
+    __syncthreads();
+    for (int r = wid; r < kb; r += nw) X[r][lane] *= sc.pivot[r];
     __syncthreads();
 }
 

@@ -387,7 +387,7 @@ __global__ void k_oz_make_T(const double *R, long long nn, int N, const double *
 // what the previous launch wrote, and the splitting hides behind the factor's
 // chain of pivots.  By events around the launches (32 x 32, 4 items): 34 us for
 // a factor with the library's rsqrt and separate arrays for R and T and 8 us
-// for the splitting; 20.5 us together.
+// for the splitting; 18.7 us together.
 struct OzPanelPrep {
     const double *W;
     long long sW;
@@ -404,6 +404,7 @@ __global__ void __launch_bounds__(256) k_oz_panel_prep(OzPanelPrep f, OzPanelSli
 {
     __shared__ double X[32][33];
     __shared__ double root[32];
+    __shared__ CholScratch sc;
     if (blockIdx.x > 0) {
         oz_slice_panel(a, blockIdx.x - 1, f.N, f.N, f.kb, f.k0, plane_stride, ldk, flag, X);
         return;
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(256) k_oz_panel_prep(OzPanelPrep f, OzPanelSli
         X[r][c] = r < kb && c < kb ? (c >= r ? Wb[(long long)r * f.N + c] : 0.0) : (r == c ? 1.0 : 0.0);
     }
     __syncthreads();
-    chol32(X, root, kb, flag);
+    chol32(X, root, sc, kb, flag);
     double *Rb = f.R + (long long)b * f.sR + (long long)f.k0 * f.N + f.k0;
     for (int e = tid; e < 32 * 32; e += 256) {
         const int r = e >> 5, c = e & 31;

@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_small_weight(SmallArgs a)
     __shared__ double D[SM_N], Dp[SM_N], root[SM_N], piv[SM_N], part[SM_N];
     __shared__ unsigned long long key[SM_N];
     __shared__ int perm[SM_N], s_p;
+    __shared__ CholScratch sc;
     const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int N = a.N;
     const int8_t *s = a.s + (long long)b * a.M * N;
@@ -139,7 +140,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_small_weight(SmallArgs a)
             const int r = e / N, c = e - r * N;
             W[r][c] = U[perm[r]][c];
         }
-        chol32(F, root, N, a.flag);
+        chol32(F, root, sc, N, a.flag);
         sm_solve(W, F, N);
         if (tid < N) F[tid][tid] = root[tid];
         __syncthreads();
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_small_weight(SmallArgs a)
                 U[r][c] = x;
             }
             __syncthreads();
-            chol32(U, root, N, a.flag);
+            chol32(U, root, sc, N, a.flag);
             sm_solve(W, U, N);
             if (tid < N) U[tid][tid] = root[tid];
             __syncthreads();

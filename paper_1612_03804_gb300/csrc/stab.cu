@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(128) k_chol_panel(const double *W, long long s
 {
     __shared__ double X[32][33], V[32][33];
     __shared__ double root[32];
+    __shared__ CholScratch sc;
     const int b = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double *Wb = W + (long long)b * sW;
     for (int e = threadIdx.x; e < 32 * 32; e += 128) {
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(128) k_chol_panel(const double *W, long long s
     const long long lds = isW ? ldw : N;
     for (int r = wid; r < 32; r += 4) V[r][lane] = live && r < kb ? src[(long long)(k0 + r) * lds + cc] : 0.0;
     __syncthreads();
-    chol32(X, root, kb, flag);
+    chol32(X, root, sc, kb, flag);
     double *Rb = R + (long long)b * sR;
     if (blockIdx.x == 0)
         for (int e = threadIdx.x; e < 32 * 32; e += 128) {
