@@ -121,6 +121,12 @@ bool small_fits(const sldqmc_ctx *c);
 void small_weight(sldqmc_ctx *c, const int8_t *d_s, int B, double cu, double cd, int tau0, double *d_ld, int *d_sign,
                   double *d_G, double scale, int accumulate);
 
+// One stabilisation of every item in one launch (small.cu: FP64 mode, N <= 64):
+// Xt -> Y = Q^T, D, V and the sign of the context updated.
+bool stab_block_fits(const sldqmc_ctx *c);
+void stab_block(sldqmc_ctx *c, const double *Xt, double *Y, int B, int passes);
+void stab_block_set_limits();
+
 // Slice products with the separable exp(-dtau K) (sep.cu): X^T_out =
 // U^T D_t0 E D_t0+1 E ... for nb slices, one row per CTA in shared memory.
 bool sep_supported(int Lx, int Ly);

@@ -792,6 +792,7 @@ void stab_set_limits(int Npad)
         cudaFuncSetAttribute(k_lu_panel_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, lu_sh);
         cudaFuncSetAttribute(k_lu_tslu_local, cudaFuncAttributeMaxDynamicSharedMemorySize, lu_sh);
         cudaFuncSetAttribute(k_lu_tslu_final, cudaFuncAttributeMaxDynamicSharedMemorySize, lu_sh);
+        stab_block_set_limits();
         if (dev >= 0) lu_set[dev] = true;
     }
 }
@@ -873,6 +874,10 @@ void stabilize(sldqmc_ctx *c, double *Xt, double *Wc, double *Y, int B, int pass
 {
     const int N = c->N;
     const long long nn = c->nn;
+    if (stab_block_fits(c)) {
+        stab_block(c, Xt, Y, B, passes);
+        return;
+    }
     double *W = c->buf[4];
     double *R1 = c->buf[6], *R2 = c->buf[7], *Vg = c->buf[8], *V = c->buf[1];
     // W = Xt Xt^T (upper triangle): FP64, or FP64-accurate on the tensor cores
