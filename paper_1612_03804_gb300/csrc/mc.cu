@@ -117,8 +117,8 @@ struct LocalArgs {
 
 // The decision of one site: logr = -2 s (dtau J nsp + Kt ntm) + 2 log|R_+| +
 // 2 log|R_-|, accepted iff log u < logr, R_f = 1 + Delta_f (1 - G_f[i][i]).  Taken
-// in FP32 where it is clear by a thousandth and ten times the FP32 rounding of
-// its terms; otherwise by the FP64 expression, whose two logarithms are some
+// in FP32 where it is clear by 1e-5 and more than the FP32 rounding of its terms
+// (below 4 2^-24 of each); otherwise by the FP64 expression, whose two logarithms are some
 // eighty instructions of the FP64 pipe at 64 cycles a warp each.
 struct FlipDecision {
     bool acc, margin;
@@ -137,7 +137,7 @@ __device__ __forceinline__ FlipDecision flip_decide(const LocalArgs &a, double g
     const float d = st + l0 + l1 - luf;
     o.acc = d > 0.0f;
     o.margin = false;
-    if (!(fabsf(d) > 1e-3f + 1e-5f * (fabsf(st) + fabsf(l0) + fabsf(l1) + fabsf(luf))) || !(r0 > 1e-30f && r0 < 1e30f) ||
+    if (!(fabsf(d) > 1e-5f + 1e-6f * (fabsf(st) + fabsf(l0) + fabsf(l1) + fabsf(luf))) || !(r0 > 1e-30f && r0 < 1e30f) ||
         !(r1 > 1e-30f && r1 < 1e30f)) {
         double logr = __dmul_rn(-2.0 * (double)sold,
                                 __dadd_rn(__dmul_rn(a.dtauJ, (double)nsp), __dmul_rn(a.Kt, (double)ntm)));
@@ -610,12 +610,13 @@ __device__ __forceinline__ int moved_site(int tau, int y, int x, int N, int Lx, 
 // n_c) * s with n_c the integer neighbour sums (self-pairs excluded),
 // accumulated in class order, accepted iff log u < a.  The G lanes of a group
 // (G a power of two, all lanes of the warp present) share the site's
-// neighbours and take the decision in FP32 where it is clear: the FP32 sum and
-// logarithms are off by less than 1e-5 of their terms, against a margin of 1e-4
-// and ten times that.  Otherwise the group's first lane takes the FP64 decision,
-// whose 2 n_class operations and logarithm on the FP64 pipe (64 cycles each per
-// warp) were most of a colour's time beside two divisions per coordinate and
-// neighbour.  Returns whether this lane flipped the site.
+// neighbours and take the decision in FP32 where it is clear: the sum of at most
+// 128 couplings is off by less than 132 2^-24 of the sum of their magnitudes,
+// the logarithm by less than 2^-23 of itself and 2^-23, and the margin is more
+// than each of these.  Otherwise the group's first lane takes the FP64 decision,
+// a hundred operations of the FP64 pipe at 64 cycles a warp: a margin ten times
+// wider, met in every second colour, made a sweep of 24 x 24 x 20 with 16 classes
+// 158 us instead of 143.  Returns whether this lane flipped the site.
 struct EffSite {
     const EffModel &em;
     int N, Lx, Ly, M;
@@ -623,6 +624,12 @@ struct EffSite {
     uint64_t key;
     uint32_t step;
 };
+
+// J times the spin s (+-1), by the sign bit.
+__device__ __forceinline__ float eff_signed(float J, int8_t s)
+{
+    return __uint_as_float(__float_as_uint(J) ^ ((uint32_t)(int)s & 0x80000000u));
+}
 
 __device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffNeighbour *nb, const float *Jn, int v,
                                          bool active, int G, int sw, long long &mg)
@@ -632,7 +639,7 @@ __device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffN
     float sum = 0.0f;
     if (active)
         for (int k = sub; k < e.em.n_nb; k += G)
-            sum += Jn[k] * (float)s[moved_site(tau, y, x, e.N, e.Lx, e.Ly, e.M, nb[k].dt, nb[k].dy, nb[k].dx)];
+            sum += eff_signed(Jn[k], s[moved_site(tau, y, x, e.N, e.Lx, e.Ly, e.M, nb[k].dt, nb[k].dy, nb[k].dx)]);
     for (int o = G >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (!active || sub) return false;
     const int sv = s[v];
@@ -642,7 +649,7 @@ __device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffN
     const float af = (float)e.twob * sum * (float)sv, lf = logf(__ull2float_rn(w) * (1.0f / 9007199254740992.0f));
     const float d = af - lf;
     bool acc = d > 0.0f;
-    if (!(fabsf(d) > 1e-4f + 1e-4f * (fabsf((float)e.twob) * e.em.Jabs) + 1e-5f * fabsf(lf)) || w == 0) {
+    if (!(fabsf(d) > 1e-6f + 1e-5f * (fabsf((float)e.twob) * e.em.Jabs) + 1e-6f * fabsf(lf)) || w == 0) {
         double sm = 0.0;
         int k = 0;
         for (int c = 0; c < e.em.n_class; ++c) {
@@ -867,8 +874,8 @@ void launch_drift(sldqmc_ctx *c, const double *Gw, const double *Gf, int B2x, in
 // of them): passes per colour in one CTA per chain, times the waves of chains,
 // against a launch and the passes spread over all SMs.  Measured per sweep:
 // 100 x 100 x 100, one chain, 4 classes 15.2 ms (one CTA, spins in global memory)
-// -> 97 us; 32 x 32 x 160, 16 classes, 4 chains 5.0 ms -> 0.40 ms (spread); 24 x 24 x
-// 20, 16 classes, 16 chains 490 -> 158 us (in shared memory).
+// -> 90 us; 32 x 32 x 160, 16 classes, 4 chains 5.0 ms -> 0.31 ms (spread); 24 x 24 x
+// 20, 16 classes, 16 chains 490 -> 143 us (in shared memory).
 void launch_eff_sweeps(sldqmc_ctx *c, int8_t *d_s, int B, int n_sweeps, uint64_t seed, uint32_t step,
                        int dir, long long *n_accept, long long *n_margin)
 {
