@@ -18,6 +18,7 @@
 // kappa(X) <= exp(n_wrap * dtau * (8t + 2 xi)), checked by the host.
 // Every matrix is stored row-major; the chain works on X^T so that columns
 // of X are contiguous rows.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -250,14 +251,22 @@ __device__ __forceinline__ unsigned long long lu_key(double v)
     return (unsigned long long)__double_as_longlong(fabs(v));
 }
 
+// The best key and row of the warp, in every lane, by three integer
+// reductions (the two halves of the key, then the row).
 __device__ __forceinline__ void lu_warp_argmax(unsigned long long &k, int &i)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long ok = __shfl_down_sync(0xffffffffu, k, o);
-        const int oi = __shfl_down_sync(0xffffffffu, i, o);
-        if (lu_key_better(ok, oi, k, i)) { k = ok; i = oi; }
-    }
+    const uint32_t hi = (uint32_t)(k >> 32), lo = (uint32_t)k;
+    const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    i = __reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? i : 0x7fffffff);
+    k = ((unsigned long long)mh << 32) | ml;
+}
+
+// 1 / v of a pivot (finite, not zero).
+__device__ __forceinline__ double lu_reciprocal(double v)
+{
+    double a = fabs(v);
+    return copysign(chol_reciprocal(a, false, nullptr), v);
 }
 
 // Logarithm, sign and the interchange record of a factored panel (pr[j]: the
@@ -341,7 +350,7 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_panel_smem(double *A, long lo
             unsigned long long k = lane < LU_THREADS / 32 ? wk[lane] : 0ull;
             int i = lane < LU_THREADS / 32 ? wi[lane] : R;
             lu_warp_argmax(k, i);
-            const int p = __shfl_sync(0xffffffffu, i, 0) < R ? __shfl_sync(0xffffffffu, i, 0) : j;
+            const int p = i < R ? i : j;
             if (p != j) {
                 const double t = P[j * 33 + lane];
                 P[j * 33 + lane] = P[p * 33 + lane];
@@ -362,7 +371,7 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_panel_smem(double *A, long lo
                 }
                 pvv[j] = v;
                 pr[j] = p;
-                s_vinv = 1.0 / v;
+                s_vinv = lu_reciprocal(v);
             }
         }
         __syncthreads();
@@ -390,7 +399,223 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_panel_smem(double *A, long lo
 }
 
 // ---------------------------------------------------------------------------
-// Panels taller than LU_SMEM_MAX_ROWS: tournament pivoting.  The panel's rows
+// Panels factored by a cluster of CTAs, partial pivoting over all rows: each
+// CTA keeps a balanced block of rows in shared memory.  Per column every CTA
+// sends its best candidate (key and row) and the first CTA the row to be
+// replaced into all CTAs' shared memory; after one cluster barrier every CTA
+// knows the pivot row, the owner takes the replaced one, and all update their
+// own rows.  The exchange is double-buffered, so the next column's writes
+// cannot meet a slower CTA's reads.
+// One CTA is bound by its FP64 pipe (R 32^2 / 2 FMAs at two per clock, 53 of 82
+// us for 400 rows) while a few items leave most SMs idle, and takes 800 rows at
+// most; a cluster divides that work by its size.  Measured by events:
+// up to 10^4 rows, one item 161 us a panel (tournament pivoting 418); up to 1024
+// rows, 4 items 75 us (one CTA up to 800 rows 118, tournament 339); 576 rows, 8
+// items 71 us (100).
+constexpr int LU_CLUSTER_MAX = 16;
+
+struct LuExchange {
+    double row[LU_CLUSTER_MAX][32], top[32];
+    unsigned long long key[LU_CLUSTER_MAX];
+    int idx[LU_CLUSTER_MAX];
+};
+
+__global__ void __launch_bounds__(LU_THREADS) k_lu_panel_cluster(double *A, long long sA, int lda, int N, int k0, int kb,
+                                                                 int *piv, double *logacc, int *lusgn, int *flag)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    extern __shared__ double P[];  // [nr][33]
+    __shared__ LuExchange ex[2];
+    __shared__ unsigned long long wk[LU_THREADS / 32];
+    __shared__ int wi[LU_THREADS / 32];
+    __shared__ double pvv[32], s_vinv;
+    __shared__ int pr[32], s_win;
+    const int C = gridDim.x, rank = blockIdx.x, b = blockIdx.y;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    double *Ab = A + (long long)b * sA + (long long)k0 * lda + k0;
+    const int R = N - k0;
+    const int r0 = (int)((long long)rank * R / C), nr = (int)((long long)(rank + 1) * R / C) - r0;
+    for (int e = tid; e < nr * 32; e += LU_THREADS) {
+        const int r = e >> 5, l = e & 31;
+        P[r * 33 + l] = l < kb ? Ab[(long long)(r0 + r) * lda + l] : 0.0;
+    }
+    // threads per row, each every T-th column
+    int T = 1;
+    while (T < 8 && 2 * T * nr <= LU_THREADS) T *= 2;
+    const int sub = tid & (T - 1), rstep = LU_THREADS / T;
+    __syncthreads();
+    unsigned long long bk = 0;
+    int bi = R;  // rows as numbered in the panel
+    for (int r = tid; r < nr; r += LU_THREADS) {
+        const unsigned long long k = lu_key(P[r * 33]);
+        if (lu_key_better(k, r0 + r, bk, bi)) { bk = k; bi = r0 + r; }
+    }
+    cl.sync();  // every CTA of the cluster has started: its shared memory may be written
+    for (int j = 0; j < kb; ++j) {
+        LuExchange &x = ex[j & 1];
+        lu_warp_argmax(bk, bi);
+        if (lane == 0) { wk[wid] = bk; wi[wid] = bi; }
+        __syncthreads();
+        if (wid == 0) {
+            unsigned long long k = lane < LU_THREADS / 32 ? wk[lane] : 0ull;
+            int i = lane < LU_THREADS / 32 ? wi[lane] : R;
+            lu_warp_argmax(k, i);
+            // no comparable entry in this block (all NaN or none left): its row j if it is here
+            if (i >= R && j >= r0 && j < r0 + nr) i = j;
+            const double v = i < R ? P[(i - r0) * 33 + lane] : 0.0;
+            const double top = rank == 0 ? P[j * 33 + lane] : 0.0;
+            for (int q = 0; q < C; ++q) {
+                LuExchange *y = cl.map_shared_rank(&x, q);
+                y->row[rank][lane] = v;
+                if (rank == 0) y->top[lane] = top;
+                if (lane == 0) {
+                    y->key[rank] = k;
+                    y->idx[rank] = i;
+                }
+            }
+        }
+        cl.sync();
+        if (wid == 0) {
+            unsigned long long k = lane < C ? x.key[lane] : 0ull;
+            int i = lane < C ? x.idx[lane] : R;
+            lu_warp_argmax(k, i);
+            const int p = i;
+            const unsigned m = __ballot_sync(0xffffffffu, lane < C && x.idx[lane < C ? lane : 0] == p);
+            const int w = __ffs(m) - 1;  // the pivot row's CTA
+            double v = x.row[w][j];
+            const bool bad = v == 0.0 || !isfinite(v);
+            if (bad) v = 1.0;
+            if (rank == w && p != j) P[(p - r0) * 33 + lane] = x.top[lane];
+            __syncwarp();
+            if (rank == 0) P[j * 33 + lane] = bad && lane == j ? 1.0 : x.row[w][lane];
+            if (lane == 0) {
+                if (rank == 0) {
+                    if (bad) atomicOr(flag, FLAG_NUMERICAL);
+                    pvv[j] = v;
+                    pr[j] = p;
+                }
+                s_vinv = lu_reciprocal(v);
+                s_win = w;
+            }
+        }
+        __syncthreads();
+        const double vinv = s_vinv;
+        const double *pw = x.row[s_win];
+        bk = 0;
+        bi = R;
+        for (int rb = 0; rb < nr; rb += rstep) {  // the same passes for all lanes
+            const int r = rb + tid / T;
+            const bool live = r < nr && r0 + r > j;
+            double *row = P + (live ? r : 0) * 33;
+            const double m = live ? row[j] * vinv : 0.0;
+            __syncwarp();  // the T lanes of a row have read its entry before one writes the multiplier
+            if (live) {
+                if (sub == 0) row[j] = m;
+                for (int l = j + 1 + ((sub - (j + 1)) & (T - 1)); l < kb; l += T) {
+                    const double v = row[l] - m * pw[l];
+                    row[l] = v;
+                    if (l == j + 1) {
+                        const unsigned long long k = lu_key(v);
+                        if (lu_key_better(k, r0 + r, bk, bi)) { bk = k; bi = r0 + r; }
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < nr * 32; e += LU_THREADS) {
+        const int r = e >> 5, l = e & 31;
+        if (l < kb) Ab[(long long)(r0 + r) * lda + l] = P[r * 33 + l];
+    }
+    if (rank == 0 && wid == 0) {
+        // the interchange record (see above): lane t follows row t < kb, lane e of
+        // the list the e-th row >= kb that was a pivot row
+        int top = lane, lrow = -1, lsrc = -1, n = 0, sg = 1;
+        double acc = lane < kb ? log(fabs(pvv[lane])) : 0.0;
+        for (int j = 0; j < kb; ++j) {
+            const int p = pr[j];
+            if (pvv[j] < 0.0) sg = -sg;
+            if (p == j) continue;
+            sg = -sg;
+            const int tj = __shfl_sync(0xffffffffu, top, j);
+            if (p < kb) {
+                const int tp = __shfl_sync(0xffffffffu, top, p);
+                if (lane == j) top = tp;
+                if (lane == p) top = tj;
+            } else {
+                unsigned m = __ballot_sync(0xffffffffu, lane < n && lrow == p);
+                if (!m) {
+                    if (lane == n) lrow = lsrc = p;
+                    m = 1u << n++;
+                }
+                const int e = __ffs(m) - 1, se = __shfl_sync(0xffffffffu, lsrc, e);
+                if (lane == j) top = se;
+                if (lane == e) lsrc = tj;
+            }
+        }
+        int *out = piv + (long long)b * N + k0;
+        if (lane < kb) out[lane] = top;
+        int pos = 0;
+        for (int e = 0; e < n; ++e) pos += __shfl_sync(0xffffffffu, lrow, e) < lrow;
+        if (lane < n) out[kb + pos] = lrow * 64 + lsrc;
+        if (lane == 0 && k0 + kb + n < N) out[kb + n] = -1;
+        // the logarithms are added in order, as the other panel kernels do
+        double s = logacc[b];
+        for (int j = 0; j < kb; ++j) s += __shfl_sync(0xffffffffu, acc, j);
+        if (lane == 0) {
+            logacc[b] = s;
+            lusgn[b] *= sg;
+        }
+    }
+    cl.sync();  // no CTA leaves while another may still write to its shared memory
+}
+
+static cudaLaunchConfig_t lu_cluster_config(const sldqmc_ctx *c, int R, int B, int C)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(C, B);
+    cfg.blockDim = dim3(LU_THREADS);
+    cfg.dynamicSmemBytes = sizeof(double) * 33 * (size_t)((R + C - 1) / C);
+    cfg.stream = c->st;
+    return cfg;
+}
+
+static cudaLaunchAttribute lu_cluster_attribute(int C)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    return at;
+}
+
+// CTAs per item of a panel of R rows: up to 8 while every CTA has 64 rows and
+// all items fit one wave, and as many as hold the rows (16 is beyond the
+// portable cluster size, so the device is asked); 0 when no cluster does.
+static int lu_cluster(const sldqmc_ctx *c, int R, int B)
+{
+    int C = 1;
+    while (C * LU_SMEM_MAX_ROWS < R) C *= 2;
+    if (C > LU_CLUSTER_MAX) return 0;
+    while (2 * C <= 8 && 2 * C * B <= c->num_sms && R / (2 * C) >= 64) C *= 2;
+    if (C > 8) {
+        cudaLaunchConfig_t cfg = lu_cluster_config(c, R, B, C);
+        cudaLaunchAttribute at = lu_cluster_attribute(C);
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_lu_panel_cluster, &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            return 0;
+        }
+    }
+    return C;
+}
+
+// ---------------------------------------------------------------------------
+// Panels taller than a cluster holds (12800 rows): tournament pivoting.  The panel's rows
 // are cut into up to TSLU_BLOCKS balanced row blocks; each block (one CTA)
 // runs partial pivoting on its own rows in shared memory and nominates the
 // kb rows it pivoted on; one CTA then runs partial pivoting on the
@@ -429,7 +654,7 @@ __device__ void lu_gepp_rows(double *P, int *org, int R, int kb, double *pvv, in
             unsigned long long k = lane < LU_THREADS / 32 ? wk[lane] : 0ull;
             int i = lane < LU_THREADS / 32 ? wi[lane] : R;
             lu_warp_argmax(k, i);
-            const int p = __shfl_sync(0xffffffffu, i, 0) < R ? __shfl_sync(0xffffffffu, i, 0) : j;
+            const int p = i < R ? i : j;
             if (p != j) {
                 const double t = P[j * 33 + lane];
                 P[j * 33 + lane] = P[p * 33 + lane];
@@ -450,7 +675,7 @@ __device__ void lu_gepp_rows(double *P, int *org, int R, int kb, double *pvv, in
                 }
                 pvv[j] = v;
                 pr[j] = p;
-                *s_vinv = 1.0 / v;
+                *s_vinv = lu_reciprocal(v);
             }
         }
         __syncthreads();
@@ -793,6 +1018,9 @@ void stab_set_limits(int Npad)
         cudaFuncSetAttribute(k_lu_tslu_local, cudaFuncAttributeMaxDynamicSharedMemorySize, lu_sh);
         cudaFuncSetAttribute(k_lu_tslu_final, cudaFuncAttributeMaxDynamicSharedMemorySize, lu_sh);
         stab_block_set_limits();
+        cudaFuncSetAttribute(k_lu_panel_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(sizeof(double) * 33 * LU_SMEM_MAX_ROWS));
+        cudaFuncSetAttribute(k_lu_panel_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (dev >= 0) lu_set[dev] = true;
     }
 }
@@ -963,8 +1191,17 @@ void finalize(sldqmc_ctx *c, const double *Ut, int B, double *d_ld, int *d_sign,
     const long long sItem = (long long)N * lda;
     for (int k0 = 0; k0 < N; k0 += 32) {
         int kb = N - k0 < 32 ? N - k0 : 32;
-        prof_begin(c, SLDQMC_KC_PANEL_F64, (double)B * (N - k0) * kb * kb, N - k0 <= LU_SMEM_MAX_ROWS ? "lu_panel_smem" : "lu_panel_tournament");
-        if (N - k0 <= LU_SMEM_MAX_ROWS) {
+        const int C = lu_cluster(c, N - k0, B);
+        prof_begin(c, SLDQMC_KC_PANEL_F64, (double)B * (N - k0) * kb * kb, C > 1 ? "lu_panel_cluster" : C == 1 ? "lu_panel_smem" : "lu_panel_tournament");
+        if (C > 1) {
+            cudaLaunchConfig_t cfg = lu_cluster_config(c, N - k0, B, C);
+            cudaLaunchAttribute at = lu_cluster_attribute(C);
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            cudaLaunchKernelEx(&cfg, k_lu_panel_cluster, A, sItem, lda, N, k0, kb, c->d_piv, c->d_logacc, c->d_sgn + c->cap,
+                               c->d_flag);
+            c->launches++;
+        } else if (C == 1) {
             k_lu_panel_smem<<<B, LU_THREADS, (sizeof(double) * 33 + sizeof(int)) * (N - k0), c->st>>>(
                 A, sItem, lda, N, k0, kb, c->d_piv, c->d_logacc, c->d_sgn + c->cap, c->d_flag);
             c->launches++;
