@@ -37,21 +37,24 @@ struct SmallArgs {
     int *flag;
 };
 
-// C = A B (sum over k0(r) <= k < k1(c)) for N x N matrices, C distinct from both.
+// C = A B (sum over k0(r) <= k < k1(c)) for N x N matrices, C distinct from both;
+// with a field slice sl, column c times cu where sl[c] > 0 and cd otherwise.
 template <class K0, class K1, class Load>
-__device__ __forceinline__ void sm_product(Mat C, int N, K0 k0, K1 k1, Load ab)
+__device__ __forceinline__ void sm_product(Mat C, int N, K0 k0, K1 k1, Load ab, const int8_t *sl = nullptr, double cu = 1.0,
+                                           double cd = 1.0)
 {
     for (int e = threadIdx.x; e < N * N; e += SM_THREADS) {
         const int r = e / N, c = e - r * N;
         double a0 = 0.0, a1 = 0.0;  // two chains
         int k = k0(r);
         const int kend = k1(c);
+        const double d = sl ? (sl[c] > 0 ? cu : cd) : 1.0;
         for (; k + 1 < kend; k += 2) {
             a0 = ab(a0, r, k, c);
             a1 = ab(a1, r, k + 1, c);
         }
         if (k < kend) a0 = ab(a0, r, k, c);
-        C[r][c] = a0 + a1;
+        C[r][c] = sl ? (a0 + a1) * d : a0 + a1;
     }
     __syncthreads();
 }
@@ -95,18 +98,22 @@ __global__ void __launch_bounds__(SM_THREADS) k_small_weight(SmallArgs a)
     for (int m = 0; m < a.M; m += a.n_wrap) {
         const int nb = a.n_wrap < a.M - m ? a.n_wrap : a.M - m;
         const int passes = m + nb >= a.M ? 2 : 1;
-        for (int j = 0; j < nb; ++j) {
+        {
             const int8_t *sl = s + (long long)slice * N;
             for (int e = tid; e < N * N; e += SM_THREADS) {
                 const int r = e / N, c = e - r * N;
                 U[r][c] *= sl[c] > 0 ? a.cu : a.cd;
             }
             __syncthreads();
-            sm_product(F, N, from0, toN, [=](double x, int r, int k, int c) { return fma(U[r][k], E[k][c], x); });
+        }
+        for (int j = 0; j < nb; ++j) {
+            if (++slice == a.M) slice = 0;
+            // the next slice's D with the result, while there is one in the block
+            sm_product(F, N, from0, toN, [=](double x, int r, int k, int c) { return fma(U[r][k], E[k][c], x); },
+                       j + 1 < nb ? s + (long long)slice * N : nullptr, a.cu, a.cd);
             Mat t = U;
             U = F;
             F = t;
-            if (++slice == a.M) slice = 0;
         }
         // Gram matrix of the rows of U = X^T
         sm_product(W, N, from0, toN, [=](double x, int r, int k, int c) { return fma(U[r][k], U[c][k], x); });
