@@ -862,26 +862,27 @@ __global__ void __launch_bounds__(128) k_lu_tslu_l21(double *A, long long sA, in
 
 // U12 = L11^{-1} A12 for the block row k0..k0+kb (L11 unit lower), with the
 // panel's row interchanges applied to these columns on the way (the record
-// in piv, see above): each thread owns one column, reads the kb source rows
-// and the sources of the changed rows below the block before it writes.
-template <int KB>
-__global__ void __launch_bounds__(128) k_lu_trsm_row(double *A, long long sA, int lda, int N, int ncols, int k0,
-                                                     int kb, const int *piv)
+// in piv, see above): the kb source rows and the sources of the changed rows
+// below the block are all read before the first write.  A CTA has 32 columns
+// (lanes), its four warps every fourth row each, as the panel solves of the
+// Cholesky-QR: a column's 496 FMAs on one thread hold one sub-partition's FP64
+// pipe for 17 us (33 us a launch by events at N = 576, 8 items, 18 us so).
+__global__ void __launch_bounds__(128) k_lu_trsm_row(double *A, long long sA, int lda, int N, int ncols, int k0, int kb,
+                                                     const int *piv)
 {
-    __shared__ double Lk[KB][KB + 1];
-    __shared__ int src[KB], edst[KB], esrc[KB];
+    __shared__ double Lk[32][33], W[32][33];
+    __shared__ int src[32], edst[32], esrc[32];
     __shared__ int s_E;
-    const int b = blockIdx.y;
+    const int b = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     double *Ab = A + (long long)b * sA;
     const int *rec = piv + (long long)b * N + k0;
-    for (int e = threadIdx.x; e < KB * KB; e += blockDim.x) {
-        int r = e / KB, c = e % KB;
+    for (int e = threadIdx.x; e < 32 * 32; e += 128) {
+        const int r = e >> 5, c = e & 31;
         Lk[r][c] = (r < kb && c < r) ? Ab[(long long)(k0 + r) * lda + k0 + c] : 0.0;
     }
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
+    if (wid == 0) {
         src[lane] = lane < kb ? rec[lane] : 0;
-        const int v = (lane < KB && k0 + kb + lane < N) ? rec[kb + lane] : -1;
+        const int v = k0 + kb + lane < N ? rec[kb + lane] : -1;
         const unsigned m = __ballot_sync(0xffffffffu, v >= 0);
         const int E = ~m ? __ffs(~m) - 1 : 32;
         if (lane < E) {
@@ -891,65 +892,70 @@ __global__ void __launch_bounds__(128) k_lu_trsm_row(double *A, long long sA, in
         if (lane == 0) s_E = E;
     }
     __syncthreads();
-    const int c = k0 + kb + blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncols) return;
+    const int c = k0 + kb + blockIdx.x * 32 + lane;
+    const bool live = c < ncols;
     const int E = s_E;
     double *col = Ab + (long long)k0 * lda + c;
-    double w[KB], x[KB];
+    double w[8], x[8];  // rows and changed rows 4 q + wid
 #pragma unroll
-    for (int r = 0; r < KB; ++r) w[r] = (r < kb) ? col[(long long)src[r] * lda] : 0.0;
-#pragma unroll
-    for (int e = 0; e < KB; ++e)
-        if (e < E) x[e] = col[(long long)esrc[e] * lda];
-#pragma unroll
-    for (int r = 0; r < KB; ++r) {
-        double acc = w[r];
-#pragma unroll
-        for (int l = 0; l < r; ++l) acc -= Lk[r][l] * w[l];
-        w[r] = acc;
+    for (int q = 0; q < 8; ++q) {
+        const int r = 4 * q + wid;
+        w[q] = live && r < kb ? col[(long long)src[r] * lda] : 0.0;
+        x[q] = live && r < E ? col[(long long)esrc[r] * lda] : 0.0;
     }
 #pragma unroll
-    for (int e = 0; e < KB; ++e)
-        if (e < E) col[(long long)edst[e] * lda] = x[e];
+    for (int l = 0; l < 32; ++l) {
+        if ((l & 3) == wid) W[l][lane] = w[l >> 2];
+        __syncthreads();  // the first one: all warps have read their rows
+        const double v = W[l][lane];
 #pragma unroll
-    for (int r = 0; r < KB; ++r)
-        if (r < kb) col[(long long)r * lda] = w[r];
+        for (int q = l >> 2; q < 8; ++q)
+            if (4 * q + wid > l) w[q] -= Lk[4 * q + wid][l] * v;
+    }
+    if (!live) return;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int r = 4 * q + wid;
+        if (r < E) col[(long long)edst[r] * lda] = x[q];
+        if (r < kb) col[(long long)r * lda] = w[q];
+    }
 }
 
 // X_k = U_kk^{-1} Y_k for the block row k0..k0+kb of the right-hand side
-// held in columns N..2N-1 (back substitution of the Green's function).
-template <int KB>
+// held in columns N..2N-1 (back substitution of the Green's function), laid
+// out as k_lu_trsm_row.
 __global__ void __launch_bounds__(128) k_trsm_upper_rhs(double *A, long long sA, int lda, int N, int k0, int kb)
 {
-    __shared__ double Uk[KB][KB + 1];
-    __shared__ double uinv[KB];
-    const int b = blockIdx.y;
+    __shared__ double Uk[32][33], W[32][33];
+    __shared__ double uinv[32];
+    const int b = blockIdx.y, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     double *Ab = A + (long long)b * sA;
-    for (int e = threadIdx.x; e < KB * KB; e += blockDim.x) {
-        int r = e / KB, c = e % KB;
-        double v = 0.0;
-        if (r < kb && c < kb && c >= r) v = Ab[(long long)(k0 + r) * lda + k0 + c];
-        else if (r == c) v = 1.0;
-        Uk[r][c] = v;
+    for (int e = threadIdx.x; e < 32 * 32; e += 128) {
+        const int r = e >> 5, c = e & 31;
+        Uk[r][c] = r < kb && c < kb ? (c >= r ? Ab[(long long)(k0 + r) * lda + k0 + c] : 0.0) : (r == c ? 1.0 : 0.0);
     }
     __syncthreads();
-    if (threadIdx.x < KB) uinv[threadIdx.x] = 1.0 / Uk[threadIdx.x][threadIdx.x];
+    if (wid == 0) uinv[lane] = 1.0 / Uk[lane][lane];
+    const int c = blockIdx.x * 32 + lane;
+    const bool live = c < N;
+    double *col = Ab + (long long)k0 * lda + N + c;
+    double w[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) w[q] = live && 4 * q + wid < kb ? col[(long long)(4 * q + wid) * lda] : 0.0;
     __syncthreads();
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= N) return;
-    double w[KB];
 #pragma unroll
-    for (int r = 0; r < KB; ++r) w[r] = (r < kb) ? Ab[(long long)(k0 + r) * lda + N + c] : 0.0;
+    for (int l = 31; l >= 0; --l) {
+        if ((l & 3) == wid) W[l][lane] = w[l >> 2] *= uinv[l];
+        __syncthreads();
+        const double v = W[l][lane];
 #pragma unroll
-    for (int r = KB - 1; r >= 0; --r) {
-        double acc = w[r];
-#pragma unroll
-        for (int l = r + 1; l < KB; ++l) acc -= Uk[r][l] * w[l];
-        w[r] = acc * uinv[r];
+        for (int q = 0; q <= (l >> 2); ++q)
+            if (4 * q + wid < l) w[q] -= Uk[4 * q + wid][l] * v;
     }
+    if (!live) return;
 #pragma unroll
-    for (int r = 0; r < KB; ++r)
-        if (r < kb) Ab[(long long)(k0 + r) * lda + N + c] = w[r];
+    for (int q = 0; q < 8; ++q)
+        if (4 * q + wid < kb) col[(long long)(4 * q + wid) * lda] = w[q];
 }
 
 // log|det(1 + U D V)| = sum log D_b + log|det M_mid|, sign = det(U) sign * LU sign.
@@ -1222,9 +1228,9 @@ void finalize(sldqmc_ctx *c, const double *Ut, int B, double *d_ld, int *d_sign,
         prof_end(c);
         int rest = ncols - (k0 + kb);
         if (rest > 0) {
-            dim3 gt(cdiv(rest, 128), B);
+            dim3 gt(cdiv(rest, 32), B);
             prof_begin(c, SLDQMC_KC_PANEL_F64, (double)B * rest * kb * kb, "lu_trsm_row");
-            k_lu_trsm_row<32><<<gt, 128, 0, c->st>>>(A, sItem, lda, N, ncols, k0, kb, c->d_piv);
+            k_lu_trsm_row<<<gt, 128, 0, c->st>>>(A, sItem, lda, N, ncols, k0, kb, c->d_piv);
             prof_end(c);
             c->launches++;
             int m2 = N - (k0 + kb);
@@ -1244,9 +1250,9 @@ void finalize(sldqmc_ctx *c, const double *Ut, int B, double *d_ld, int *d_sign,
         for (int kbi = nblk - 1; kbi >= 0; --kbi) {
             int k0 = kbi * 32;
             int kb = N - k0 < 32 ? N - k0 : 32;
-            dim3 gt(cdiv(N, 128), B);
+            dim3 gt(cdiv(N, 32), B);
             prof_begin(c, SLDQMC_KC_PANEL_F64, (double)B * N * kb * kb, "trsm_upper_rhs");
-            k_trsm_upper_rhs<32><<<gt, 128, 0, c->st>>>(A, sItem, lda, N, k0, kb);
+            k_trsm_upper_rhs<<<gt, 128, 0, c->st>>>(A, sItem, lda, N, k0, kb);
             prof_end(c);
             c->launches++;
             if (k0 > 0 && oz_full(c)) {
