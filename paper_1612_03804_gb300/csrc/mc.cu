@@ -606,6 +606,18 @@ __device__ __forceinline__ int moved_site(int tau, int y, int x, int N, int Lx, 
     return tau * N + y * Lx + x;
 }
 
+// The neighbours as the kernels read them.  A colour of a lattice in shared memory
+// is bound by the integer work of its neighbour loop, not by its loads: with the
+// offsets multiplied into units of sites beforehand (dx, dy Lx, dtau N), one 16-byte
+// load an entry and the wrap an unsigned minimum, a sweep of 24 x 24 x 20 with 16
+// classes takes 99 us instead of 143 (8-byte offsets, the coupling loaded apart,
+// comparisons and two products an entry).  A table of 16-bit neighbour numbers, read
+// from L2, took 187.
+struct __align__(16) EffEntry {
+    uint32_t dx, dy, dt;
+    float J;
+};
+
 // One Metropolis decision of H_eff: log acceptance a = ((2 beta) * sum_c J_c
 // n_c) * s with n_c the integer neighbour sums (self-pairs excluded),
 // accumulated in class order, accepted iff log u < a.  The G lanes of a group
@@ -616,7 +628,7 @@ __device__ __forceinline__ int moved_site(int tau, int y, int x, int N, int Lx, 
 // than each of these.  Otherwise the group's first lane takes the FP64 decision,
 // a hundred operations of the FP64 pipe at 64 cycles a warp: a margin ten times
 // wider, met in every second colour, made a sweep of 24 x 24 x 20 with 16 classes
-// 158 us instead of 143.  Returns whether this lane flipped the site.
+// 158 us instead of 143 (with the neighbours still as 8-byte offsets).  Returns whether this lane flipped the site.
 struct EffSite {
     const EffModel &em;
     int N, Lx, Ly, M;
@@ -631,15 +643,24 @@ __device__ __forceinline__ float eff_signed(float J, int8_t s)
     return __uint_as_float(__float_as_uint(J) ^ ((uint32_t)(int)s & 0x80000000u));
 }
 
-__device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffNeighbour *nb, const float *Jn, int v,
-                                         bool active, int G, int sw, long long &mg)
+// a - L if that is not negative, a otherwise, given a < 2 L and a - L modulo 2^32.
+__device__ __forceinline__ uint32_t eff_wrap(uint32_t a, uint32_t a_minus_L) { return min(a, a_minus_L); }
+
+__device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffEntry *nb, int v, bool active, int G, int sw,
+                                         long long &mg)
 {
     const int sub = threadIdx.x & (G - 1);
     const int tau = v / e.N, i = v - tau * e.N, y = i / e.Lx, x = i - y * e.Lx;
     float sum = 0.0f;
-    if (active)
-        for (int k = sub; k < e.em.n_nb; k += G)
-            sum += eff_signed(Jn[k], s[moved_site(tau, y, x, e.N, e.Lx, e.Ly, e.M, nb[k].dt, nb[k].dy, nb[k].dx)]);
+    if (active) {
+        const uint32_t x0 = x, yL = y * e.Lx, tN = (uint32_t)tau * e.N, xm = x0 - e.Lx, ym = yL - e.N,
+                       tm = tN - (uint32_t)e.N * e.M;
+#pragma unroll 5
+        for (int k = sub; k < e.em.n_nb; k += G) {
+            const EffEntry n = nb[k];
+            sum += eff_signed(n.J, s[eff_wrap(tN + n.dt, tm + n.dt) + eff_wrap(yL + n.dy, ym + n.dy) + eff_wrap(x0 + n.dx, xm + n.dx)]);
+        }
+    }
     for (int o = G >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (!active || sub) return false;
     const int sv = s[v];
@@ -655,7 +676,8 @@ __device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffN
         for (int c = 0; c < e.em.n_class; ++c) {
             int n = 0;
             for (int t = 0; t < 2 * e.em.noff[c]; ++t, ++k) {
-                const int u = moved_site(tau, y, x, e.N, e.Lx, e.Ly, e.M, nb[k].dt, nb[k].dy, nb[k].dx);
+                const EffNeighbour &o = e.em.nb[k];
+                const int u = moved_site(tau, y, x, e.N, e.Lx, e.Ly, e.M, o.dt, o.dy, o.dx);
                 if (u != v) n += s[u];
             }
             sm = __dadd_rn(sm, __dmul_rn(e.em.J[c], (double)n));
@@ -681,12 +703,10 @@ __device__ __forceinline__ void eff_counts(long long acc, long long mg, int b, l
     }
 }
 
-__device__ __forceinline__ void eff_load_nb(const EffModel &em, EffNeighbour *nb, float *Jn)
+__device__ __forceinline__ void eff_load_nb(const EffModel &em, EffEntry *nb, int Lx, int N)
 {
-    for (int k = threadIdx.x; k < em.n_nb; k += blockDim.x) {
-        nb[k] = em.nb[k];
-        Jn[k] = em.Jn[k];
-    }
+    for (int k = threadIdx.x; k < em.n_nb; k += blockDim.x)
+        nb[k] = EffEntry{(uint32_t)em.nb[k].dx, (uint32_t)em.nb[k].dy * Lx, (uint32_t)em.nb[k].dt * N, em.Jn[k]};
     __syncthreads();
 }
 
@@ -704,12 +724,11 @@ __global__ void __launch_bounds__(1024) k_eff_sweeps(int8_t *s_all, int Lx, int 
     const int N = Lx * Ly;
     const int V = N * M;
     extern __shared__ int8_t s[];
-    __shared__ EffNeighbour nb[128];
-    __shared__ float Jn[128];
+    __shared__ EffEntry nb[128];
     int8_t *gs = s_all + (long long)b * V;
     const uint64_t key = seed + ((uint64_t)b << 32);
     for (int v = threadIdx.x; v < V; v += blockDim.x) s[v] = gs[v];
-    eff_load_nb(em, nb, Jn);
+    eff_load_nb(em, nb, Lx, N);
     int dir = dir_fixed;
     if (dir < 0) dir = (int)(philox_word(key, 0, 0, step, PURPOSE_DIR) & 1u);
     long long acc = 0, mg = 0;
@@ -721,7 +740,7 @@ __global__ void __launch_bounds__(1024) k_eff_sweeps(int8_t *s_all, int Lx, int 
             const int q1 = col_start[col + 1];
             for (int q0 = col_start[col]; q0 < q1; q0 += per) {
                 const int q = q0 + threadIdx.x / G;
-                acc += eff_site(e, s, nb, Jn, q < q1 ? col_sites[q] : 0, q < q1, G, sw, mg);
+                acc += eff_site(e, s, nb, q < q1 ? col_sites[q] : 0, q < q1, G, sw, mg);
             }
             __syncthreads();
         }
@@ -740,9 +759,8 @@ __global__ void __launch_bounds__(256) k_eff_colour(int8_t *s_all, int Lx, int L
     if (d_step) step = *d_step;
     const int b = blockIdx.y;
     const int N = Lx * Ly;
-    __shared__ EffNeighbour nb[128];
-    __shared__ float Jn[128];
-    eff_load_nb(em, nb, Jn);
+    __shared__ EffEntry nb[128];
+    eff_load_nb(em, nb, Lx, N);
     const uint64_t key = seed + ((uint64_t)b << 32);
     int dir = dir_fixed;
     if (dir < 0) dir = (int)(philox_word(key, 0, 0, step, PURPOSE_DIR) & 1u);
@@ -752,7 +770,7 @@ __global__ void __launch_bounds__(256) k_eff_colour(int8_t *s_all, int Lx, int L
     const int q0 = col_start[col], n = col_start[col + 1] - q0;
     for (int k0 = blockIdx.x * blockDim.x; k0 < n; k0 += gridDim.x * blockDim.x) {
         const int k = k0 + threadIdx.x;
-        acc += eff_site(e, s_all + (long long)b * N * M, nb, Jn, k < n ? col_sites[q0 + k] : 0, k < n, 1, sw, mg);
+        acc += eff_site(e, s_all + (long long)b * N * M, nb, k < n ? col_sites[q0 + k] : 0, k < n, 1, sw, mg);
     }
     eff_counts(acc, mg, b, n_accept, n_margin);
 }
@@ -874,8 +892,8 @@ void launch_drift(sldqmc_ctx *c, const double *Gw, const double *Gf, int B2x, in
 // of them): passes per colour in one CTA per chain, times the waves of chains,
 // against a launch and the passes spread over all SMs.  Measured per sweep:
 // 100 x 100 x 100, one chain, 4 classes 15.2 ms (one CTA, spins in global memory)
-// -> 90 us; 32 x 32 x 160, 16 classes, 4 chains 5.0 ms -> 0.31 ms (spread); 24 x 24 x
-// 20, 16 classes, 16 chains 490 -> 143 us (in shared memory).
+// -> 90 us; 32 x 32 x 160, 16 classes, 4 chains 5.0 ms -> 0.28 ms (spread); 24 x 24 x
+// 20, 16 classes, 16 chains 490 -> 99 us (in shared memory).
 void launch_eff_sweeps(sldqmc_ctx *c, int8_t *d_s, int B, int n_sweeps, uint64_t seed, uint32_t step,
                        int dir, long long *n_accept, long long *n_margin)
 {
