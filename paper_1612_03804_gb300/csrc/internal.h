@@ -206,7 +206,7 @@ struct sldqmc_ctx {
     double h_J[32];
     double E0;
     int have_model;
-    int n_colors;
+    int n_colors, max_color;  // colours and the sites of the largest
     int *d_col_start, *d_col_sites;
     long long *d_feat0, *d_feat1;
     double *d_Jdev;

@@ -3,6 +3,7 @@
 // (Eq. 2, step iii), the bare Ising weight and the cumulative-update
 // acceptance (Eq. 4).  Every decision is taken in FP64 with explicitly
 // rounded operations so that it matches a plain IEEE evaluation.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
@@ -628,7 +629,8 @@ struct __align__(16) EffEntry {
 // than each of these.  Otherwise the group's first lane takes the FP64 decision,
 // a hundred operations of the FP64 pipe at 64 cycles a warp: a margin ten times
 // wider, met in every second colour, made a sweep of 24 x 24 x 20 with 16 classes
-// 158 us instead of 143 (with the neighbours still as 8-byte offsets).  Returns whether this lane flipped the site.
+// 158 us instead of 143 (one CTA, the neighbours as 8-byte offsets).  Returns whether
+// this lane flipped the site.
 struct EffSite {
     const EffModel &em;
     int N, Lx, Ly, M;
@@ -646,11 +648,34 @@ __device__ __forceinline__ float eff_signed(float J, int8_t s)
 // a - L if that is not negative, a otherwise, given a < 2 L and a - L modulo 2^32.
 __device__ __forceinline__ uint32_t eff_wrap(uint32_t a, uint32_t a_minus_L) { return min(a, a_minus_L); }
 
-__device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffEntry *nb, int v, bool active, int G, int sw,
+// What a decision needs that does not depend on the spins: the site's coordinates,
+// its random word and the word's logarithm.
+struct EffDraw {
+    int v, tau, y, x;
+    uint64_t w;
+    float lf;
+};
+
+__device__ __forceinline__ EffDraw eff_draw(const EffSite &e, int v, int sw)
+{
+    EffDraw d;
+    d.v = v;
+    d.tau = v / e.N;
+    const int i = v - d.tau * e.N;
+    d.y = i / e.Lx;
+    d.x = i - d.y * e.Lx;
+    uint32_t r[4] = {(uint32_t)i, (uint32_t)d.tau, e.step, PURPOSE_EFF | ((uint32_t)sw << 8)};
+    philox4x32_10(r, (uint32_t)e.key, (uint32_t)(e.key >> 32));
+    d.w = (((uint64_t)r[1] << 32) | (uint64_t)r[0]) >> 11;
+    d.lf = logf(__ull2float_rn(d.w) * (1.0f / 9007199254740992.0f));
+    return d;
+}
+
+__device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffEntry *nb, const EffDraw &d, bool active, int G,
                                          long long &mg)
 {
     const int sub = threadIdx.x & (G - 1);
-    const int tau = v / e.N, i = v - tau * e.N, y = i / e.Lx, x = i - y * e.Lx;
+    const int v = d.v, tau = d.tau, y = d.y, x = d.x;
     float sum = 0.0f;
     if (active) {
         const uint32_t x0 = x, yL = y * e.Lx, tN = (uint32_t)tau * e.N, xm = x0 - e.Lx, ym = yL - e.N,
@@ -664,13 +689,11 @@ __device__ __forceinline__ bool eff_site(const EffSite &e, int8_t *s, const EffE
     for (int o = G >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (!active || sub) return false;
     const int sv = s[v];
-    uint32_t r[4] = {(uint32_t)i, (uint32_t)tau, e.step, PURPOSE_EFF | ((uint32_t)sw << 8)};
-    philox4x32_10(r, (uint32_t)e.key, (uint32_t)(e.key >> 32));
-    const uint64_t w = (((uint64_t)r[1] << 32) | (uint64_t)r[0]) >> 11;
-    const float af = (float)e.twob * sum * (float)sv, lf = logf(__ull2float_rn(w) * (1.0f / 9007199254740992.0f));
-    const float d = af - lf;
-    bool acc = d > 0.0f;
-    if (!(fabsf(d) > 1e-6f + 1e-5f * (fabsf((float)e.twob) * e.em.Jabs) + 1e-6f * fabsf(lf)) || w == 0) {
+    const uint64_t w = d.w;
+    const float af = (float)e.twob * sum * (float)sv, lf = d.lf;
+    const float df = af - lf;
+    bool acc = df > 0.0f;
+    if (!(fabsf(df) > 1e-6f + 1e-5f * (fabsf((float)e.twob) * e.em.Jabs) + 1e-6f * fabsf(lf)) || w == 0) {
         double sm = 0.0;
         int k = 0;
         for (int c = 0; c < e.em.n_class; ++c) {
@@ -710,8 +733,24 @@ __device__ __forceinline__ void eff_load_nb(const EffModel &em, EffEntry *nb, in
     __syncthreads();
 }
 
-// n_sweeps colour-ordered sweeps of one chain per CTA, its spins in shared
-// memory, G lanes per site.
+// Copies n bytes, 16 at a time where both sides allow it.
+__device__ __forceinline__ void eff_copy(int8_t *dst, const int8_t *src, int n)
+{
+    int v = threadIdx.x;
+    if (!((((uintptr_t)dst) | (uintptr_t)src) & 15)) {
+        for (int q = threadIdx.x; q < n / 16; q += blockDim.x) ((int4 *)dst)[q] = ((const int4 *)src)[q];
+        v += n / 16 * 16;
+    }
+    for (; v < n; v += blockDim.x) dst[v] = src[v];
+}
+
+// n_sweeps colour-ordered sweeps of one chain per cluster of CTAs (or one CTA), its
+// spins in each CTA's shared memory, G lanes per site.  A CTA takes its share of a
+// colour's sites and writes a flipped spin into every CTA's copy; one cluster
+// barrier per colour, and the next sites are drawn before the wait for it.  A colour's
+// time in one CTA is its neighbour loop and its decisions, on one SM of 152: dividing
+// them took 24 x 24 x 20 with 16 classes and 16 chains from 4.1 to 2.1 us a colour.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(1024) k_eff_sweeps(int8_t *s_all, int Lx, int Ly, int M, double beta,
                                                      const __grid_constant__ EffModel em, const int *col_start,
                                                      const int *col_sites, int n_colors, int n_sweeps,
@@ -720,31 +759,74 @@ __global__ void __launch_bounds__(1024) k_eff_sweeps(int8_t *s_all, int Lx, int 
                                                      const uint32_t *d_step)
 {
     if (d_step) step = *d_step;  // graph replays read the step from device memory
-    const int b = blockIdx.x;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = CLUSTER ? cl.num_blocks() : 1, rank = CLUSTER ? cl.block_rank() : 0;
+    const int b = blockIdx.x / C;
     const int N = Lx * Ly;
     const int V = N * M;
-    extern __shared__ int8_t s[];
+    extern __shared__ __align__(16) int8_t s[];
     __shared__ EffEntry nb[128];
     int8_t *gs = s_all + (long long)b * V;
     const uint64_t key = seed + ((uint64_t)b << 32);
-    for (int v = threadIdx.x; v < V; v += blockDim.x) s[v] = gs[v];
+    eff_copy(s, gs, V);
     eff_load_nb(em, nb, Lx, N);
+    if (CLUSTER) cl.sync();  // every copy is loaded: spins may be written into it
     int dir = dir_fixed;
     if (dir < 0) dir = (int)(philox_word(key, 0, 0, step, PURPOSE_DIR) & 1u);
     long long acc = 0, mg = 0;
     const EffSite e{em, N, Lx, Ly, M, 2.0 * beta, key, step};
     const int per = blockDim.x / G;
-    for (int sw = 0; sw < n_sweeps; ++sw)
-        for (int cc = 0; cc < n_colors; ++cc) {
-            const int col = dir ? (n_colors - 1 - cc) : cc;
-            const int q1 = col_start[col + 1];
-            for (int q0 = col_start[col]; q0 < q1; q0 += per) {
-                const int q = q0 + threadIdx.x / G;
-                acc += eff_site(e, s, nb, q < q1 ? col_sites[q] : 0, q < q1, G, sw, mg);
+    int sw = 0, cc = 0, q = 0, q1 = 0;
+    auto colour = [&] {  // this CTA's share of the cc-th colour
+        const int col = dir ? (n_colors - 1 - cc) : cc;
+        const int c0 = col_start[col], c1 = col_start[col + 1], share = (c1 - c0 + C - 1) / C;
+        q = c0 + rank * share;
+        q1 = min(q + share, c1);
+    };
+    EffDraw d{};
+    auto draw = [&] {
+        const int k = q + threadIdx.x / G;
+        if (k < q1) d = eff_draw(e, col_sites[k], sw);
+    };
+    if (n_sweeps > 0) {
+        colour();
+        if (CLUSTER) draw();
+        for (;;) {
+            if (!CLUSTER) draw();
+            const bool flip = eff_site(e, s, nb, d, q + (int)threadIdx.x / G < q1, G, mg);
+            acc += flip;
+            if (CLUSTER && flip) {
+                const int8_t sv = s[d.v];
+                for (int r = 0; r < C; ++r)
+                    if (r != rank) *cl.map_shared_rank(s + d.v, r) = sv;
             }
-            __syncthreads();
+            q += per;
+            const bool last = q >= q1;
+            if (last) {
+                if (CLUSTER) cl.barrier_arrive();
+                if (++cc == n_colors) {
+                    cc = 0;
+                    ++sw;
+                }
+                if (sw < n_sweeps) colour();
+            }
+            if (CLUSTER && sw < n_sweeps) draw();
+            if (last) {
+                if (CLUSTER)
+                    cl.barrier_wait();
+                else
+                    __syncthreads();
+            }
+            if (sw == n_sweeps) break;
         }
-    for (int v = threadIdx.x; v < V; v += blockDim.x) gs[v] = s[v];
+    }
+    if (!CLUSTER) {
+        eff_copy(gs, s, V);
+    } else {
+        const int part = (V / C + 15) / 16 * 16, v0 = min(rank * part, V), v1 = rank == C - 1 ? V : min(v0 + part, V);
+        eff_copy(gs + v0, s + v0, v1 - v0);
+    }
     eff_counts(acc, mg, b, n_accept, n_margin);
 }
 
@@ -770,7 +852,7 @@ __global__ void __launch_bounds__(256) k_eff_colour(int8_t *s_all, int Lx, int L
     const int q0 = col_start[col], n = col_start[col + 1] - q0;
     for (int k0 = blockIdx.x * blockDim.x; k0 < n; k0 += gridDim.x * blockDim.x) {
         const int k = k0 + threadIdx.x;
-        acc += eff_site(e, s_all + (long long)b * N * M, nb, k < n ? col_sites[q0 + k] : 0, k < n, 1, sw, mg);
+        acc += eff_site(e, s_all + (long long)b * N * M, nb, eff_draw(e, k < n ? col_sites[q0 + k] : 0, sw), k < n, 1, mg);
     }
     eff_counts(acc, mg, b, n_accept, n_margin);
 }
@@ -886,29 +968,89 @@ void launch_drift(sldqmc_ctx *c, const double *Gw, const double *Gf, int B2x, in
     c->launches++;
 }
 
-// A chain's spins stay in one CTA's shared memory while its colours are small
-// or the chains fill the GPU; otherwise each colour is one launch over all SMs.
-// In units of the time of one pass of 1024 sites (about 1.5 us, a launch three
-// of them): passes per colour in one CTA per chain, times the waves of chains,
-// against a launch and the passes spread over all SMs.  Measured per sweep:
-// 100 x 100 x 100, one chain, 4 classes 15.2 ms (one CTA, spins in global memory)
-// -> 90 us; 32 x 32 x 160, 16 classes, 4 chains 5.0 ms -> 0.28 ms (spread); 24 x 24 x
-// 20, 16 classes, 16 chains 490 -> 99 us (in shared memory).
+static const int EFF_SMEM = 200 * 1024;  // the largest chain held in shared memory
+
+static cudaLaunchConfig_t eff_config(const sldqmc_ctx *c, int B, int C, int threads, long long V)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(B * C);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = (size_t)V;
+    cfg.stream = c->st;
+    return cfg;
+}
+
+static cudaLaunchAttribute eff_attribute(int C)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    return at;
+}
+
+// CTAs per chain: as many (up to the portable 8) as leave each EFF_READS neighbour
+// reads of a colour, while all chains run at once.  A colour ends with a cluster
+// barrier and with flips on their way to the other copies, which costs about as much
+// as that: 12 x 12 x 20 with 4 classes (4000 reads a colour) takes 14.8 us a sweep in
+// one CTA and 19.5 in two; with 16 classes (7200) 62 in one, 47 in two.
+static const int EFF_READS = 3072;
+static int eff_cluster(const sldqmc_ctx *c, int B, long long cs, int n_nb, long long V)
+{
+    if (V > EFF_SMEM) return 1;
+    for (int C = 8; C > 1; --C) {
+        if ((long long)B * C > c->num_sms || cs * n_nb < EFF_READS * C) continue;
+        cudaLaunchConfig_t cfg = eff_config(c, B, C, 1024, V);
+        cudaLaunchAttribute at = eff_attribute(C);
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, k_eff_sweeps<true>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (n >= B) return C;
+    }
+    return 1;
+}
+
+// A chain's spins stay in the shared memory of one CTA or of a cluster's CTAs while
+// its colours are small or the chains fill the GPU; otherwise each colour is one
+// launch over all SMs.  In units of the time of one pass of 1024 sites (about 1.5
+// us, a launch three of them): passes per colour in the chain's CTAs, times the waves
+// of chains, against a launch and the passes spread over all SMs; a cluster's barrier
+// counts as one more (48 x 48 x 80, 4 chains: 71 us a sweep spread, 79 in clusters).
+// Measured per sweep: 100 x 100 x 100, one chain, 4 classes 15.2 ms (one CTA, spins in
+// global memory) -> 89 us (spread); 64 x 64 x 100, 16 classes 12.2 ms -> 218 us (spread);
+// 32 x 32 x 160, 16 classes, 4 chains 5.0 ms -> 283 us (spread) -> 182 (clusters of 8);
+// 16 x 16 x 160, 4 classes, 16 chains 648 -> 99 us (one CTA) -> 36 (clusters); 24 x 24 x
+// 20, 16 classes, 16 chains 490 -> 99 us (one CTA) -> 50 (clusters).
 void launch_eff_sweeps(sldqmc_ctx *c, int8_t *d_s, int B, int n_sweeps, uint64_t seed, uint32_t step,
                        int dir, long long *n_accept, long long *n_margin)
 {
     const long long V = (long long)c->N * c->M;
     const EffModel em = eff_model_of(c);
     const long long cs = (V + c->n_colors - 1) / c->n_colors;  // sites per colour
-    const long long in_cta = ((cs + 1023) / 1024) * ((B + c->num_sms - 1) / c->num_sms);
+    const int C = eff_cluster(c, B, cs, em.n_nb, V);  // CTAs per chain
+    const long long share = (cs + C - 1) / C;
+    const long long in_cta = ((share + 1023) / 1024) * (((long long)B * C + c->num_sms - 1) / c->num_sms);
     const long long spread = 3 + (cs * B + 1024LL * c->num_sms - 1) / (1024LL * c->num_sms);
     prof_begin(c, SLDQMC_KC_EFF, 0.0, "eff_sweeps");
-    if (V <= 200 * 1024 && in_cta <= spread) {
-        int G = 1;  // lanes per site, while a colour leaves them idle
-        while (G < 8 && 2 * G * cs <= 1024) G *= 2;
-        k_eff_sweeps<<<B, 1024, (size_t)V, c->st>>>(d_s, c->p.Lx, c->p.Ly, c->M, c->p.beta, em, c->d_col_start,
-                                                    c->d_col_sites, c->n_colors, n_sweeps, seed, step, dir, G, n_accept,
-                                                    n_margin, c->step_dev);
+    if (V <= EFF_SMEM && (C == 1 ? in_cta <= spread : in_cta + 1 < spread)) {
+        // Lanes per site, while a colour leaves them idle; at most four in a cluster,
+        // where more would only add warps (24 x 24 x 20, 16 classes: 54, 50 and 58 us a
+        // sweep with up to 2, 4 and 8).
+        int G = 1;
+        const long long most = C > 1 ? (c->max_color + C - 1) / C : cs;  // a CTA's sites
+        while (G < (C > 1 ? 4 : 8) && 2 * G * most <= 1024) G *= 2;
+        const int threads = C > 1 && most * G < 1024 ? (int)((most * G + 31) / 32 * 32) : 1024;
+        cudaLaunchConfig_t cfg = eff_config(c, B, C, threads, V);
+        cudaLaunchAttribute at = eff_attribute(C);
+        cfg.attrs = &at;
+        cfg.numAttrs = C > 1;
+        cudaLaunchKernelEx(&cfg, C > 1 ? k_eff_sweeps<true> : k_eff_sweeps<false>, d_s, c->p.Lx, c->p.Ly, c->M, c->p.beta, em,
+                           (const int *)c->d_col_start, (const int *)c->d_col_sites, c->n_colors, n_sweeps, seed, step, dir,
+                           G, n_accept, n_margin, (const uint32_t *)c->step_dev);
         c->launches++;
     } else {
         const int bx = cdiv(cs, 256) < 1024 ? cdiv(cs, 256) : 1024;
@@ -961,7 +1103,8 @@ void launch_step_advance(sldqmc_ctx *c, uint32_t *d_step)
 
 void set_eff_smem_limits()
 {
-    cudaFuncSetAttribute(k_eff_sweeps, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_eff_sweeps<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, EFF_SMEM);
+    cudaFuncSetAttribute(k_eff_sweeps<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, EFF_SMEM);
     cudaFuncSetAttribute(k_local_flips<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_local_flips<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }

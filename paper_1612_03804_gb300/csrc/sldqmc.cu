@@ -1040,6 +1040,8 @@ int sldqmc_set_effective_model(sldqmc_ctx *c, int n_class, const int *n_off, con
     std::vector<int> start, sites;
     build_colouring(c, start, sites);
     c->n_colors = (int)start.size() - 1;
+    c->max_color = 0;
+    for (int k = 0; k < c->n_colors; ++k) c->max_color = std::max(c->max_color, start[k + 1] - start[k]);
     cudaFree(c->d_col_start);
     cudaFree(c->d_col_sites);
     c->d_col_start = nullptr;
