@@ -1155,7 +1155,9 @@ int sldqmc_fit_effective_action(sldqmc_ctx *c, const int8_t *cfgs, const double 
     const double e0 = -coef[0] / beta;
     if (E0) *E0 = e0;
     if (r2) *r2 = sst > 0.0 ? 1.0 - ssr / sst : 1.0;
-    return sldqmc_set_effective_model(c, nc, c->h_n_off, c->h_offsets, J, e0);
+    // the context's own class table is cleared before the new one is copied in
+    const std::vector<int> n_off(c->h_n_off, c->h_n_off + nc), off(c->h_offsets, c->h_offsets + 3 * c->n_off_total);
+    return sldqmc_set_effective_model(c, nc, n_off.data(), off.data(), J, e0);
 }
 
 int sldqmc_eff_sweeps(sldqmc_ctx *c, int8_t *s, int n_sweeps, uint64_t seed, uint32_t step, int dir,
