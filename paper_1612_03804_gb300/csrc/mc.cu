@@ -118,9 +118,11 @@ struct LocalArgs {
 
 // The decision of one site: logr = -2 s (dtau J nsp + Kt ntm) + 2 log|R_+| +
 // 2 log|R_-|, accepted iff log u < logr, R_f = 1 + Delta_f (1 - G_f[i][i]).  Taken
-// in FP32 where it is clear by 1e-5 and more than the FP32 rounding of its terms
-// (below 4 2^-24 of each); otherwise by the FP64 expression, whose two logarithms are some
-// eighty instructions of the FP64 pipe at 64 cycles a warp each.
+// in FP32 where it is clear by 1e-5 and by 1e-6 of the terms' magnitudes, those of
+// the two bare parts before they cancel; otherwise by the FP64 expression, whose two
+// logarithms are some eighty instructions of the FP64 pipe at 64 cycles a warp each.
+// FP32 is off by less: 3 2^-24 of each bare part (constant, product, sum), 2^-23 of each
+// logarithm and 4 2^-24 for its argument, 3 2^-24 of all terms for their sum.
 struct FlipDecision {
     bool acc, margin;
     double R[2];
@@ -134,12 +136,12 @@ __device__ __forceinline__ FlipDecision flip_decide(const LocalArgs &a, double g
     o.R[1] = __dadd_rn(1.0, __dmul_rn(dls[1][sold > 0], __dadd_rn(1.0, -gm)));
     const float r0 = fabsf((float)o.R[0]), r1 = fabsf((float)o.R[1]), luf = (float)lu;
     const float l0 = 2.0f * logf(r0), l1 = 2.0f * logf(r1);
-    const float st = -2.0f * (float)sold * ((float)a.dtauJ * (float)nsp + (float)a.Kt * (float)ntm);
-    const float d = st + l0 + l1 - luf;
+    const float sj = (float)a.dtauJ * (float)nsp, sk = (float)a.Kt * (float)ntm;
+    const float d = -2.0f * (float)sold * (sj + sk) + l0 + l1 - luf;
     o.acc = d > 0.0f;
     o.margin = false;
-    if (!(fabsf(d) > 1e-5f + 1e-6f * (fabsf(st) + fabsf(l0) + fabsf(l1) + fabsf(luf))) || !(r0 > 1e-30f && r0 < 1e30f) ||
-        !(r1 > 1e-30f && r1 < 1e30f)) {
+    if (!(fabsf(d) > 1e-5f + 1e-6f * (2.0f * (fabsf(sj) + fabsf(sk)) + fabsf(l0) + fabsf(l1) + fabsf(luf))) ||
+        !(r0 > 1e-30f && r0 < 1e30f) || !(r1 > 1e-30f && r1 < 1e30f)) {
         double logr = __dmul_rn(-2.0 * (double)sold,
                                 __dadd_rn(__dmul_rn(a.dtauJ, (double)nsp), __dmul_rn(a.Kt, (double)ntm)));
         logr = __dadd_rn(logr, __dmul_rn(2.0, log(fabs(o.R[0]))));
