@@ -1495,11 +1495,17 @@ void oz_rank_update(sldqmc_ctx *c, const double *L, const RankPart *pt, int npar
 }
 
 // Digit planes of exp(-dtau K) and exp(+dtau K), on first use; false when
-// there is no room for them (the callers then stay on the FP64 pipe).
+// there is no room for them, or while the stream is being captured and they are
+// not there yet (the callers then stay on the FP64 pipe).
 bool oz_e_planes(sldqmc_ctx *c)
 {
     OzWs *w = (OzWs *)c->oz_ws;
     if (w->e_tried) return w->emem != nullptr;
+    cudaStreamCaptureStatus cs;
+    if (cudaStreamIsCapturing(c->st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
     w->e_tried = 1;
     const int N = c->N;
     const int erows = N < OBN ? OBN : N;
