@@ -18,9 +18,29 @@ struct CholScratch {
 // of the chain of pivots, an integer one 5).  With d = M 2^k, M of 53 bits, and
 // the FP32 reciprocal R0 2^-24 of M 2^-52 rounded to FP32, the remainder e = 1 - M
 // R0 2^-76 is below 3 2^-24, so its integer is the low 64 bits of -M R0, and 1/d =
-// R0 (1 + e + e^2) 2^.. (e^3 is below 2^-67), within 0.9 units in the last place.  A pivot that
-// is not positive and finite raises the flag and counts as 1 (d is set to
-// it); binary exponents beyond -500 .. 499 take the division.
+// R0 (1 + e + e^2) 2^.. (e^3 is below 2^-67), within 0.9 units in the last place.
+// u: the bits of d (positive, biased exponent 523 .. 1522); rb: those of the FP32
+// reciprocal, which may be off by one unit in the last place, also to just below
+// 1/2 or above 1, where it counts as 1/2 or 1.
+__host__ __device__ __forceinline__ long long chol_reciprocal_bits(long long u, uint32_t rb)
+{
+    const unsigned long long M = ((unsigned long long)u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const uint32_t R0 = rb >= 0x3F800000u ? 1u << 24 : rb <= 0x3F000000u ? 1u << 23 : (rb & 0x7FFFFFu) | 0x800000u;
+    const long long e = -(long long)(M * (unsigned long long)R0);  // units of 2^-76
+    const long long s = e >> 40;
+    const long long R = ((long long)R0 << 31) + (((e >> 15) * (long long)R0 + (1ll << 29)) >> 30) +
+                        ((s * s * (long long)R0 + (1ll << 40)) >> 41);  // units of 2^-55
+    return ((2044 - (u >> 52)) << 52) + ((R + 2) >> 2);
+}
+
+// The bits of M 2^-52 rounded to FP32, in [1, 2].
+__host__ __device__ __forceinline__ uint32_t chol_seed_bits(long long u)
+{
+    return 0x3F800000u + (uint32_t)((((unsigned long long)u & 0xFFFFFFFFFFFFFull) + (1ull << 28)) >> 29);
+}
+
+// A pivot that is not positive and finite raises the flag and counts as 1 (d is
+// set to it); binary exponents beyond -500 .. 499 take the division.
 __device__ __forceinline__ double chol_reciprocal(double &d, bool real, int *flag)
 {
     const long long u = __double_as_longlong(d);
@@ -32,17 +52,9 @@ __device__ __forceinline__ double chol_reciprocal(double &d, bool real, int *fla
         }
         return 1.0 / d;
     }
-    const unsigned long long M = ((unsigned long long)u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const float f = __uint_as_float(0x3F800000u + (uint32_t)((M - (1ull << 52) + (1ull << 28)) >> 29));  // in [1, 2]
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
-    const uint32_t rb = __float_as_uint(r);
-    const uint32_t R0 = rb >= 0x3F800000u ? 1u << 24 : (rb & 0x7FFFFFu) | 0x800000u;  // r in [1/2, 1]
-    const long long e = -(long long)(M * (unsigned long long)R0);                     // units of 2^-76
-    const long long s = e >> 40;
-    const long long R = ((long long)R0 << 31) + (((e >> 15) * (long long)R0 + (1ll << 29)) >> 30) +
-                        ((s * s * (long long)R0 + (1ll << 40)) >> 41);  // units of 2^-55
-    return __longlong_as_double(((long long)(2044 - ef) << 52) + ((R + 2) >> 2));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(chol_seed_bits(u))));
+    return __longlong_as_double(chol_reciprocal_bits(u, __float_as_uint(r)));
 }
 
 // W = R^T R of the block W (X[r][c], c >= r; X[r][c] = 0 below the diagonal;
