@@ -41,19 +41,31 @@ def host(tmp_path_factory):
     return ctypes.CDLL(lib)
 
 
-def test_reciprocal_of_every_allowed_seed(host):
+def _pivots():
     rng = np.random.default_rng(8)
     m = np.concatenate([rng.integers(0, 2 ** 52, 1 << 18), np.arange(4096), 2 ** 52 - 1 - np.arange(4096),
                         rng.integers(0, 2 ** 31, 1 << 15), 2 ** 52 - 1 - rng.integers(0, 2 ** 31, 1 << 15)]).astype(np.int64)
     ef = np.where(np.arange(m.size) % 3 == 0, 1023, np.where(np.arange(m.size) % 3 == 1, 523, 1522)).astype(np.int64)
-    u = (ef << 52) | m
-    d = u.view(np.float64)
-    ref = (1.0 / d).view(np.int64)
-    for ulp in (-2, -1, 0, 1):  # two units below 1/2 are one of the binade above
-        shift = np.full(u.size, ulp, dtype=np.int32)
-        if ulp == -2:
-            shift[m < 2 ** 52 - 2 ** 29] = -1
-        out = np.zeros_like(u)
-        host.recip_bits(*(a.ctypes.data_as(ctypes.c_void_p) for a in (u, shift, out)), ctypes.c_int(u.size))
-        off = np.abs(out - ref)
-        assert off.max() <= 1, (ulp, int(off.max()), d[off.argmax()])
+    return (ef << 52) | m
+
+
+def _units_off(host, u, ulp):
+    """How far 1/d is from the division's, in units in the last place, with seeds ulp units off."""
+    shift = np.full(u.size, ulp, dtype=np.int32)
+    if ulp == -2:  # two units below 1/2 are one of the binade above
+        shift[(u & (2 ** 52 - 1)) < 2 ** 52 - 2 ** 29] = -1
+    out = np.zeros_like(u)
+    host.recip_bits(*(a.ctypes.data_as(ctypes.c_void_p) for a in (u, shift, out)), ctypes.c_int(u.size))
+    return np.abs(out - (1.0 / u.view(np.float64)).view(np.int64))
+
+
+def test_reciprocal_of_every_allowed_seed(host):
+    u = _pivots()
+    for ulp in (-2, -1, 0, 1):
+        assert _units_off(host, u, ulp).max() <= 1
+
+
+def test_reciprocal_is_the_division_whatever_the_seed(host):
+    u = _pivots()
+    for ulp in (-2, -1, 0, 1):
+        assert _units_off(host, u, ulp).max() == 0
