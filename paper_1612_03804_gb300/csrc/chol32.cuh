@@ -10,7 +10,7 @@ namespace sldqmc {
 
 // Scratch of chol32.
 struct CholScratch {
-    double mult[2][32];  // row j over its pivot, for the step j's updates
+    double mult[2][32];  // row j over its pivot, for the step j's updates; at the end 1 / sqrt of the pivots
     double pivot[32];
 };
 
@@ -70,7 +70,8 @@ __device__ __forceinline__ double chol_reciprocal(double &d, bool real, int *fla
 // forward substitution) in the same array: at step j row r > j loses
 // X[j][r] / d_j times row j in the lanes c >= r (D L^T) and c <= j (L^-1, whose
 // diagonal is 1), one FMA per row; the rows are scaled by 1 / sqrt(d_j) at the
-// end, all pivots at once.  Warp 0 updates row j + 1, divides it by its pivot
+// end, all pivots at once (R_jj is sqrt(d_j), not d_j / sqrt(d_j), which rounds twice;
+// warp 0 has the roots, warp 1 their reciprocals, each on a pipe of its own).  Warp 0 updates row j + 1, divides it by its pivot
 // and leaves it to the next step while the others update the rows below, so a
 // step costs one barrier and two FP64 operations in sequence (seven when the
 // rows were scaled by 1 / sqrt as they went; a panel's preparation 20.4 -> 18.7
@@ -102,13 +103,10 @@ __device__ __forceinline__ void chol32(double (*X)[33], double *root, CholScratc
         }
         __syncthreads();
     }
-    if (wid == 0 && lane < kb) {
-        const double d = sc.pivot[lane], y = rsqrt(d);
-        sc.pivot[lane] = y;
-        root[lane] = d * y;
-    }
+    if (wid == 0 && lane < kb) root[lane] = sqrt(sc.pivot[lane]);
+    if (wid == 1 && lane < kb) sc.mult[0][lane] = rsqrt(sc.pivot[lane]);
     __syncthreads();
-    for (int r = wid; r < kb; r += nw) X[r][lane] *= sc.pivot[r];
+    for (int r = wid; r < kb; r += nw) X[r][lane] *= sc.mult[0][r];
     __syncthreads();
 }
 

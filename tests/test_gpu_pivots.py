@@ -2,7 +2,9 @@
 division, bit for bit, over random mantissas, the mantissas where the FP32 seed or
 a rounding can go wrong (zeros, ones, within 2^30 of either end, the seed's
 rounding boundaries) and binary exponents at both ends of the integer range and
-beyond it."""
+beyond it; the Cholesky factor of 32 x 32 blocks against their exact roots
+(diagonal blocks: R_jj is the correctly rounded square root, its inverse within
+one unit in the last place) and against extended precision (dense blocks)."""
 import ctypes
 import subprocess
 
@@ -21,9 +23,24 @@ __global__ void k_recip(const double *d, double *out, int n, int *flag)
     double x = d[i];
     out[i] = chol_reciprocal(x, true, flag);
 }
+__global__ void k_chol(const double *W, double *R, double *root, int kb, int *flag)
+{
+    __shared__ double X[32][33], rt[32];
+    __shared__ CholScratch sc;
+    for (int e = threadIdx.x; e < 1024; e += blockDim.x) X[e >> 5][e & 31] = W[blockIdx.x * 1024 + e];
+    __syncthreads();
+    chol32(X, rt, sc, kb, flag);
+    for (int e = threadIdx.x; e < 1024; e += blockDim.x) R[blockIdx.x * 1024 + e] = X[e >> 5][e & 31];
+    if (threadIdx.x < kb) root[blockIdx.x * 32 + threadIdx.x] = rt[threadIdx.x];
+}
 extern "C" int run_recip(const double *d, double *out, int n, int *flag)
 {
     k_recip<<<(n + 255) / 256, 256>>>(d, out, n, flag);
+    return (int)cudaDeviceSynchronize();
+}
+extern "C" int run_chol(const double *W, double *R, double *root, int blocks, int threads, int kb, int *flag)
+{
+    k_chol<<<blocks, threads>>>(W, R, root, kb, flag);
     return (int)cudaDeviceSynchronize();
 }
 """
@@ -84,3 +101,48 @@ def test_bad_pivots_count_as_one_and_raise_the_flag(probe):
         flag = torch.zeros(1, dtype=torch.int32, device="cuda")
         assert probe.run_recip(_p(dd), _p(out), ctypes.c_int(1), _p(flag)) == 0
         assert flag.item() == 1 and out.item() == 1.0
+
+
+def _chol(probe, W, threads, kb):
+    import torch
+    n = W.shape[0]
+    dW = torch.from_numpy(np.ascontiguousarray(W)).cuda()
+    R = torch.zeros_like(dW)
+    root = torch.zeros((n, 32), dtype=torch.float64, device="cuda")
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert probe.run_chol(_p(dW), _p(R), _p(root), ctypes.c_int(n), ctypes.c_int(threads), ctypes.c_int(kb), _p(flag)) == 0
+    assert flag.item() == 0
+    return R.cpu().numpy(), root.cpu().numpy()
+
+
+@pytest.mark.parametrize("threads", [64, 128, 512])
+def test_roots_of_diagonal_blocks(probe, threads):
+    d = _pivots()
+    d = d[(d > 1e-140) & (d < 1e140)][: 32 * 4096].reshape(-1, 32)
+    W = np.zeros((d.shape[0], 32, 32))
+    W[:, np.arange(32), np.arange(32)] = d
+    X, root = _chol(probe, W, threads, 32)
+    np.testing.assert_array_equal(root, np.sqrt(d))
+    inv = X[:, np.arange(32), np.arange(32)]
+    exact = 1.0 / np.sqrt(d.astype(np.longdouble))
+    assert np.abs((inv - exact) / exact).max() <= 2.0 ** -52
+    off = X.copy()
+    off[:, np.arange(32), np.arange(32)] = 0.0
+    assert np.all(off == 0.0)
+
+
+@pytest.mark.parametrize("kb", [1, 7, 31, 32])
+def test_factor_and_inverse_of_dense_blocks(probe, kb):
+    rng = np.random.default_rng(kb)
+    A = rng.standard_normal((64, kb, kb + 8)) * np.exp(rng.uniform(-3, 3, (64, kb, 1)))
+    S = A @ A.transpose(0, 2, 1)
+    W = np.tile(np.eye(32), (64, 1, 1))
+    W[:, :kb, :kb] = np.triu(S)
+    X, root = _chol(probe, W, 128, kb)
+    eps = 2.0 ** -53
+    for b in range(64):
+        R = np.triu(X[b, :kb, :kb], 1) + np.diag(root[b, :kb])
+        T = np.tril(X[b, :kb, :kb])
+        den = np.sqrt(np.outer(np.diag(S[b]), np.diag(S[b])))
+        assert (np.abs((R.T @ R - S[b])) / den).max() <= 4 * (kb + 4) * eps  # backward error of a Cholesky factorisation
+        assert np.abs(T @ R.T - np.eye(kb)).max() <= 4 * (kb + 4) * eps * np.linalg.cond(R)
