@@ -157,10 +157,10 @@ __device__ __forceinline__ uint4 oz_pair8(const long long (&v)[8], int p)
 // Digits of the rows of one or two matrices (rows x cols, row stride ld, item
 // stride sX; blockIdx.z selects the matrix): row i becomes plane row i (prow
 // plane rows per item, leading dimension ldp) with K positions 0..cols-1 and
-// exponent E[b * prow + i]; the planes' columns beyond cols are left as they
-// are (zero pads of the buffer).  With a field slice sk the entries of column
-// k are first multiplied by cu where sk > 0 and by cd otherwise (the D of a
-// slice product X D E).  One warp per row, eight rows per CTA: the row's
+// exponent E[b * prow + i]; the planes' columns from cols to the next multiple
+// of 32 are zero, those beyond are left as they are (zero pads of the buffer).
+// With a field slice sk the entries of column k are first multiplied by cu
+// where sk > 0 and by cd otherwise (the D of a slice product X D E).  One warp per row, eight rows per CTA: the row's
 // maximum by warp shuffles, then each lane converts pairs of adjacent entries
 // and stores each plane's pair as one BF16x2.
 struct OzRows {
@@ -201,8 +201,8 @@ __global__ void __launch_bounds__(256) k_oz_slice(OzRows a, long long sX, int ro
     const int Ei = oz_exponent(ef_max);
     if (lane == 0) (blockIdx.z ? a.E[1] : a.E[0])[(long long)b * prow + i] = Ei;
     __nv_bfloat16 *row = (blockIdx.z ? a.planes[1] : a.planes[0]) + ((long long)b * prow + i) * ldp;
-    for (int k = 2 * lane; k < N; k += 64) {
-        const long long v0 = oz_fixed(at(k), Ei), v1 = oz_fixed(k + 1 < N ? at(k + 1) : 0.0, Ei);
+    for (int k = 2 * lane; k < (N + 31) / 32 * 32; k += 64) {
+        const long long v0 = oz_fixed(k < N ? at(k) : 0.0, Ei), v1 = oz_fixed(k + 1 < N ? at(k + 1) : 0.0, Ei);
 #pragma unroll
         for (int p = 0; p < OZ_S; ++p)
             *reinterpret_cast<uint32_t *>(row + (long long)p * plane_stride + k) = oz_pair(v0, v1, p);
@@ -1137,7 +1137,8 @@ struct OzWs {
     CUtensorMap mapT;
     CUtensorMap mapAS, mapRAS;  // planes and rplanes with the items' rows one after another (128-row boxes)
     // rank-32 updates: digit planes of the N x 32 left factors (two matrices
-    // per item), their row exponents
+    // per item), their row exponents; in the context's R2 and Vg buffers, which only
+    // a stabilisation uses (1032 N bytes per item of 16 N^2)
     __nv_bfloat16 *lplanes[2];
     long long lplane_stride;
     int *EL[2];
@@ -1186,8 +1187,8 @@ int oz_prepare(sldqmc_ctx *c)
     const size_t tebytes = sizeof(int) * (size_t)c->cap * 32;
     w->lplane_stride = (long long)c->cap * N * 32;
     const size_t lbytes = (size_t)OZ_S * w->lplane_stride * sizeof(__nv_bfloat16);
-    const size_t eoff = 2 * pbytes + tbytes + 2 * lbytes;  // the int arrays follow the planes
-    const size_t total = eoff + 7 * ebytes + tebytes + sizeof(int) * N;
+    const size_t eoff = 2 * pbytes + tbytes;  // the int arrays follow the planes
+    const size_t total = eoff + 5 * ebytes + tebytes + sizeof(int) * N;
     // The FP64 mode also runs without this workspace (on the FP64 pipe), so
     // there it is taken only when it leaves most of the free memory.
     const bool optional = c->p.prec == SLDQMC_FP64;
@@ -1208,20 +1209,21 @@ int oz_prepare(sldqmc_ctx *c)
     w->planes = (__nv_bfloat16 *)mem;
     w->rplanes = (__nv_bfloat16 *)((uint8_t *)mem + pbytes);
     w->tplanes = (__nv_bfloat16 *)((uint8_t *)mem + 2 * pbytes);
-    w->lplanes[0] = (__nv_bfloat16 *)((uint8_t *)mem + 2 * pbytes + tbytes);
-    w->lplanes[1] = (__nv_bfloat16 *)((uint8_t *)mem + 2 * pbytes + tbytes + lbytes);
+    uint8_t *left = (uint8_t *)c->buf[7];  // 64 cap N^2 bytes into the workspace: aligned for TMA
+    for (int f = 0; f < 2; ++f) {
+        w->lplanes[f] = small ? nullptr : (__nv_bfloat16 *)(left + f * lbytes);
+        w->EL[f] = small ? nullptr : (int *)(left + 2 * lbytes + f * ebytes);
+    }
     w->E = (int *)((uint8_t *)mem + eoff);
     w->ER = w->E + (size_t)c->cap * N;
     w->ER1 = w->ER + (size_t)c->cap * N;
     w->EPY = w->ER1 + (size_t)c->cap * N;
     w->EPW = w->EPY + (size_t)c->cap * N;
-    w->EL[0] = w->EPW + (size_t)c->cap * N;
-    w->EL[1] = w->EL[0] + (size_t)c->cap * N;
-    w->ET = w->EL[1] + (size_t)c->cap * N;
+    w->ET = w->EPW + (size_t)c->cap * N;
     w->EQ = w->ET + (size_t)c->cap * 32;
     w->emem = nullptr;
     w->e_tried = 0;
-    cudaMemsetAsync(mem, 0, eoff + 7 * ebytes + tebytes, c->st);  // zero pads: never written
+    cudaMemsetAsync(mem, 0, eoff + 5 * ebytes + tebytes, c->st);  // zero pads: never written
     {
         std::vector<int> ones((size_t)N, 1);
         if (cudaMemcpyAsync(w->EQ, ones.data(), sizeof(int) * N, cudaMemcpyHostToDevice, c->st) != cudaSuccess ||
