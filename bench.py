@@ -15,7 +15,8 @@ One step = one cumulative update (steps iii+iv): one sweep of N*M = 10^6
 effective-model flips, the exact log weight of the proposal (both flavours,
 i.e. two single-flavour fermion-weight evaluations through the stabilised
 B-chain) and the Eq. 4 acceptance.  value = fermion-weight evaluations/s.
-Beside it, in the same JSON line:
+Standard output is one JSON line with the headline and the compact part of what
+stands beside it; the whole record goes to standard error as one JSON line:
   fp64           -- the FP64-product path on the same lattice, extrapolated
                     from one timed block of n_wrap slices (labelled so);
   precision      -- log|det| relative/absolute error and max|dG| of the
@@ -1179,6 +1180,34 @@ def run_local_delayed(env):
             "rows": rows}
 
 
+LINE_BYTES = 2800  # of the result line: readers keep the last few KB of a run's output
+
+
+def result_line(head):
+    """The one line of standard output: the headline's contract keys with the
+    compact part of its breakdowns.  The whole record (other workloads, launch
+    sites, per-class breakdowns, notes) goes to standard error."""
+    def take(d, keys):
+        return {k: d[k] for k in keys if k in d} if isinstance(d, dict) else d
+
+    line = {k: v for k, v in head.items() if k not in ("workloads", "decorrelated_samples_per_s", "decorrelation_note")}
+    line["config"] = {k: v for k, v in head["config"].items() if k not in ("fit", "setup_s")}
+    for key, keys in (("roofline", ("kernel", "class", "bound", "achieved", "peak", "unit", "frac", "dtype", "issue_efficiency",
+                                    "mmas_per_product", "traffic", "launches", "ms_per_launch", "share")),
+                      ("precision", ("logdet_rel_err", "max_abs_dG")),
+                      ("separable", ("value", "unit", "ms_per_step", "closed_form_rel_err")),
+                      ("fp64", ("value", "unit", "extrapolated"))):
+        if key in line:
+            line[key] = take(line[key], keys)
+    text = json.dumps(line)
+    for key in ("separable", "fp64", "precision", "ms_per_accept_step"):  # never the contract's keys
+        if len(text) <= LINE_BYTES:
+            break
+        line.pop(key, None)
+        text = json.dumps(line)
+    return text
+
+
 def run_ours(args):
     env = Env(args)
     chosen = ALL_WORKLOADS if args.workloads == "all" else tuple(w for w in args.workloads.split(",") if w)
@@ -1213,7 +1242,8 @@ def run_ours(args):
                     "data": "synthetic", "config": {"workload": first.get("workload")},
                     "partial": "headline workload not run"}
         head["workloads"] = wls
-        print(json.dumps(head), flush=True)
+        print(json.dumps(head), file=sys.stderr, flush=True)
+        print(result_line(head), flush=True)
     if env.dist:
         env.dist.barrier()
         env.dist.destroy_process_group()
