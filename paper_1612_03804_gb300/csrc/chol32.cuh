@@ -18,10 +18,10 @@ struct CholScratch {
 // of the chain of pivots, an integer one 5).  With d = M 2^k, M of 53 bits, and
 // the FP32 reciprocal R0 2^-24 of M 2^-52 rounded to FP32, the remainder e = 1 - M
 // R0 2^-76 is below 3 2^-24, so its integer is the low 64 bits of -M R0, and 1/d =
-// R0 (1 + e + e^2) 2^.. (e^3 is below 2^-67), within 0.9 units in the last place.  The
-// remainder 2^105 - q M of that q (its integer again the low 64 bits) then says whether
-// q, q + 1 or q - 1 is nearest: 1/d correctly rounded, as the division gives it (no
-// reciprocal lies half way).
+// R0 (1 + e + e^2) 2^.. (e^3 is below 2^-67), within 1.3 quarters of a unit in the last
+// place.  So the nearest double is those quarters rounded down, q, or the next, and the
+// remainder 2^105 - q M (its integer again the low 64 bits) says which: 1/d correctly
+// rounded, as the division gives it (no reciprocal lies half way).
 // u: the bits of d (positive, biased exponent 523 .. 1522); rb: those of the FP32
 // reciprocal, which may be off by one unit in the last place, also to just below
 // 1/2 or above 1, where it counts as 1/2 or 1.
@@ -33,9 +33,9 @@ __host__ __device__ __forceinline__ long long chol_reciprocal_bits(long long u, 
     const long long s = e >> 40;
     const long long R = ((long long)R0 << 31) + (((e >> 15) * (long long)R0 + (1ll << 29)) >> 30) +
                         ((s * s * (long long)R0 + (1ll << 40)) >> 41);  // units of 2^-55
-    const long long q = (R + 2) >> 2;
-    const long long rem2 = -2 * (long long)(M * (unsigned long long)q);  // |remainder| < 1.5 M
-    return ((2044 - (u >> 52)) << 52) + q + (rem2 > (long long)M) - (rem2 < -(long long)M);
+    const long long q = R >> 2;
+    const long long rem = -(long long)(M * (unsigned long long)q);  // |rem| < 1.4 M
+    return ((2044 - (u >> 52)) << 52) + q + (2 * rem > (long long)M);
 }
 
 // The bits of M 2^-52 rounded to FP32, in [1, 2].
