@@ -69,6 +69,9 @@ GemmF64 gemm_desc(int M, int N, int K, const double *A, long long lda, long long
 // pipe then does these products).  Defined in oz_gram.cu.
 int oz_prepare(sldqmc_ctx *c);
 void oz_release(sldqmc_ctx *c);
+// Gives the twin t the context's ways of the FP64 mode's products: what c lacks t
+// gives back; false if t has no room for what c has.
+bool oz_match(const sldqmc_ctx *c, sldqmc_ctx *t);
 void oz_gram(sldqmc_ctx *c, const double *X, long long sX, double *W, long long sW, int ldw, int B);
 // Left-looking Cholesky-QR on the tensor cores (same N range):
 // oz_chol_begin fixes the digit exponents of R's columns from diag(W);

@@ -1666,6 +1666,23 @@ bool oz_worth(const sldqmc_ctx *c, int times)
     return c->N >= OBM || (double)c->N * c->N * c->N * c->plan_cap * times >= 8e6;
 }
 
+bool oz_match(const sldqmc_ctx *c, sldqmc_ctx *t)
+{
+    const OzWs *w = (const OzWs *)c->oz_ws;
+    OzWs *v = (OzWs *)t->oz_ws;
+    if (!w) {
+        oz_release(t);
+        return true;
+    }
+    if (!v) return false;
+    if (c->p.prec != SLDQMC_FP64) return true;  // propagator planes serve the wraps alone, on the context
+    if (!w->emem && v->emem) {
+        cudaFree(v->emem);
+        v->emem = nullptr;
+    }
+    return !w->emem == !v->emem;
+}
+
 bool oz_full(const sldqmc_ctx *c) { return c->oz_ws && c->N >= OBM; }
 
 bool oz_chain_fits(const sldqmc_ctx *c) { return c->N <= CH_N; }

@@ -259,7 +259,9 @@ int weight_run(sldqmc_ctx *c, const int8_t *d_s, int B, int eta, int tau0, doubl
 // kernels already fill the GPU, and the flavours run as two batches on the
 // two streams at once, where each fills the other's serial phases.  Created
 // on first use when its workspace takes under a third of the free device
-// memory; otherwise the flavours run in sequence on the context itself.
+// memory; otherwise the flavours run in sequence on the context itself.  Its
+// digit planes are there if the context's are, whatever memory was free when
+// each was made, so that both give the same bits.
 sldqmc_ctx *get_twin(sldqmc_ctx *c)
 {
     if (c->no_twin) return nullptr;
@@ -281,7 +283,7 @@ sldqmc_ctx *get_twin(sldqmc_ctx *c)
     sldqmc_ctx *t = nullptr;
     sldqmc_params p = c->p;
     p.max_batch = 2 * c->cap;
-    if (sldqmc_create(&p, (void *)st, &t) != SLDQMC_OK ||
+    if (sldqmc_create(&p, (void *)st, &t) != SLDQMC_OK || !oz_match(c, t) ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {
         if (t) sldqmc_destroy(t);
