@@ -27,8 +27,10 @@
  *   - Matrices are row-major double, N x N.
  *
  * Ownership and threading: a context owns all device memory it allocates
- * (at create time, and the exact log weight's second workspace on its first
- * use, see sldqmc_log_weight_batch_dev) and one CUDA stream (the caller's, or
+ * (at create time; local sweeps' buffers on their first use; and a second
+ * workspace of twice max_batch on the first log weight or local sweep, see
+ * sldqmc_log_weight_batch_dev), keeps it until it is destroyed, and owns one
+ * CUDA stream (the caller's, or
  * the legacy default stream when NULL).  Host-pointer calls copy in, run and copy out, and
  * return after the stream has finished (synchronous).  Device-pointer calls
  * (suffix _dev) take caller-owned device memory, are ordered on the
@@ -56,13 +58,20 @@ extern "C" {
 #define SLDQMC_ERR_UNSUPPORTED (-6)
 
 /* Arithmetic of the slice products inside a stabilisation block.  The
- * stabilisation (QR), the final determinant, the Green's function and every
- * Monte Carlo decision are FP64 in all modes. */
+ * stabilisation (QR), the final determinant and the Green's function are FP64
+ * or FP64-accurate in all modes.  Every Monte Carlo decision is the FP64 one: it
+ * is taken in FP32 only where it is clear by more than FP32's error bound. */
 typedef enum {
-    SLDQMC_FP64 = 0,   /* FP64-accurate products: FP64 FMA below 128 sites; from 128 sites on
-                          error-free digit splitting on the BF16 tensor cores (errors at the
-                          level of FP64 rounding), or FP64 FMA where its workspace would take
-                          more than a third of the free device memory */
+    SLDQMC_FP64 = 0,   /* FP64-accurate products, by error-free digit splitting on the BF16
+                          tensor cores (57 bits relative to each row's largest entry, errors
+                          at the level of FP64 rounding) or by FP64 FMA.  Digit splitting:
+                          everything from 128 sites on; the slice products from 33 to 64 sites
+                          (from 26 where N^3 max_batch > 7.5e6) and, where N^3 max_batch >=
+                          8e6, from 65 to 127; the wraps where 2 N^3 max_batch >= 8e6.  FP64
+                          FMA: the rest, and everything where the digit planes would take
+                          more than a third of the memory free at create time.  The route,
+                          and with it the last bits, goes by the lattice, max_batch and that
+                          memory, not by the batch of a call */
     SLDQMC_3XTF32 = 1, /* split-TF32 tensor-core products: the running product in two TF32
                           parts, exp(-dtau K) in three (five MMAs per K-step), FP32
                           accumulation spread over eight tensor-memory accumulators */
@@ -165,7 +174,8 @@ int sldqmc_local_sweep_batch_dev(sldqmc_ctx *ctx, int8_t *d_s, int B, uint64_t s
  * decisions agree outside the 1e-8 margin).  From 128 sites on the library
  * takes blocks of 32 sites whatever k (unless their workspace would take more
  * than a third of the free device memory), and up to 111 sites, where both
- * Green's functions fit shared memory, immediate updates. */
+ * Green's functions fit shared memory, immediate updates.  Above 5120 sites
+ * k >= 2 has to be set (SLDQMC_ERR_UNSUPPORTED otherwise). */
 int sldqmc_set_local_update_rank(sldqmc_ctx *ctx, int k);
 
 /* Effective model (Eq. 2): H_eff = E0 + sum_c J_c f_c(C),
@@ -330,7 +340,8 @@ int sldqmc_weight_noalloc(const sldqmc_params *p, void *stream, const int8_t *d_
  * rest is unspecified).  In the mixed-precision modes with N >= 128 computed as
  * the context's stabilisation does, on the BF16 tensor cores by error-free
  * digit splitting (FP64 accuracy: error below ~2^-52 of sqrt(W_ii W_jj));
- * otherwise by the FP64 GEMM.  1 <= B <= max_batch.
+ * otherwise by the FP64 GEMM (the FP64 mode's stabilisation itself uses digit
+ * splitting from 128 sites on).  1 <= B <= max_batch.
  * Stream-ordered on the context's stream; caller-owned device buffers. */
 int sldqmc_gram_batch_dev(sldqmc_ctx *ctx, const double *d_X, int B, double *d_W);
 
@@ -342,7 +353,7 @@ int sldqmc_gram_batch_dev(sldqmc_ctx *ctx, const double *d_X, int B, double *d_W
 int sldqmc_wait_selftest(sldqmc_ctx *ctx, int max_polls);
 
 /* Kernel classes for the timing hooks below. */
-#define SLDQMC_KC_GEMM_F64 0   /* FP64 GEMM (products below 128 sites, Gram entry point in FP64 mode) */
+#define SLDQMC_KC_GEMM_F64 0   /* FP64 GEMM (FP64-mode products outside the ranges of digit splitting, Gram entry point in FP64 mode) */
 #define SLDQMC_KC_GEMM_TC 1    /* tensor-core slice products (3xTF32 / BF16) */
 #define SLDQMC_KC_PANEL_F64 2  /* FP64 panel kernels (32x32 Cholesky blocks and inverses, LU panels, triangular solves, pivot sort) */
 #define SLDQMC_KC_EFF 3        /* effective-model sweeps */

@@ -71,11 +71,11 @@ __device__ __forceinline__ double chol_reciprocal(double &d, bool real, int *fla
 // X[j][r] / d_j times row j in the lanes c >= r (D L^T) and c <= j (L^-1, whose
 // diagonal is 1), one FMA per row; the rows are scaled by 1 / sqrt(d_j) at the
 // end, all pivots at once (R_jj is sqrt(d_j), not d_j / sqrt(d_j), which rounds twice;
-// warp 0 has the roots, warp 1 their reciprocals, each on a pipe of its own).  Warp 0 updates row j + 1, divides it by its pivot
-// and leaves it to the next step while the others update the rows below, so a
-// step costs one barrier and two FP64 operations in sequence (seven when the
-// rows were scaled by 1 / sqrt as they went; a panel's preparation 20.4 -> 18.7
-// us by events, 32 x 32, 4 items).
+// warp 0 has the roots, warp 1 their reciprocals, each on a pipe of its own).
+// Warp 0 updates row j + 1, divides it by its pivot and leaves it to the next
+// step while the others update the rows below, so a step costs one barrier and
+// two FP64 operations in sequence (seven when the rows were scaled by 1 / sqrt as
+// they went; a panel's preparation 20.4 -> 19.0 us by events, 32 x 32, 4 items).
 // All threads of the CTA call it between barriers; blockDim.x a multiple of 32
 // (at least 64).
 __device__ __forceinline__ void chol32(double (*X)[33], double *root, CholScratch &sc, int kb, int *flag)

@@ -10,9 +10,10 @@
 // is prefetched into registers while the current one is consumed.
 //
 // The tensor cores' digit-split products (oz_gram.cu) replace it from 128
-// sites on; below, and where their workspace does not fit, the same kernel
-// serves the slice products of the FP64 mode (with the
-// field scalings of B_tau = exp(-dtau K) diag(exp(eta dtau xi s)) fused in:
+// sites on, and in the slice products and wraps below where they are the faster
+// way; one CTA per item (small.cu) in the stabilisation up to 64 sites.  Otherwise,
+// and where the digit planes do not fit, it serves the FP64 mode's slice products
+// (with the field scalings of B_tau = exp(-dtau K) diag(exp(eta dtau xi s)) fused in:
 // the first slice of a block scales the K index, later slices scale the
 // output columns), the Gram matrices and trailing updates of the
 // stabilisation, and the LU updates of the final determinant.

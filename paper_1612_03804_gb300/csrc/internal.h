@@ -64,9 +64,9 @@ GemmF64 gemm_desc(int M, int N, int K, const double *A, long long lda, long long
 // N >= 128: W = X X^T to FP64 accuracy on the
 // BF16 tensor cores (Ozaki splitting; X row stride N, batch stride sX; W row
 // stride ldw, batch stride sW; tiles on or above the diagonal written).
-// oz_prepare leaves c->oz_ws null outside that range, and in the FP64 mode
-// when the planes would take more than a third of the free memory (the FP64
-// pipe then does these products).  Defined in oz_gram.cu.
+// oz_prepare leaves c->oz_ws null when the planes of the FP64 mode (made at any
+// N) would take more than a third of the free memory; the FP64 pipe then does
+// these products.  Defined in oz_gram.cu.
 int oz_prepare(sldqmc_ctx *c);
 void oz_release(sldqmc_ctx *c);
 // Gives the twin t the context's ways of the FP64 mode's products: what c lacks t

@@ -1,8 +1,9 @@
 // mc.cu -- Monte Carlo kernels: the DQMC local update ("Basics of DQMC"),
 // the effective-model sweeps and features of the self-learned action
 // (Eq. 2, step iii), the bare Ising weight and the cumulative-update
-// acceptance (Eq. 4).  Every decision is taken in FP64 with explicitly
-// rounded operations so that it matches a plain IEEE evaluation.
+// acceptance (Eq. 4).  Every decision is that of FP64 with explicitly rounded
+// operations, so that it matches a plain IEEE evaluation: flips are decided in
+// FP32 only where they are clear by more than FP32's error bound.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>

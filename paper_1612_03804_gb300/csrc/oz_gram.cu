@@ -1,10 +1,12 @@
 // oz_gram.cu -- FP64-accurate products on the BF16 tensor cores (Ozaki's
-// error-free splitting) for N >= 128: the stabilisation and the determinant in
+// error-free splitting).  For N >= 128: the stabilisation and the determinant in
 // every mode (Gram matrices, the left-looking Cholesky-QR updates and panel
 // products with the inverse of each 32 x 32 diagonal factor, formed here in
 // FP64, R = R2 R1, the V update, the trailing updates of the LU and the back
 // substitution of G), the slice products of the FP64 mode, and the wraps and
-// delayed corrections of the local sweep's Green's functions.
+// delayed corrections of the local sweep's Green's functions.  Below: the FP64
+// mode's slice products up to 64 sites (k_oz_chain), and those and the wraps to 127
+// sites where there is enough work (oz_worth); the FP64 pipe keeps the rest.
 //
 // Why not the FP64 pipe in the FP64 mode: it runs at 1.05-1.10 TFLOP/s however
 // a product is tiled (64 lanes-clocks per warp instruction), these products
@@ -12,7 +14,7 @@
 // two flavours: 185 us against 5600).  The largest error of a product against
 // extended precision is about a tenth of the FP64 GEMM's (Q D E, G E^-1,
 // E G E^-1 at N = 144 .. 576: 0.7e-16 .. 1.2e-16 against 1.0e-15 .. 1.7e-15 of the
-// largest element).  Below N = 128 (one tile row) the FP64 pipe keeps them.
+// largest element).
 //
 // The Gram matrix shows the scheme:
 //
@@ -387,7 +389,7 @@ __global__ void k_oz_make_T(const double *R, long long nn, int N, const double *
 // what the previous launch wrote, and the splitting hides behind the factor's
 // chain of pivots.  By events around the launches (32 x 32, 4 items): 34 us for
 // a factor with the library's rsqrt and separate arrays for R and T and 8 us
-// for the splitting; 18.7 us together.
+// for the splitting; 19.0 us together.
 struct OzPanelPrep {
     const double *W;
     long long sW;

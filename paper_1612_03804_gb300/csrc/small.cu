@@ -4,7 +4,7 @@
 // A weight of such a lattice is a chain of some forty dependent steps (slice
 // products, Gram matrix, pivot sort, Cholesky, V update per block, then the LU),
 // each of a few microseconds of launch latency and almost no work: 4 x 4, 20
-// slices 675 us as 42 launches, 107 us here.  All matrices live in shared memory (five
+// slices 675 us as 42 launches, 106 us here.  All matrices live in shared memory (five
 // of 32 x 33 doubles), a step costs a barrier instead of a launch, and the FP64
 // pipe is the bound: a warp's instruction holds it for 64 cycles, so elements
 // are dealt to threads without gaps (thread e, e + 256, ... of the N x N).
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_small_weight(SmallArgs a)
 // with the second pass) of the FP64 pipe become one; the pipe stays the bound
 // (0.44 M FMAs of one SM for 64 sites, 115 us of each SM whatever the number of
 // items up to one per SM), so a step's elements are dealt to threads densely.
-// Measured at 8 x 8, 64 items: 187 us; an 8 x 8 sweep of 64 chains (256
+// Measured at 8 x 8, 64 items: 192 us; an 8 x 8 sweep of 64 chains (256
 // stabilisations of 128 items) 141.6 -> 106.2 ms.
 constexpr int ST_N = 64, ST_LD = 65, ST_THREADS = 512;
 typedef double (*Mat64)[ST_LD];

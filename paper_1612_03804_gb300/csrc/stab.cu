@@ -410,8 +410,8 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_panel_smem(double *A, long lo
 // us for 400 rows) while a few items leave most SMs idle, and takes 800 rows at
 // most; a cluster divides that work by its size.  Measured by events:
 // up to 10^4 rows, one item 161 us a panel (tournament pivoting 418); up to 1024
-// rows, 4 items 75 us (one CTA up to 800 rows 118, tournament 339); 576 rows, 8
-// items 71 us (100).
+// rows, 4 items 76 us (one CTA up to 800 rows 118, tournament 339); 576 rows, 8
+// items 72 us (100).
 constexpr int LU_CLUSTER_MAX = 16;
 
 struct LuExchange {
