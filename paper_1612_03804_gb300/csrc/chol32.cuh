@@ -25,6 +25,8 @@ struct CholScratch {
 // u: the bits of d (positive, biased exponent 523 .. 1522); rb: those of the FP32
 // reciprocal, which may be off by one unit in the last place, also to just below
 // 1/2 or above 1, where it counts as 1/2 or 1.
+// EXACT = false: the quarters rounded to the nearest unit, within 0.9 units.
+template <bool EXACT = true>
 __host__ __device__ __forceinline__ long long chol_reciprocal_bits(long long u, uint32_t rb)
 {
     const unsigned long long M = ((unsigned long long)u & 0xFFFFFFFFFFFFFull) | (1ull << 52);
@@ -33,6 +35,7 @@ __host__ __device__ __forceinline__ long long chol_reciprocal_bits(long long u, 
     const long long s = e >> 40;
     const long long R = ((long long)R0 << 31) + (((e >> 15) * (long long)R0 + (1ll << 29)) >> 30) +
                         ((s * s * (long long)R0 + (1ll << 40)) >> 41);  // units of 2^-55
+    if (!EXACT) return ((2044 - (u >> 52)) << 52) + ((R + 2) >> 2);
     const long long q = R >> 2;
     const long long rem = -(long long)(M * (unsigned long long)q);  // |rem| < 1.4 M
     return ((2044 - (u >> 52)) << 52) + q + (2 * rem > (long long)M);
@@ -46,6 +49,7 @@ __host__ __device__ __forceinline__ uint32_t chol_seed_bits(long long u)
 
 // A pivot that is not positive and finite raises the flag and counts as 1 (d is
 // set to it); binary exponents beyond -500 .. 499 take the division.
+template <bool EXACT = true>
 __device__ __forceinline__ double chol_reciprocal(double &d, bool real, int *flag)
 {
     const long long u = __double_as_longlong(d);
@@ -59,7 +63,7 @@ __device__ __forceinline__ double chol_reciprocal(double &d, bool real, int *fla
     }
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(chol_seed_bits(u))));
-    return __longlong_as_double(chol_reciprocal_bits(u, __float_as_uint(r)));
+    return __longlong_as_double(chol_reciprocal_bits<EXACT>(u, __float_as_uint(r)));
 }
 
 // W = R^T R of the block W (X[r][c], c >= r; X[r][c] = 0 below the diagonal;
@@ -75,9 +79,15 @@ __device__ __forceinline__ double chol_reciprocal(double &d, bool real, int *fla
 // Warp 0 updates row j + 1, divides it by its pivot and leaves it to the next
 // step while the others update the rows below, so a step costs one barrier and
 // two FP64 operations in sequence (seven when the rows were scaled by 1 / sqrt as
-// they went; a panel's preparation 20.4 -> 19.0 us by events, 32 x 32, 4 items).
+// they went; a panel's preparation 20.4 -> 18.7 us by events, 32 x 32, 4 items).
+// EXACT: reciprocals and roots correctly rounded, as the FP64 mode has them.  The
+// mixed modes' factors never were (their panels took the library's rsqrt, now
+// reciprocals within 0.9 units and R_jj = d_j / sqrt(d_j)), and a bit changed there
+// moves a BF16 log|det| by 2e-8 through the products that follow (50 x 48, M = 181),
+// so they keep that form (18.7 us a panel's preparation, 19.0 with EXACT).
 // All threads of the CTA call it between barriers; blockDim.x a multiple of 32
 // (at least 64).
+template <bool EXACT = true>
 __device__ __forceinline__ void chol32(double (*X)[33], double *root, CholScratch &sc, int kb, int *flag)
 {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -91,7 +101,7 @@ __device__ __forceinline__ void chol32(double (*X)[33], double *root, CholScratc
                 if (lane >= r || lane <= j) v -= mr * xj;
             }
             double d = __shfl_sync(0xffffffffu, v, r);
-            const double inv = chol_reciprocal(d, lane == 0, flag);
+            const double inv = chol_reciprocal<EXACT>(d, lane == 0, flag);
             m = v * inv;
             X[r][lane] = lane == r ? 1.0 : v;
             sc.mult[r & 1][lane] = m;
@@ -103,8 +113,12 @@ __device__ __forceinline__ void chol32(double (*X)[33], double *root, CholScratc
         }
         __syncthreads();
     }
-    if (wid == 0 && lane < kb) root[lane] = sqrt(sc.pivot[lane]);
-    if (wid == 1 && lane < kb) sc.mult[0][lane] = rsqrt(sc.pivot[lane]);
+    if (EXACT && wid == 0 && lane < kb) root[lane] = sqrt(sc.pivot[lane]);
+    if (wid == 1 && lane < kb) {
+        const double d = sc.pivot[lane], y = rsqrt(d);
+        sc.mult[0][lane] = y;
+        if (!EXACT) root[lane] = d * y;
+    }
     __syncthreads();
     for (int r = wid; r < kb; r += nw) X[r][lane] *= sc.mult[0][r];
     __syncthreads();

@@ -389,7 +389,7 @@ __global__ void k_oz_make_T(const double *R, long long nn, int N, const double *
 // what the previous launch wrote, and the splitting hides behind the factor's
 // chain of pivots.  By events around the launches (32 x 32, 4 items): 34 us for
 // a factor with the library's rsqrt and separate arrays for R and T and 8 us
-// for the splitting; 19.0 us together.
+// for the splitting; 18.7 us together.
 struct OzPanelPrep {
     const double *W;
     long long sW;
@@ -401,6 +401,7 @@ struct OzPanelPrep {
     int *ET;
 };
 
+template <bool EXACT>
 __global__ void __launch_bounds__(256) k_oz_panel_prep(OzPanelPrep f, OzPanelSlice a, long long plane_stride, int ldk,
                                                        int *flag)
 {
@@ -418,7 +419,7 @@ __global__ void __launch_bounds__(256) k_oz_panel_prep(OzPanelPrep f, OzPanelSli
         X[r][c] = r < kb && c < kb ? (c >= r ? Wb[(long long)r * f.N + c] : 0.0) : (r == c ? 1.0 : 0.0);
     }
     __syncthreads();
-    chol32(X, root, sc, kb, flag);
+    chol32<EXACT>(X, root, sc, kb, flag);
     double *Rb = f.R + (long long)b * f.sR + (long long)f.k0 * f.N + f.k0;
     for (int e = tid; e < 32 * 32; e += 256) {
         const int r = e >> 5, c = e & 31;
@@ -1410,7 +1411,9 @@ void oz_chol_panel(sldqmc_ctx *c, int k0, int kb, const double *W, long long sW,
     sl.E[1] = w->EPW;
     const OzPanelPrep f{W, sW, R, c->nn, N, k0, kb, w->tplanes, w->tplane_stride, w->ET};
     prof_begin(c, SLDQMC_KC_PANEL_F64, (double)B * 2.0 * kb * kb * kb / 3.0, "oz_panel_prep");
-    k_oz_panel_prep<<<dim3(1 + sl.nb0 + (nW + 31) / 32, B), 256, 0, c->st>>>(f, sl, w->plane_stride, w->ldp, c->d_flag);
+    const dim3 grid(1 + sl.nb0 + (nW + 31) / 32, B);
+    if (c->p.prec == SLDQMC_FP64) k_oz_panel_prep<true><<<grid, 256, 0, c->st>>>(f, sl, w->plane_stride, w->ldp, c->d_flag);
+    else k_oz_panel_prep<false><<<grid, 256, 0, c->st>>>(f, sl, w->plane_stride, w->ldp, c->d_flag);
     prof_end(c);
     OzArgs a{};
     a.pt[0] = oz_part(N, 0, w->EPY, N, w->ET, 32, Y + (long long)k0 * N, c->nn, N);

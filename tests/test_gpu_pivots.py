@@ -4,7 +4,8 @@ a rounding can go wrong (zeros, ones, within 2^30 of either end, the seed's
 rounding boundaries) and binary exponents at both ends of the integer range and
 beyond it; the Cholesky factor of 32 x 32 blocks against their exact roots
 (diagonal blocks: R_jj is the correctly rounded square root, its inverse within
-one unit in the last place) and against extended precision (dense blocks)."""
+one unit in the last place) and against extended precision (dense blocks).  The
+mixed modes' form of both, within one unit and two."""
 import ctypes
 import subprocess
 
@@ -16,31 +17,35 @@ pytestmark = pytest.mark.gpu
 PROBE = r"""
 #include "chol32.cuh"
 using namespace sldqmc;
+template <bool EXACT>
 __global__ void k_recip(const double *d, double *out, int n, int *flag)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double x = d[i];
-    out[i] = chol_reciprocal(x, true, flag);
+    out[i] = chol_reciprocal<EXACT>(x, true, flag);
 }
+template <bool EXACT>
 __global__ void k_chol(const double *W, double *R, double *root, int kb, int *flag)
 {
     __shared__ double X[32][33], rt[32];
     __shared__ CholScratch sc;
     for (int e = threadIdx.x; e < 1024; e += blockDim.x) X[e >> 5][e & 31] = W[blockIdx.x * 1024 + e];
     __syncthreads();
-    chol32(X, rt, sc, kb, flag);
+    chol32<EXACT>(X, rt, sc, kb, flag);
     for (int e = threadIdx.x; e < 1024; e += blockDim.x) R[blockIdx.x * 1024 + e] = X[e >> 5][e & 31];
     if (threadIdx.x < kb) root[blockIdx.x * 32 + threadIdx.x] = rt[threadIdx.x];
 }
-extern "C" int run_recip(const double *d, double *out, int n, int *flag)
+extern "C" int run_recip(const double *d, double *out, int n, int *flag, int exact)
 {
-    k_recip<<<(n + 255) / 256, 256>>>(d, out, n, flag);
+    if (exact) k_recip<true><<<(n + 255) / 256, 256>>>(d, out, n, flag);
+    else k_recip<false><<<(n + 255) / 256, 256>>>(d, out, n, flag);
     return (int)cudaDeviceSynchronize();
 }
-extern "C" int run_chol(const double *W, double *R, double *root, int blocks, int threads, int kb, int *flag)
+extern "C" int run_chol(const double *W, double *R, double *root, int blocks, int threads, int kb, int *flag, int exact)
 {
-    k_chol<<<blocks, threads>>>(W, R, root, kb, flag);
+    if (exact) k_chol<true><<<blocks, threads>>>(W, R, root, kb, flag);
+    else k_chol<false><<<blocks, threads>>>(W, R, root, kb, flag);
     return (int)cudaDeviceSynchronize();
 }
 """
@@ -85,7 +90,7 @@ def test_pivot_reciprocals_are_ieee_divisions(probe):
     dd = torch.from_numpy(d).cuda()
     out = torch.zeros_like(dd)
     flag = torch.zeros(1, dtype=torch.int32, device="cuda")
-    assert probe.run_recip(_p(dd), _p(out), ctypes.c_int(d.size), _p(flag)) == 0
+    assert probe.run_recip(_p(dd), _p(out), ctypes.c_int(d.size), _p(flag), ctypes.c_int(1)) == 0
     got, ref = out.cpu().numpy(), 1.0 / d
     assert flag.item() == 0
     wrong = got.view(np.int64) != ref.view(np.int64)
@@ -99,18 +104,19 @@ def test_bad_pivots_count_as_one_and_raise_the_flag(probe):
         dd = torch.tensor([x], dtype=torch.float64, device="cuda")
         out = torch.zeros_like(dd)
         flag = torch.zeros(1, dtype=torch.int32, device="cuda")
-        assert probe.run_recip(_p(dd), _p(out), ctypes.c_int(1), _p(flag)) == 0
+        assert probe.run_recip(_p(dd), _p(out), ctypes.c_int(1), _p(flag), ctypes.c_int(1)) == 0
         assert flag.item() == 1 and out.item() == 1.0
 
 
-def _chol(probe, W, threads, kb):
+def _chol(probe, W, threads, kb, exact=1):
     import torch
     n = W.shape[0]
     dW = torch.from_numpy(np.ascontiguousarray(W)).cuda()
     R = torch.zeros_like(dW)
     root = torch.zeros((n, 32), dtype=torch.float64, device="cuda")
     flag = torch.zeros(1, dtype=torch.int32, device="cuda")
-    assert probe.run_chol(_p(dW), _p(R), _p(root), ctypes.c_int(n), ctypes.c_int(threads), ctypes.c_int(kb), _p(flag)) == 0
+    assert probe.run_chol(_p(dW), _p(R), _p(root), ctypes.c_int(n), ctypes.c_int(threads), ctypes.c_int(kb), _p(flag),
+                          ctypes.c_int(exact)) == 0
     assert flag.item() == 0
     return R.cpu().numpy(), root.cpu().numpy()
 
@@ -146,3 +152,21 @@ def test_factor_and_inverse_of_dense_blocks(probe, kb):
         den = np.sqrt(np.outer(np.diag(S[b]), np.diag(S[b])))
         assert (np.abs((R.T @ R - S[b])) / den).max() <= 4 * (kb + 4) * eps  # backward error of a Cholesky factorisation
         assert np.abs(T @ R.T - np.eye(kb)).max() <= 4 * (kb + 4) * eps * np.linalg.cond(R)
+
+
+def test_mixed_mode_reciprocals_and_roots(probe):
+    import torch
+    d = _pivots()
+    dd = torch.from_numpy(d).cuda()
+    out = torch.zeros_like(dd)
+    flag = torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert probe.run_recip(_p(dd), _p(out), ctypes.c_int(d.size), _p(flag), ctypes.c_int(0)) == 0
+    assert flag.item() == 0
+    assert np.abs(out.cpu().numpy().view(np.int64) - (1.0 / d).view(np.int64)).max() <= 1
+    d = d[(d > 1e-140) & (d < 1e140)][: 32 * 4096].reshape(-1, 32)
+    W = np.zeros((d.shape[0], 32, 32))
+    W[:, np.arange(32), np.arange(32)] = d
+    X, root = _chol(probe, W, 256, 32, exact=0)
+    assert np.abs(root.view(np.int64) - np.sqrt(d).view(np.int64)).max() <= 2
+    exact = 1.0 / np.sqrt(d.astype(np.longdouble))
+    assert np.abs((X[:, np.arange(32), np.arange(32)] - exact) / exact).max() <= 2.0 ** -52
