@@ -4,7 +4,7 @@
 // A weight of such a lattice is a chain of some forty dependent steps (slice
 // products, Gram matrix, pivot sort, Cholesky, V update per block, then the LU),
 // each of a few microseconds of launch latency and almost no work: 4 x 4, 20
-// slices 675 us as 42 launches, 106 us here.  All matrices live in shared memory (five
+// slices 675 us as 42 launches, 104 us here.  All matrices live in shared memory (five
 // of 32 x 33 doubles), a step costs a barrier instead of a launch, and the FP64
 // pipe is the bound: a warp's instruction holds it for 64 cycles, so elements
 // are dealt to threads without gaps (thread e, e + 256, ... of the N x N).
